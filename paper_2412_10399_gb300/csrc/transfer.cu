@@ -1709,44 +1709,88 @@ __device__ __forceinline__ void recover_B(const Pool& P, const SceneDev& s, cons
   for (int q = 0; q < 9; ++q) B[q] = (M[q] + dtv * tau[q]) * im;
 }
 
+// Floats of a particle field (x, v: 3; B, C, F: 9; E: 1).
+__host__ __device__ constexpr int field_width(int field) { return field <= 1 ? 3 : field == 5 ? 1 : 9; }
+
+// One particle field in the scene's original order.  Bound by HBM: it reads
+// the field (and the ids) once and writes it once.  Particles lie in binned
+// order, so the output rows are scattered by id, but neighbours in memory are
+// mostly neighbours in the original order too: a warp takes 32 particles,
+// turns their rows through shared memory (row pitch = width, odd: no bank
+// conflicts) and lets consecutive lanes write consecutive floats, so a store
+// instruction covers whole 32-byte sectors instead of 32 separate ones.
+// Only what the field needs is loaded (x and the material for B and C only).
+// Measured on 16.27 M particles (x, v, F): 127, 123 and 267 us (3.6, 3.7 and
+// 4.6 TB/s) against 1261 us for the three with one 4-byte store per lane and
+// float, rows apart, and every load made for every field.
 // pic: the PIC transfer keeps B = 0, so B and C read as 0.
-template <int KIND>
-__global__ void k_read_particles(Pool P, const SceneDev* scenes, const MatDev* mats, int scene, uint32_t start,
-                                 uint32_t n, int field, int pic, float* out) {
-  const SceneDev s = scenes[scene];
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    uint32_t t = start + i;
-    uint32_t id = P.ID[t];
-    float4 X = P.X[t];
-    const MatDev mt = mats[__float_as_uint(X.w)];
-    if (field == 0) {
-      out[3 * id] = X.x; out[3 * id + 1] = X.y; out[3 * id + 2] = X.z;
-    } else if (field == 1) {
-      float4 a = P.VM0[t];
-      out[3 * id] = a.x; out[3 * id + 1] = a.y; out[3 * id + 2] = a.z;
-    } else if (field == 4) {
-      float F[9];
-      load_F(P, t, F);
-      for (int q = 0; q < 9; ++q) out[9 * id + q] = F[q];
-    } else if (field == 5) {
-      out[id] = P.E ? P.E[t] : 0.f;
-    } else if (pic) {
-      for (int q = 0; q < 9; ++q) out[9 * id + q] = 0.f;
-    } else {
-      float B[9];
-      recover_B(P, s, mt, t, B);
-      if (field == 2) {
-        for (int q = 0; q < 9; ++q) out[9 * id + q] = B[q];
-      } else {  // C = B D^-1 = B Di / dx^2
-        Sten<KIND> st;
-        float ux = X.x * s.inv_dx, uy = X.y * s.inv_dx, uz = X.z * s.inv_dx;
-        Cell<KIND> cx, cy, cz;
-        cx.set(ux); cy.set(uy); cz.set(uz);
-        st.set(ux, uy, uz, cx.block() * 4, cy.block() * 4, cz.block() * 4);
-        float C[9];
-        mul_dinv(st, B, s.inv_dx * s.inv_dx, C);
-        for (int q = 0; q < 9; ++q) out[9 * id + q] = C[q];
+template <int KIND, int FIELD>
+__global__ void __launch_bounds__(256) k_read_particles(Pool P, const SceneDev* scenes, const MatDev* mats, int scene,
+                                                        uint32_t start, uint32_t n, int pic, float* out) {
+  constexpr int W = field_width(FIELD);
+  constexpr int U = FIELD == 2 || FIELD == 3 ? 1 : 2;  // groups of 32 particles whose loads are in flight together
+  __shared__ float rows[8][32 * W];
+  const uint32_t lane = threadIdx.x & 31u;
+  float* const row = rows[threadIdx.x >> 5];
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x * U;
+  // the loop runs on the warp's first particle: every lane takes every round
+  for (uint64_t i0 = ((uint64_t)blockIdx.x * blockDim.x + (threadIdx.x - lane)) * U; i0 < n; i0 += stride) {
+    const uint32_t cnt = (uint32_t)min((uint64_t)(32u * U), n - i0);
+    uint32_t id[U];
+    float r[U][W];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      id[u] = 0u;
+      if (u * 32u + lane >= cnt) continue;
+      const uint32_t t = start + (uint32_t)i0 + u * 32u + lane;
+      id[u] = P.ID[t];
+      if constexpr (FIELD == 0) {
+        const float4 X = P.X[t];
+        r[u][0] = X.x; r[u][1] = X.y; r[u][2] = X.z;
+      } else if constexpr (FIELD == 1) {
+        const float4 a = P.VM0[t];
+        r[u][0] = a.x; r[u][1] = a.y; r[u][2] = a.z;
+      } else if constexpr (FIELD == 4) {
+        load_F(P, t, r[u]);
+      } else if constexpr (FIELD == 5) {
+        r[u][0] = P.E ? P.E[t] : 0.f;
+      } else {
+        if (pic) {
+#pragma unroll
+          for (int q = 0; q < 9; ++q) r[u][q] = 0.f;
+        } else {
+          const SceneDev s = scenes[scene];
+          const float4 X = P.X[t];
+          const MatDev mt = mats[__float_as_uint(X.w)];
+          recover_B(P, s, mt, t, r[u]);
+          if constexpr (FIELD == 3) {  // C = B D^-1 = B Di / dx^2
+            Sten<KIND> st;
+            const float ux = X.x * s.inv_dx, uy = X.y * s.inv_dx, uz = X.z * s.inv_dx;
+            Cell<KIND> cx, cy, cz;
+            cx.set(ux); cy.set(uy); cz.set(uz);
+            st.set(ux, uy, uz, cx.block() * 4, cy.block() * 4, cz.block() * 4);
+            float C[9];
+            mul_dinv(st, r[u], s.inv_dx * s.inv_dx, C);
+#pragma unroll
+            for (int q = 0; q < 9; ++q) r[u][q] = C[q];
+          }
+        }
       }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (u * 32u + lane < cnt) {
+#pragma unroll
+        for (int q = 0; q < W; ++q) row[lane * W + q] = r[u][q];
+      }
+      __syncwarp();
+#pragma unroll
+      for (int k = 0; k < W; ++k) {
+        const uint32_t e = (uint32_t)k * 32u + lane, p = e / W;
+        const uint32_t idp = __shfl_sync(0xffffffffu, id[u], p);
+        if (u * 32u + p < cnt) out[(size_t)idp * W + (e - p * W)] = row[e];
+      }
+      __syncwarp();  // the next group overwrites the rows
     }
   }
 }
@@ -2021,15 +2065,29 @@ void launch_transfer(int kind, const LaunchCfg& lc, const StepView& v, int which
     launch_all<1>(lc, v, which);
 }
 
+template <int KIND>
+static void launch_read_field(int blocks, bool pic, cudaStream_t st, Pool P, const SceneDev* scenes,
+                              const MatDev* mats, int scene, uint32_t start, uint32_t n, int field, float* out) {
+  const int pc = pic ? 1 : 0;
+  switch (field) {
+    case 0: k_read_particles<KIND, 0><<<blocks, 256, 0, st>>>(P, scenes, mats, scene, start, n, pc, out); break;
+    case 1: k_read_particles<KIND, 1><<<blocks, 256, 0, st>>>(P, scenes, mats, scene, start, n, pc, out); break;
+    case 2: k_read_particles<KIND, 2><<<blocks, 256, 0, st>>>(P, scenes, mats, scene, start, n, pc, out); break;
+    case 3: k_read_particles<KIND, 3><<<blocks, 256, 0, st>>>(P, scenes, mats, scene, start, n, pc, out); break;
+    case 4: k_read_particles<KIND, 4><<<blocks, 256, 0, st>>>(P, scenes, mats, scene, start, n, pc, out); break;
+    case 5: k_read_particles<KIND, 5><<<blocks, 256, 0, st>>>(P, scenes, mats, scene, start, n, pc, out); break;
+  }
+}
+
 void launch_read_particles(int kind, bool pic, cudaStream_t st, Pool P, const SceneDev* scenes, const MatDev* mats,
                            int scene, uint32_t start, uint32_t n, int field, float* out) {
   int blocks = (int)((n + 255) / 256);
   if (blocks < 1) blocks = 1;
-  if (blocks > 4096) blocks = 4096;
+  if (blocks > 16384) blocks = 16384;
   if (kind == 0)
-    k_read_particles<0><<<blocks, 256, 0, st>>>(P, scenes, mats, scene, start, n, field, pic ? 1 : 0, out);
+    launch_read_field<0>(blocks, pic, st, P, scenes, mats, scene, start, n, field, out);
   else
-    k_read_particles<1><<<blocks, 256, 0, st>>>(P, scenes, mats, scene, start, n, field, pic ? 1 : 0, out);
+    launch_read_field<1>(blocks, pic, st, P, scenes, mats, scene, start, n, field, out);
 }
 
 void launch_write_particles(bool pic, cudaStream_t st, Pool P, const SceneDev* scenes, const MatDev* mats, int scene,
