@@ -3,7 +3,7 @@
 // One step of the compact-kernel MPM on the dual grid (Sec. 4.3-4.5) with the
 // fixed-corotated model, written as a pure function of the particle state
 // (x, v, B, F) and a per-particle Young's modulus E, with particles kept in
-// the caller's order and a dense grid of (res+1)^3 nodes per grid:
+// the caller's order and every node of both grids resident:
 //   P2G   m_i = sum w m,  P_i = sum w (m v + A d),  A = (m B - dt V0 tau(F)) D^-1
 //   grid  v~_i = mask (P_i / m_i + dt g)   (m_i > 0; sticky walls)
 //   G2P   v' = 1/2 sum w v~,  B' = 1/2 sum w v~ (x_i - x_p)^T,
@@ -16,6 +16,16 @@
 // stress adjoint goes through the polar decomposition F = R S with
 // dR = R Omega, Omega S + S Omega = R^T dF - dF^T R, whose (sigma_i + sigma_j)
 // denominators stay well conditioned when singular values coincide.
+//
+// Grid layout and its upkeep.  A node holds one float4 (m, P), (v~, 0) or
+// (p_bar, m_bar), so that a scatter is one 16-byte vector reduction per node
+// and a gather one 16-byte load, and nodes lie in 4x4x4 blocks (1 KiB).  P2G
+// lists the blocks its particles touch (a flag per block, taken once by an
+// exchange); the grid kernels run over that list alone and leave behind what
+// the next call expects: accumulators and flags at zero, and the last kernel
+// of a call returns the list's count to zero.  No call clears or sweeps the
+// whole domain (a body fills a few per cent of it), and the state lives in
+// device memory only, so a captured sequence can be replayed.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -32,23 +42,33 @@ using ck::svd3;
 
 struct DP {
   float dx, inv_dx, dt, V0, mass, nu, gx, gy, gz, bc;
-  int res, nn, n;
+  int res, nb, n;  // nb: 4x4x4-node blocks per axis, ceil((res + 1) / 4)
+};
+
+// The grids and their active blocks.
+struct DGrid {
+  float4* G;        // (m, P) per node: [grid][block][64]; zero between calls
+  float4* V;        // (v~, unused), valid in listed blocks
+  float4* A;        // adjoint: v~_bar, then (p_bar, m_bar), valid in listed blocks
+  uint32_t* flag;   // per block: 1 while listed
+  uint32_t* list;   // listed blocks
+  uint32_t* count;  // their number; zero between calls
+  uint32_t* err;
 };
 
 constexpr float kInv2Pi = 0.15915494309189535f;
-constexpr float kTwoPi = 6.283185307179586f;
 
 // Per-particle stencil on both grids with derivatives with respect to x.
 struct DS {
   int base[2][3];      // base node per grid (0: G-, 1: G+) and axis
   float W[2][3][2];    // 1-D weights
-  float dW[2][3][2];   // d W / d x (per unit length)
-  float d[2][3][2];    // x_i - x_p in cells
+  float dW[2][3];      // d W / d x of node 1 (per unit length); node 0 has the negative
+  float f[2][3];       // fraction: x_i - x_p = (node - f) cells
   float Di[9];         // D^-1 (cells^-2)
   float sg[3], dsg[3]; // sigma = sin(2 pi f+)/(2 pi) and d sigma / dx
   float dLam[3];       // d Lambda / dx
-  __device__ void set(const DP& p, float x0, float x1, float x2) {
-    float xs[3] = {x0, x1, x2};
+  __device__ __forceinline__ void set(const DP& p, float x0, float x1, float x2) {
+    const float xs[3] = {x0, x1, x2};
     float lam[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -74,14 +94,10 @@ struct DS {
       W[1][a][1] = fp - s;
       W[0][a][0] = 1.0f - fm - s;
       W[0][a][1] = fm + s;
-      dW[1][a][0] = (-1.0f + c2) * p.inv_dx;
-      dW[1][a][1] = (1.0f - c2) * p.inv_dx;
-      dW[0][a][0] = (-1.0f - c2) * p.inv_dx;
-      dW[0][a][1] = (1.0f + c2) * p.inv_dx;
-      d[1][a][0] = -fp;
-      d[1][a][1] = 1.0f - fp;
-      d[0][a][0] = -fm;
-      d[0][a][1] = 1.0f - fm;
+      dW[1][a] = (1.0f - c2) * p.inv_dx;
+      dW[0][a] = (1.0f + c2) * p.inv_dx;
+      f[1][a] = fp;
+      f[0][a] = fm;
       float m2p = fp * (1.0f - fp) - s * (1.0f - 2.0f * fp);
       float m2m = fm * (1.0f - fm) + s * (1.0f - 2.0f * fm);
       lam[a] = 0.5f * (m2p + m2m) - s * s;
@@ -100,7 +116,7 @@ struct DS {
       for (int j = 0; j < 3; ++j) Di[i * 3 + j] = (i == j ? li[i] : 0.0f) - y[i] * y[j] * den;
   }
   // x_bar contribution of an adjoint Dib on D^-1 (cells^-2)
-  __device__ void dinv_to_x(const float* Dib, float* xb) const {
+  __device__ __forceinline__ void dinv_to_x(const float* Dib, float* xb) const {
     // D_bar = -Di^T Dib Di^T  (Di symmetric)
     float T[9], Db[9];
 #pragma unroll
@@ -122,9 +138,27 @@ struct DS {
   }
 };
 
-__device__ __forceinline__ long long node_index(const DP& p, int g, int ix, int iy, int iz) {
-  return (((long long)g * p.nn + iz) * p.nn + iy) * p.nn + ix;
+// Offset of node i along an axis whose blocks are `bs` blocks apart and whose
+// local nodes `ls` nodes apart; a node's index is the sum over the axes.
+__device__ __forceinline__ uint32_t axis_off(int i, uint32_t bs, uint32_t ls) {
+  return (uint32_t)(i >> 2) * (bs * 64u) + (uint32_t)(i & 3) * ls;
 }
+
+// Node offsets of a particle's stencil on one grid, per axis and node.
+struct DOff {
+  uint32_t o[3][2];
+  __device__ __forceinline__ DOff(const DP& p, const DS& s, int g) {
+    const uint32_t nb = (uint32_t)p.nb;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      o[0][k] = axis_off(s.base[g][0] + k, 1u, 1u);
+      o[1][k] = axis_off(s.base[g][1] + k, nb, 4u);
+      o[2][k] = axis_off(s.base[g][2] + k, nb * nb, 16u);
+    }
+  }
+};
+
+__device__ __forceinline__ size_t grid_size(const DP& p) { return (size_t)p.nb * p.nb * p.nb * 64u; }
 
 __device__ __forceinline__ bool nodes_in_range(const DP& p, const DS& s) {
   bool ok = true;
@@ -135,9 +169,118 @@ __device__ __forceinline__ bool nodes_in_range(const DP& p, const DS& s) {
   return ok;
 }
 
-__device__ __forceinline__ void load9(const float* a, long long i, float* o) {
+// *a += v as one 16-byte reduction (a quarter of the L2 operations of four
+// scalar atomics).
+__device__ __forceinline__ void red_add4(float4* a, float x, float y, float z, float w) {
+  asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"l"(a), "f"(x), "f"(y), "f"(z), "f"(w) : "memory");
+}
+
+__device__ __forceinline__ void list_block(const DGrid& D, uint32_t b) {
+  // the plain read skips the exchange once the flag is seen; a stale 0 only
+  // costs an exchange
+  if (D.flag[b] == 0u && atomicExch(&D.flag[b], 1u) == 0u) D.list[atomicAdd(D.count, 1u)] = b;
+}
+
+// List the blocks of the nodes a warp's particles touch on either grid (nodes
+// base[0] .. base[1] + 1 per axis; all lanes call, `on` marks those with a
+// particle).  Neighbours in the caller's order are mostly neighbours in
+// space, so the warp takes the bounding box of its blocks, one lane a block,
+// when that is at most 32 blocks (a listed block without mass only costs its
+// visit); each lane lists its own otherwise.  One exchange per warp and block
+// instead of one per particle: the flags of a small body are contended.
+__device__ __forceinline__ void list_blocks(const DP& p, const DGrid& D, const DS& s, bool on) {
+  int lo[3], hi[3], wl[3], wn[3];
 #pragma unroll
-  for (int q = 0; q < 9; ++q) o[q] = a[9 * i + q];
+  for (int a = 0; a < 3; ++a) {
+    lo[a] = s.base[0][a] >> 2;
+    hi[a] = (s.base[1][a] + 1) >> 2;
+    wl[a] = __reduce_min_sync(0xffffffffu, on ? lo[a] : 0x7fffffff);
+    wn[a] = __reduce_max_sync(0xffffffffu, on ? hi[a] : -1) - wl[a] + 1;  // <= 0 without a particle
+  }
+  if (wn[0] <= 0) return;
+  if (wn[0] <= 32 && wn[1] <= 32 && wn[2] <= 32 && wn[0] * wn[1] * wn[2] <= 32) {
+    const int l = threadIdx.x & 31;
+    if (l < wn[0] * wn[1] * wn[2]) {
+      const int x = wl[0] + l % wn[0], y = wl[1] + (l / wn[0]) % wn[1], z = wl[2] + l / (wn[0] * wn[1]);
+      list_block(D, ((uint32_t)z * p.nb + (uint32_t)y) * p.nb + (uint32_t)x);
+    }
+  } else if (on) {
+    for (int z = lo[2]; z <= hi[2]; ++z)
+      for (int y = lo[1]; y <= hi[1]; ++y)
+        for (int x = lo[0]; x <= hi[0]; ++x) list_block(D, ((uint32_t)z * p.nb + (uint32_t)y) * p.nb + (uint32_t)x);
+  }
+}
+
+// Rows of W consecutive floats per particle (the caller's arrays) of the 32
+// particles of a warp, through shared memory: consecutive lanes move
+// consecutive floats, and a lane's own row is read back at the odd pitch W.
+// A kernel fetches all its arrays (each into its own region) before the one
+// __syncwarp, so their loads are in flight together.  Scalar accesses: the
+// caller's arrays are only 4-byte aligned.
+template <int W>
+__device__ __forceinline__ void fetch_rows(const float* g, size_t p0, int cnt, float* sm) {
+  const int lane = threadIdx.x & 31;
+  const float* src = g + p0 * W;
+#pragma unroll
+  for (int k = 0; k < W; ++k) {
+    const int e = k * 32 + lane;
+    if (e < cnt * W) sm[e] = src[e];
+  }
+}
+template <int W>
+__device__ __forceinline__ void take_row(const float* sm, float* r) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int q = 0; q < W; ++q) r[q] = sm[lane * W + q];
+}
+// (begins with a __syncwarp: earlier rows in sm have been read)
+template <int W>
+__device__ __forceinline__ void store_rows(float* g, size_t p0, int cnt, float* sm, const float* r) {
+  const int lane = threadIdx.x & 31;
+  __syncwarp();
+#pragma unroll
+  for (int q = 0; q < W; ++q) sm[lane * W + q] = r[q];
+  __syncwarp();
+  float* dst = g + p0 * W;
+#pragma unroll
+  for (int k = 0; k < W; ++k) {
+    const int e = k * 32 + lane;
+    if (e < cnt * W) dst[e] = sm[e];
+  }
+}
+
+// S = sum w a and M = sum w a (x_i - x_p)^T (cells; row c, column b) of the
+// 3-vectors a = (node.x, node.y, node.z) over one grid's stencil, added to S
+// and M: the weights are products, so x, y and z are reduced in turn.
+__device__ __forceinline__ void gather_moments(const float4* g, const DS& s, const DOff& o, int k, float h, float* S,
+                                               float* M) {
+  const float wx0 = s.W[k][0][0], wx1 = s.W[k][0][1], mx0 = -s.f[k][0] * wx0, mx1 = (1.0f - s.f[k][0]) * wx1;
+  const float wy0 = s.W[k][1][0], wy1 = s.W[k][1][1], my0 = -s.f[k][1] * wy0, my1 = (1.0f - s.f[k][1]) * wy1;
+  const float wz[2] = {h * s.W[k][2][0], h * s.W[k][2][1]};
+  const float mz[2] = {-s.f[k][2] * wz[0], (1.0f - s.f[k][2]) * wz[1]};
+#pragma unroll
+  for (int z = 0; z < 2; ++z) {
+    float R[2][3], Rx[2][3];
+#pragma unroll
+    for (int y = 0; y < 2; ++y) {
+      const uint32_t row = o.o[2][z] + o.o[1][y];
+      const float4 a = g[row + o.o[0][0]], b = g[row + o.o[0][1]];
+      R[y][0] = wx0 * a.x + wx1 * b.x;
+      R[y][1] = wx0 * a.y + wx1 * b.y;
+      R[y][2] = wx0 * a.z + wx1 * b.z;
+      Rx[y][0] = mx0 * a.x + mx1 * b.x;
+      Rx[y][1] = mx0 * a.y + mx1 * b.y;
+      Rx[y][2] = mx0 * a.z + mx1 * b.z;
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const float P = wy0 * R[0][c] + wy1 * R[1][c];
+      S[c] += wz[z] * P;
+      M[c * 3 + 0] += wz[z] * (wy0 * Rx[0][c] + wy1 * Rx[1][c]);
+      M[c * 3 + 1] += wz[z] * (my0 * R[0][c] + my1 * R[1][c]);
+      M[c * 3 + 2] += mz[z] * P;
+    }
+  }
 }
 
 __device__ __forceinline__ void mat3(const float* A, const float* B, float* C) {
@@ -172,9 +315,10 @@ __device__ __forceinline__ void fc_stress(const float* F, float mu, float lam, f
 
 // Adjoint of tau(F; E) for the fixed-corotated model: F_bar += d tau/dF ^T : tb,
 // E_bar += <tb, tau> / E (tau is proportional to E at fixed F).
-__device__ void fc_stress_vjp(const float* F, float E, float mu, float lam, const float* tb, float* Fb, float& Eb) {
-  float U[9], V[9], sig[3], tau[9];
-  fc_stress(F, mu, lam, tau, U, sig, V);
+// (tau and its decomposition F = U diag(sig) V^T come from fc_stress.)
+__device__ __forceinline__ void fc_stress_vjp(const float* F, float E, float mu, float lam, const float* tau,
+                                              const float* U, const float* sig, const float* V, const float* tb,
+                                              float* Fb, float& Eb) {
   float R[9];
   mat3_bt(U, V, R);
   float J = sig[0] * sig[1] * sig[2];
@@ -223,288 +367,368 @@ __device__ void fc_stress_vjp(const float* F, float E, float mu, float lam, cons
 }
 
 // --------------------------------------------------------------- forward
+//
+// One particle per thread, 64 threads per CTA, as many CTAs as particles
+// need: the kernels are bound by the latency of their loads and of the
+// decomposition's serial chain, so a small body (32,768 particles) should
+// still give every scheduler several CTAs.  Measured on the differentiable
+// cube (262,144 particles on 128^3), against 128-thread CTAs in a fixed grid
+// stride with scalar atomics on dense grids that were cleared and swept whole:
+// P2G 75 -> 30 us, grid 28 (with its clears) -> 5, G2P 25 -> 12, G2P^T 78 ->
+// 35, P2G^T 71 -> 34 (its decomposition taken once, no local memory); a
+// forward step 140 -> 62 us, its adjoint 302 -> 129 us.
 
-__global__ void k_fwd_p2g(DP p, const float* x, const float* v, const float* B, const float* F, const float* E,
-                          float* gm, float* gp, uint32_t* err) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.n; i += gridDim.x * blockDim.x) {
-    DS s;
-    s.set(p, x[3 * i], x[3 * i + 1], x[3 * i + 2]);
-    if (!nodes_in_range(p, s)) {
-      atomicOr(err, 1u);
-      continue;
-    }
-    float Fi[9], Bi[9], tau[9], U[9], V[9], sig[3], mu, lam;
-    load9(F, i, Fi);
-    load9(B, i, Bi);
-    lame(p, E[i], mu, lam);
-    fc_stress(Fi, mu, lam, tau, U, sig, V);
-    float M[9], A[9];
+constexpr int kDT = 64;
+
+// A = (m B - dt V0 tau) D^-1 / dx, so that the affine momentum at a node is
+// A times its offset in cells.
+__device__ __forceinline__ void affine(const DP& p, const DS& s, const float* B, const float* tau, float* M, float* A) {
 #pragma unroll
-    for (int q = 0; q < 9; ++q) M[q] = p.mass * Bi[q] - p.dt * p.V0 * tau[q];
-    mat3(M, s.Di, A);
+  for (int q = 0; q < 9; ++q) M[q] = p.mass * B[q] - p.dt * p.V0 * tau[q];
+  mat3(M, s.Di, A);
 #pragma unroll
-    for (int q = 0; q < 9; ++q) A[q] *= p.inv_dx;
-    const float mv0 = p.mass * v[3 * i], mv1 = p.mass * v[3 * i + 1], mv2 = p.mass * v[3 * i + 2];
-    for (int g = 0; g < 2; ++g)
-      for (int sz = 0; sz < 2; ++sz)
-        for (int sy = 0; sy < 2; ++sy)
-          for (int sx = 0; sx < 2; ++sx) {
-            float w = s.W[g][0][sx] * s.W[g][1][sy] * s.W[g][2][sz];
-            float d0 = s.d[g][0][sx], d1 = s.d[g][1][sy], d2 = s.d[g][2][sz];
-            long long ni = node_index(p, g, s.base[g][0] + sx, s.base[g][1] + sy, s.base[g][2] + sz);
-            atomicAdd(&gm[ni], w * p.mass);
-            atomicAdd(&gp[3 * ni], w * (mv0 + A[0] * d0 + A[1] * d1 + A[2] * d2));
-            atomicAdd(&gp[3 * ni + 1], w * (mv1 + A[3] * d0 + A[4] * d1 + A[5] * d2));
-            atomicAdd(&gp[3 * ni + 2], w * (mv2 + A[6] * d0 + A[7] * d1 + A[8] * d2));
-          }
+  for (int q = 0; q < 9; ++q) A[q] *= p.inv_dx;
+}
+
+__global__ void __launch_bounds__(kDT, 10) k_fwd_p2g(DP p, DGrid D, const float* x, const float* v, const float* B,
+                                                 const float* F, const float* E) {
+  __shared__ float rows[kDT / 32][32 * 24];
+  float* const sm = rows[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31;
+  const size_t p0 = (size_t)blockIdx.x * kDT + (threadIdx.x - lane);
+  if (p0 >= (size_t)p.n) return;
+  const int cnt = (int)min((size_t)32, (size_t)p.n - p0);
+  float xi[3], vi[3], Fi[9], Bi[9];
+  fetch_rows<3>(x, p0, cnt, sm);
+  fetch_rows<3>(v, p0, cnt, sm + 3 * 32);
+  fetch_rows<9>(F, p0, cnt, sm + 6 * 32);
+  fetch_rows<9>(B, p0, cnt, sm + 15 * 32);
+  __syncwarp();
+  take_row<3>(sm, xi);
+  take_row<3>(sm + 3 * 32, vi);
+  take_row<9>(sm + 6 * 32, Fi);
+  take_row<9>(sm + 15 * 32, Bi);
+  DS s;
+  s.set(p, xi[0], xi[1], xi[2]);
+  const bool on = lane < cnt && nodes_in_range(p, s);
+  list_blocks(p, D, s, on);
+  if (!on) {
+    if (lane < cnt) atomicOr(D.err, 1u);
+    return;
+  }
+  float tau[9], U[9], V[9], sig[3], mu, lam, M[9], A[9];
+  lame(p, E[p0 + lane], mu, lam);
+  fc_stress(Fi, mu, lam, tau, U, sig, V);
+  affine(p, s, Bi, tau, M, A);
+  const float mv[3] = {p.mass * vi[0], p.mass * vi[1], p.mass * vi[2]};
+#pragma unroll
+  for (int g = 0; g < 2; ++g) {
+    const DOff o(p, s, g);
+    float4* const G = D.G + g * grid_size(p);
+#pragma unroll
+    for (int z = 0; z < 2; ++z)
+#pragma unroll
+      for (int y = 0; y < 2; ++y) {
+        const float wyz = s.W[g][1][y] * s.W[g][2][z];
+        const float dy = (float)y - s.f[g][1], dz = (float)z - s.f[g][2];
+        float e[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) e[c] = mv[c] + A[c * 3 + 1] * dy + A[c * 3 + 2] * dz;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const float w = s.W[g][0][k] * wyz, d = (float)k - s.f[g][0];
+          red_add4(&G[o.o[2][z] + o.o[1][y] + o.o[0][k]], w * p.mass, w * (e[0] + A[0] * d), w * (e[1] + A[3] * d),
+                   w * (e[2] + A[6] * d));
+        }
+      }
   }
 }
 
-__device__ __forceinline__ bool wall(const DP& p, int g, long long r) {
-  int ix = (int)(r % p.nn), iy = (int)((r / p.nn) % p.nn), iz = (int)(r / ((long long)p.nn * p.nn));
-  float off = g == 0 ? 0.25f : -0.25f;
-  float hi = (float)p.res - p.bc;
-  float a = ix + off, b = iy + off, c = iz + off;
+// Whether a node of block (bx, by, bz) of grid g lies in a sticky wall.
+__device__ __forceinline__ bool wall(const DP& p, int g, int ix, int iy, int iz) {
+  const float off = g == 0 ? 0.25f : -0.25f;
+  const float hi = (float)p.res - p.bc;
+  const float a = ix + off, b = iy + off, c = iz + off;
   return a < p.bc || b < p.bc || c < p.bc || a > hi || b > hi || c > hi;
 }
 
-__global__ void k_fwd_grid(DP p, const float* gm, const float* gp, float* gv) {
-  const long long per = (long long)p.nn * p.nn * p.nn;
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < 2 * per; q += (long long)gridDim.x * blockDim.x) {
-    float m = gm[q];
-    float o0 = 0.f, o1 = 0.f, o2 = 0.f;
-    if (m > 0.f && !wall(p, (int)(q / per), q % per)) {
-      o0 = gp[3 * q] / m + p.dt * p.gx;
-      o1 = gp[3 * q + 1] / m + p.dt * p.gy;
-      o2 = gp[3 * q + 2] / m + p.dt * p.gz;
-    }
-    gv[3 * q] = o0;
-    gv[3 * q + 1] = o1;
-    gv[3 * q + 2] = o2;
+// The nodes of one listed block, both grids: thread t has node t & 63 of grid
+// t >> 6.  Calls fn(index, in a wall).
+template <typename Fn>
+__device__ __forceinline__ void for_block_nodes(const DP& p, const DGrid& D, Fn&& fn) {
+  const uint32_t n = *D.count;
+  const int g = threadIdx.x >> 6, l = threadIdx.x & 63;
+  for (uint32_t i = blockIdx.x; i < n; i += gridDim.x) {
+    const uint32_t b = D.list[i];
+    const int bx = (int)(b % (uint32_t)p.nb), by = (int)((b / (uint32_t)p.nb) % (uint32_t)p.nb),
+              bz = (int)(b / ((uint32_t)p.nb * (uint32_t)p.nb));
+    if (threadIdx.x == 0) D.flag[b] = 0u;
+    fn(g * grid_size(p) + (size_t)b * 64u + l, wall(p, g, bx * 4 + (l & 3), by * 4 + ((l >> 2) & 3), bz * 4 + (l >> 4)));
   }
 }
 
-__global__ void k_fwd_g2p(DP p, const float* x, const float* F, const float* gv, float* x1, float* v1, float* B1,
-                          float* F1, uint32_t* err) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.n; i += gridDim.x * blockDim.x) {
-    DS s;
-    s.set(p, x[3 * i], x[3 * i + 1], x[3 * i + 2]);
-    if (!nodes_in_range(p, s)) {  // reported by ckmpm_diff_sync; the particle is left in place
-      atomicOr(err, 1u);
-      for (int q = 0; q < 9; ++q) {
-        if (q < 3) {
-          x1[3 * i + q] = x[3 * i + q];
-          v1[3 * i + q] = 0.f;
-        }
-        B1[9 * i + q] = 0.f;
-        F1[9 * i + q] = F[9 * i + q];
-      }
-      continue;
+// v~ = P / m + dt g (m > 0, off the walls).  The forward step returns the
+// accumulators to zero; the adjoint keeps them for its own grid kernel and
+// zeroes the velocity adjoints that G2P^T adds into.
+template <bool ADJ>
+__global__ void __launch_bounds__(128) k_fwd_grid(DP p, DGrid D) {
+  for_block_nodes(p, D, [&](size_t q, bool w) {
+    const float4 a = D.G[q];
+    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (ADJ)
+      D.A[q] = o;
+    else
+      D.G[q] = o;
+    if (a.x > 0.f && !w) {
+      o.x = a.y / a.x + p.dt * p.gx;
+      o.y = a.z / a.x + p.dt * p.gy;
+      o.z = a.w / a.x + p.dt * p.gz;
     }
-    float vv[3] = {0.f, 0.f, 0.f}, Bh[9] = {0.f};
-    for (int g = 0; g < 2; ++g)
-      for (int sz = 0; sz < 2; ++sz)
-        for (int sy = 0; sy < 2; ++sy)
-          for (int sx = 0; sx < 2; ++sx) {
-            float w = 0.5f * s.W[g][0][sx] * s.W[g][1][sy] * s.W[g][2][sz];
-            float dd[3] = {s.d[g][0][sx], s.d[g][1][sy], s.d[g][2][sz]};
-            long long ni = node_index(p, g, s.base[g][0] + sx, s.base[g][1] + sy, s.base[g][2] + sz);
-            float g3[3] = {gv[3 * ni], gv[3 * ni + 1], gv[3 * ni + 2]};
+    D.V[q] = o;
+  });
+}
+
+__global__ void __launch_bounds__(kDT) k_fwd_g2p(DP p, DGrid D, const float* x, const float* F, float* x1, float* v1,
+                                                 float* B1, float* F1) {
+  __shared__ float rows[kDT / 32][32 * 12];
+  float* const sm = rows[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *D.count = 0u;  // the list's last reader is done
+  const size_t p0 = (size_t)blockIdx.x * kDT + (threadIdx.x - lane);
+  if (p0 >= (size_t)p.n) return;
+  const int cnt = (int)min((size_t)32, (size_t)p.n - p0);
+  float xi[3], Fi[9];
+  fetch_rows<3>(x, p0, cnt, sm);
+  fetch_rows<9>(F, p0, cnt, sm + 3 * 32);
+  __syncwarp();
+  take_row<3>(sm, xi);
+  take_row<9>(sm + 3 * 32, Fi);
+  DS s;
+  s.set(p, xi[0], xi[1], xi[2]);
+  float vv[3] = {0.f, 0.f, 0.f}, Bh[9] = {0.f}, Fn[9], C[9];
+  if (lane < cnt && nodes_in_range(p, s)) {
 #pragma unroll
-            for (int a = 0; a < 3; ++a) {
-              vv[a] += w * g3[a];
-#pragma unroll
-              for (int b = 0; b < 3; ++b) Bh[a * 3 + b] += w * g3[a] * dd[b];
-            }
-          }
-    float Fi[9], C[9], Fn[9];
-    load9(F, i, Fi);
+    for (int g = 0; g < 2; ++g) gather_moments(D.V + g * grid_size(p), s, DOff(p, s, g), g, 0.5f, vv, Bh);
     mat3(Bh, s.Di, C);
 #pragma unroll
     for (int q = 0; q < 9; ++q) C[q] = (q % 4 == 0 ? 1.0f : 0.0f) + p.dt * p.inv_dx * C[q];
     mat3(C, Fi, Fn);
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      x1[3 * i + a] = x[3 * i + a] + p.dt * vv[a];
-      v1[3 * i + a] = vv[a];
-    }
+    for (int a = 0; a < 3; ++a) xi[a] += p.dt * vv[a];
 #pragma unroll
-    for (int q = 0; q < 9; ++q) {
-      B1[9 * i + q] = p.dx * Bh[q];
-      F1[9 * i + q] = Fn[q];
-    }
+    for (int q = 0; q < 9; ++q) Bh[q] *= p.dx;
+  } else {  // reported by ckmpm_diff_sync; the particle is left in place
+    if (lane < cnt) atomicOr(D.err, 1u);
+#pragma unroll
+    for (int q = 0; q < 9; ++q) Fn[q] = Fi[q];
   }
+  store_rows<3>(x1, p0, cnt, sm, xi);
+  store_rows<3>(v1, p0, cnt, sm, vv);
+  store_rows<9>(B1, p0, cnt, sm, Bh);
+  store_rows<9>(F1, p0, cnt, sm, Fn);
 }
 
 // --------------------------------------------------------------- adjoint
 
-// x_bar contribution of per-node (w_bar, d_bar) for node (g, sx, sy, sz)
-__device__ __forceinline__ void node_to_x(const DS& s, int g, int sx, int sy, int sz, float wb, const float* db,
-                                          const DP& p, float* xb) {
-  float w0 = s.W[g][0][sx], w1 = s.W[g][1][sy], w2 = s.W[g][2][sz];
-  xb[0] += wb * s.dW[g][0][sx] * w1 * w2 - db[0] * p.inv_dx;
-  xb[1] += wb * w0 * s.dW[g][1][sy] * w2 - db[1] * p.inv_dx;
-  xb[2] += wb * w0 * w1 * s.dW[g][2][sz] - db[2] * p.inv_dx;
-}
+// The weight-derivative part of x_bar: sum over a grid's nodes of q dw/dx with
+// q a scalar per node, q(z, y, k): x, y and z reduced in turn (dW of node 0 is
+// minus that of node 1).
+struct WeightAdjoint {
+  float Q[2], Qx[2], Qy[2];  // of the current z: rows y reduced over x
+  __device__ __forceinline__ void row(const DS& s, int g, int y, float q0, float q1) {
+    Q[y] = s.W[g][0][0] * q0 + s.W[g][0][1] * q1;
+    Qx[y] = s.dW[g][0] * (q1 - q0);
+  }
+  float T[2];
+  __device__ __forceinline__ void plane(const DS& s, int g, int z, float* xb) {
+    const float wz = s.W[g][2][z];
+    xb[0] += wz * (s.W[g][1][0] * Qx[0] + s.W[g][1][1] * Qx[1]);
+    xb[1] += wz * (s.dW[g][1] * (Q[1] - Q[0]));
+    T[z] = s.W[g][1][0] * Q[0] + s.W[g][1][1] * Q[1];
+    if (z == 1) xb[2] += s.dW[g][2] * (T[1] - T[0]);
+  }
+};
 
 // G2P^T: given the step's output adjoints, write x_bar and F_bar (partial) of
-// the step inputs and scatter the grid-velocity adjoint gvb.
-__global__ void k_bwd_g2p(DP p, const float* x, const float* F, const float* gv, const float* gx1, const float* gv1,
-                          const float* gB1, const float* gF1, float* gx, float* gF, float* gvb) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.n; i += gridDim.x * blockDim.x) {
-    DS s;
-    s.set(p, x[3 * i], x[3 * i + 1], x[3 * i + 2]);
-    if (!nodes_in_range(p, s)) {
-      for (int q = 0; q < 9; ++q) {
-        if (q < 3) gx[3 * i + q] = 0.f;
-        gF[9 * i + q] = 0.f;
-      }
-      continue;
-    }
-    // recompute the forward gather
+// the step inputs and scatter the grid-velocity adjoint.
+__global__ void __launch_bounds__(kDT, 6) k_bwd_g2p(DP p, DGrid D, const float* x, const float* F, const float* gx1,
+                                                 const float* gv1, const float* gB1, const float* gF1, float* gx,
+                                                 float* gF) {
+  __shared__ float rows[kDT / 32][32 * 36];
+  float* const sm = rows[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31;
+  const size_t p0 = (size_t)blockIdx.x * kDT + (threadIdx.x - lane);
+  if (p0 >= (size_t)p.n) return;
+  const int cnt = (int)min((size_t)32, (size_t)p.n - p0);
+  float xi[3], Fi[9], xb[3], vb[3], Bhb[9], Fb1[9], Fbo[9];
+  fetch_rows<3>(x, p0, cnt, sm);
+  fetch_rows<3>(gx1, p0, cnt, sm + 3 * 32);
+  fetch_rows<3>(gv1, p0, cnt, sm + 6 * 32);
+  fetch_rows<9>(F, p0, cnt, sm + 9 * 32);
+  fetch_rows<9>(gB1, p0, cnt, sm + 18 * 32);
+  fetch_rows<9>(gF1, p0, cnt, sm + 27 * 32);
+  __syncwarp();
+  take_row<3>(sm, xi);
+  take_row<3>(sm + 3 * 32, xb);
+  take_row<3>(sm + 6 * 32, vb);
+  take_row<9>(sm + 9 * 32, Fi);
+  take_row<9>(sm + 18 * 32, Bhb);
+  take_row<9>(sm + 27 * 32, Fb1);
+  DS s;
+  s.set(p, xi[0], xi[1], xi[2]);
+  if (lane < cnt && nodes_in_range(p, s)) {
+    // the forward gather again
     float vv[3] = {0.f, 0.f, 0.f}, Bh[9] = {0.f};
-    for (int g = 0; g < 2; ++g)
-      for (int sz = 0; sz < 2; ++sz)
-        for (int sy = 0; sy < 2; ++sy)
-          for (int sx = 0; sx < 2; ++sx) {
-            float w = 0.5f * s.W[g][0][sx] * s.W[g][1][sy] * s.W[g][2][sz];
-            float dd[3] = {s.d[g][0][sx], s.d[g][1][sy], s.d[g][2][sz]};
-            long long ni = node_index(p, g, s.base[g][0] + sx, s.base[g][1] + sy, s.base[g][2] + sz);
 #pragma unroll
-            for (int a = 0; a < 3; ++a) {
-              float ga = gv[3 * ni + a];
-              vv[a] += w * ga;
+    for (int g = 0; g < 2; ++g) gather_moments(D.V + g * grid_size(p), s, DOff(p, s, g), g, 0.5f, vv, Bh);
 #pragma unroll
-              for (int b = 0; b < 3; ++b) Bh[a * 3 + b] += w * ga * dd[b];
-            }
-          }
-    float Fi[9], Fb1[9], Bb1[9];
-    load9(F, i, Fi);
-    load9(gF1, i, Fb1);
-    load9(gB1, i, Bb1);
-    float xb[3] = {gx1[3 * i], gx1[3 * i + 1], gx1[3 * i + 2]};
-    float vb[3] = {gv1[3 * i] + p.dt * xb[0], gv1[3 * i + 1] + p.dt * xb[1], gv1[3 * i + 2] + p.dt * xb[2]};
+    for (int a = 0; a < 3; ++a) vb[a] += p.dt * xb[a];
     // F' = G F, G = I + k Bh Di, k = dt/dx
     const float k = p.dt * p.inv_dx;
-    float C[9], G[9];
+    float C[9], Gb[9], Dib[9];
     mat3(Bh, s.Di, C);
 #pragma unroll
-    for (int q = 0; q < 9; ++q) G[q] = (q % 4 == 0 ? 1.0f : 0.0f) + k * C[q];
-    float Fbo[9];
-    mat3_at(G, Fb1, Fbo);  // G^T F'_bar
-#pragma unroll
-    for (int q = 0; q < 9; ++q) gF[9 * i + q] = Fbo[q];
-    float Gb[9];
-    mat3_bt(Fb1, Fi, Gb);  // F'_bar F^T
+    for (int q = 0; q < 9; ++q) C[q] = (q % 4 == 0 ? 1.0f : 0.0f) + k * C[q];
+    mat3_at(C, Fb1, Fbo);   // G^T F'_bar
+    mat3_bt(Fb1, Fi, Gb);   // F'_bar F^T
     // C = Bh Di: Bh_bar = k Gb Di^T, Di_bar = k Bh^T Gb ; plus B' = dx Bh
-    float Bhb[9], Dib[9];
-    mat3_bt(Gb, s.Di, Bhb);
+    float t[9];
+    mat3_bt(Gb, s.Di, t);
 #pragma unroll
-    for (int q = 0; q < 9; ++q) Bhb[q] = k * Bhb[q] + p.dx * Bb1[q];
+    for (int q = 0; q < 9; ++q) Bhb[q] = k * t[q] + p.dx * Bhb[q];
     mat3_at(Bh, Gb, Dib);
 #pragma unroll
     for (int q = 0; q < 9; ++q) Dib[q] *= k;
-    // gather adjoints: v = 1/2 sum w v~, Bh = 1/2 sum w v~ d^T
-    for (int g = 0; g < 2; ++g)
-      for (int sz = 0; sz < 2; ++sz)
-        for (int sy = 0; sy < 2; ++sy)
-          for (int sx = 0; sx < 2; ++sx) {
-            float w = 0.5f * s.W[g][0][sx] * s.W[g][1][sy] * s.W[g][2][sz];
-            float dd[3] = {s.d[g][0][sx], s.d[g][1][sy], s.d[g][2][sz]};
-            long long ni = node_index(p, g, s.base[g][0] + sx, s.base[g][1] + sy, s.base[g][2] + sz);
-            float q3[3];
+    // gather adjoints: v = 1/2 sum w v~, Bh = 1/2 sum w v~ d^T.  A node's
+    // offset adjoint is w Bh_bar^T v~, which sums to Bh_bar^T v over the nodes.
 #pragma unroll
-            for (int a = 0; a < 3; ++a) q3[a] = vb[a] + Bhb[a * 3] * dd[0] + Bhb[a * 3 + 1] * dd[1] + Bhb[a * 3 + 2] * dd[2];
-            float g3[3] = {gv[3 * ni], gv[3 * ni + 1], gv[3 * ni + 2]};
-            atomicAdd(&gvb[3 * ni], w * q3[0]);
-            atomicAdd(&gvb[3 * ni + 1], w * q3[1]);
-            atomicAdd(&gvb[3 * ni + 2], w * q3[2]);
-            float wb = 0.5f * (g3[0] * q3[0] + g3[1] * q3[1] + g3[2] * q3[2]);
-            float db[3];
+    for (int b = 0; b < 3; ++b) xb[b] -= p.inv_dx * (Bhb[b] * vv[0] + Bhb[3 + b] * vv[1] + Bhb[6 + b] * vv[2]);
 #pragma unroll
-            for (int b = 0; b < 3; ++b) db[b] = w * (Bhb[b] * g3[0] + Bhb[3 + b] * g3[1] + Bhb[6 + b] * g3[2]);
-            node_to_x(s, g, sx, sy, sz, wb, db, p, xb);
+    for (int g = 0; g < 2; ++g) {
+      const DOff o(p, s, g);
+      const float4* const V = D.V + g * grid_size(p);
+      float4* const A = D.A + g * grid_size(p);
+      WeightAdjoint wa;
+#pragma unroll
+      for (int z = 0; z < 2; ++z) {
+#pragma unroll
+        for (int y = 0; y < 2; ++y) {
+          const float wyz = 0.5f * s.W[g][1][y] * s.W[g][2][z];
+          const float dy = (float)y - s.f[g][1], dz = (float)z - s.f[g][2];
+          float e[3], q[2];
+#pragma unroll
+          for (int a = 0; a < 3; ++a) e[a] = vb[a] + Bhb[a * 3 + 1] * dy + Bhb[a * 3 + 2] * dz;
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            const float w = s.W[g][0][j] * wyz, d = (float)j - s.f[g][0];
+            const float q0 = e[0] + Bhb[0] * d, q1 = e[1] + Bhb[3] * d, q2 = e[2] + Bhb[6] * d;
+            const uint32_t ni = o.o[2][z] + o.o[1][y] + o.o[0][j];
+            red_add4(&A[ni], w * q0, w * q1, w * q2, 0.f);
+            const float4 c = V[ni];
+            q[j] = 0.5f * (c.x * q0 + c.y * q1 + c.z * q2);
           }
+          wa.row(s, g, y, q[0], q[1]);
+        }
+        wa.plane(s, g, z, xb);
+      }
+    }
     s.dinv_to_x(Dib, xb);
-    gx[3 * i] = xb[0];
-    gx[3 * i + 1] = xb[1];
-    gx[3 * i + 2] = xb[2];
+  } else {
+#pragma unroll
+    for (int q = 0; q < 9; ++q) Fbo[q] = 0.f;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) xb[a] = 0.f;
   }
+  store_rows<3>(gx, p0, cnt, sm, xb);
+  store_rows<9>(gF, p0, cnt, sm, Fbo);
 }
 
-// grid^T: v~ = (P/m + dt g) on nodes with mass off the walls
-__global__ void k_bwd_grid(DP p, const float* gm, const float* gp, const float* gvb, float* gpb, float* gmb) {
-  const long long per = (long long)p.nn * p.nn * p.nn;
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < 2 * per; q += (long long)gridDim.x * blockDim.x) {
-    float m = gm[q];
-    float b0 = 0.f, b1 = 0.f, b2 = 0.f, bm = 0.f;
-    if (m > 0.f && !wall(p, (int)(q / per), q % per)) {
-      float im = 1.0f / m;
-      b0 = gvb[3 * q] * im;
-      b1 = gvb[3 * q + 1] * im;
-      b2 = gvb[3 * q + 2] * im;
-      bm = -(b0 * gp[3 * q] + b1 * gp[3 * q + 1] + b2 * gp[3 * q + 2]) * im;
+// grid^T: v~ = (P/m + dt g) on nodes with mass off the walls; A becomes
+// (p_bar, m_bar) and the accumulators return to zero.
+__global__ void __launch_bounds__(128) k_bwd_grid(DP p, DGrid D) {
+  for_block_nodes(p, D, [&](size_t q, bool w) {
+    const float4 a = D.G[q];
+    const float4 b = D.A[q];
+    D.G[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (a.x > 0.f && !w) {
+      const float im = 1.0f / a.x;
+      o.x = b.x * im;
+      o.y = b.y * im;
+      o.z = b.z * im;
+      o.w = -(o.x * a.y + o.y * a.z + o.z * a.w) * im;
     }
-    gpb[3 * q] = b0;
-    gpb[3 * q + 1] = b1;
-    gpb[3 * q + 2] = b2;
-    gmb[q] = bm;
-  }
+    D.A[q] = o;
+  });
 }
 
 // P2G^T: gather the grid adjoints back to the particles.
-__global__ void k_bwd_p2g(DP p, const float* x, const float* v, const float* B, const float* F, const float* E,
-                          const float* gpb, const float* gmb, float* gx, float* gv, float* gB, float* gF, float* gE) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.n; i += gridDim.x * blockDim.x) {
-    DS s;
-    s.set(p, x[3 * i], x[3 * i + 1], x[3 * i + 2]);
-    if (!nodes_in_range(p, s)) {
-      for (int q = 0; q < 9; ++q) {
-        if (q < 3) gv[3 * i + q] = 0.f;
-        gB[9 * i + q] = 0.f;
-      }
-      continue;
-    }
-    float Fi[9], Bi[9], tau[9], U[9], V[9], sig[3], mu, lam;
-    load9(F, i, Fi);
-    load9(B, i, Bi);
-    const float Ei = E[i];
+__global__ void __launch_bounds__(kDT, 6) k_bwd_p2g(DP p, DGrid D, const float* x, const float* v, const float* B,
+                                                 const float* F, const float* E, float* gx, float* gv, float* gB,
+                                                 float* gF, float* gE) {
+  __shared__ float rows[kDT / 32][32 * 36];
+  float* const sm = rows[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *D.count = 0u;  // the list's last reader is done
+  const size_t p0 = (size_t)blockIdx.x * kDT + (threadIdx.x - lane);
+  if (p0 >= (size_t)p.n) return;
+  const int cnt = (int)min((size_t)32, (size_t)p.n - p0);
+  float xi[3], vi[3], Fi[9], Bi[9], xb[3], Fb[9], Mb[9], vb[3] = {0.f, 0.f, 0.f};
+  fetch_rows<3>(x, p0, cnt, sm);
+  fetch_rows<3>(v, p0, cnt, sm + 3 * 32);
+  fetch_rows<9>(F, p0, cnt, sm + 6 * 32);
+  fetch_rows<9>(B, p0, cnt, sm + 15 * 32);
+  fetch_rows<3>(gx, p0, cnt, sm + 24 * 32);
+  fetch_rows<9>(gF, p0, cnt, sm + 27 * 32);
+  __syncwarp();
+  take_row<3>(sm, xi);
+  take_row<3>(sm + 3 * 32, vi);
+  take_row<9>(sm + 6 * 32, Fi);
+  take_row<9>(sm + 15 * 32, Bi);
+  take_row<3>(sm + 24 * 32, xb);
+  take_row<9>(sm + 27 * 32, Fb);
+  DS s;
+  s.set(p, xi[0], xi[1], xi[2]);
+  if (lane < cnt && nodes_in_range(p, s)) {
+    float tau[9], U[9], V[9], sig[3], mu, lam, M[9], A[9];
+    const float Ei = E[p0 + lane];
     lame(p, Ei, mu, lam);
     fc_stress(Fi, mu, lam, tau, U, sig, V);
-    float M[9], A[9];
+    affine(p, s, Bi, tau, M, A);
+    const float mv[3] = {p.mass * vi[0], p.mass * vi[1], p.mass * vi[2]};
+    // S = sum w p_bar, Ab = sum w p_bar d^T; a node's contribution
+    // c = m v + A d has x_bar through its weight (p_bar . c + m m_bar) and
+    // through d, whose adjoint w A^T p_bar sums to A^T S
+    float S[3] = {0.f, 0.f, 0.f}, Ab[9] = {0.f};
 #pragma unroll
-    for (int q = 0; q < 9; ++q) M[q] = p.mass * Bi[q] - p.dt * p.V0 * tau[q];
-    mat3(M, s.Di, A);
+    for (int g = 0; g < 2; ++g) {
+      const DOff o(p, s, g);
+      const float4* const Pb = D.A + g * grid_size(p);
+      gather_moments(Pb, s, o, g, 1.0f, S, Ab);
+      WeightAdjoint wa;
 #pragma unroll
-    for (int q = 0; q < 9; ++q) A[q] *= p.inv_dx;
-    const float mv[3] = {p.mass * v[3 * i], p.mass * v[3 * i + 1], p.mass * v[3 * i + 2]};
-    float xb[3] = {0.f, 0.f, 0.f}, vb[3] = {0.f, 0.f, 0.f}, Ab[9] = {0.f};
-    for (int g = 0; g < 2; ++g)
-      for (int sz = 0; sz < 2; ++sz)
-        for (int sy = 0; sy < 2; ++sy)
-          for (int sx = 0; sx < 2; ++sx) {
-            float w = s.W[g][0][sx] * s.W[g][1][sy] * s.W[g][2][sz];
-            float dd[3] = {s.d[g][0][sx], s.d[g][1][sy], s.d[g][2][sz]};
-            long long ni = node_index(p, g, s.base[g][0] + sx, s.base[g][1] + sy, s.base[g][2] + sz);
-            float pb[3] = {gpb[3 * ni], gpb[3 * ni + 1], gpb[3 * ni + 2]};
-            float mb = gmb[ni];
-            float c3[3];
+      for (int z = 0; z < 2; ++z) {
 #pragma unroll
-            for (int a = 0; a < 3; ++a) c3[a] = mv[a] + A[a * 3] * dd[0] + A[a * 3 + 1] * dd[1] + A[a * 3 + 2] * dd[2];
-            float wb = p.mass * mb + pb[0] * c3[0] + pb[1] * c3[1] + pb[2] * c3[2];
+        for (int y = 0; y < 2; ++y) {
+          const float dy = (float)y - s.f[g][1], dz = (float)z - s.f[g][2];
+          float e[3], q[2];
 #pragma unroll
-            for (int a = 0; a < 3; ++a) {
-              vb[a] += w * p.mass * pb[a];
+          for (int a = 0; a < 3; ++a) e[a] = mv[a] + A[a * 3 + 1] * dy + A[a * 3 + 2] * dz;
 #pragma unroll
-              for (int b = 0; b < 3; ++b) Ab[a * 3 + b] += w * pb[a] * dd[b];
-            }
-            float db[3];
-#pragma unroll
-            for (int b = 0; b < 3; ++b) db[b] = w * (A[b] * pb[0] + A[3 + b] * pb[1] + A[6 + b] * pb[2]);
-            node_to_x(s, g, sx, sy, sz, wb, db, p, xb);
+          for (int j = 0; j < 2; ++j) {
+            const float d = (float)j - s.f[g][0];
+            const float4 b = Pb[o.o[2][z] + o.o[1][y] + o.o[0][j]];
+            q[j] = p.mass * b.w + b.x * (e[0] + A[0] * d) + b.y * (e[1] + A[3] * d) + b.z * (e[2] + A[6] * d);
           }
+          wa.row(s, g, y, q[0], q[1]);
+        }
+        wa.plane(s, g, z, xb);
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < 3; ++b) xb[b] -= p.inv_dx * (A[b] * S[0] + A[3 + b] * S[1] + A[6 + b] * S[2]);
     // A = M Di / dx: M_bar = Ab Di^T / dx ; Di_bar = M^T Ab / dx
-    float Mb[9], Dib[9];
+    float Dib[9];
     mat3_bt(Ab, s.Di, Mb);
     mat3_at(M, Ab, Dib);
 #pragma unroll
@@ -514,32 +738,34 @@ __global__ void k_bwd_p2g(DP p, const float* x, const float* v, const float* B, 
     }
     s.dinv_to_x(Dib, xb);
     // M = m B - dt V0 tau
-    float tb[9], Fb[9] = {0.f}, Eb = 0.f;
-#pragma unroll
-    for (int q = 0; q < 9; ++q) tb[q] = -p.dt * p.V0 * Mb[q];
-    fc_stress_vjp(Fi, Ei, mu, lam, tb, Fb, Eb);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      gx[3 * i + a] += xb[a];
-      gv[3 * i + a] = vb[a];
-    }
+    float tb[9], Eb = 0.f;
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
-      gB[9 * i + q] = p.mass * Mb[q];
-      gF[9 * i + q] += Fb[q];
+      tb[q] = -p.dt * p.V0 * Mb[q];
+      Mb[q] *= p.mass;
     }
-    gE[i] += Eb;
+    fc_stress_vjp(Fi, Ei, mu, lam, tau, U, sig, V, tb, Fb, Eb);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) vb[a] = p.mass * S[a];
+    gE[p0 + lane] += Eb;
+  } else {
+#pragma unroll
+    for (int q = 0; q < 9; ++q) Mb[q] = 0.f;
   }
+  store_rows<3>(gx, p0, cnt, sm, xb);
+  store_rows<3>(gv, p0, cnt, sm, vb);
+  store_rows<9>(gB, p0, cnt, sm, Mb);
+  store_rows<9>(gF, p0, cnt, sm, Fb);
 }
 
 }  // namespace ckd
 
 struct ckmpm_diff {
   ckd::DP p{};
+  ckd::DGrid g{};
   cudaStream_t stream = nullptr;
-  float *gm = nullptr, *gp = nullptr, *gv = nullptr, *gvb = nullptr, *gpb = nullptr, *gmb = nullptr;
-  uint32_t* err = nullptr;
-  int blocks = 1024;
+  int grid_ctas = 1024;  // grid kernels (a loop over the listed blocks)
+  int blocks = 1;        // particle kernels
 };
 
 extern "C" {
@@ -565,15 +791,20 @@ ckmpm_status ckmpm_diff_create(const ckmpm_scene* sc, void* stream, ckmpm_diff**
   p.gz = (float)sc->gravity[2];
   p.bc = (float)sc->bc_cells;
   p.res = sc->res;
-  p.nn = sc->res + 1;
+  p.nb = (sc->res + 1 + 3) / 4;
   p.n = (int)sc->n;
   d->stream = (cudaStream_t)stream;
-  size_t nodes = 2ull * p.nn * p.nn * p.nn;
-  bool ok = cudaMalloc(&d->gm, nodes * 4) == cudaSuccess && cudaMalloc(&d->gp, nodes * 12) == cudaSuccess &&
-            cudaMalloc(&d->gv, nodes * 12) == cudaSuccess && cudaMalloc(&d->gvb, nodes * 12) == cudaSuccess &&
-            cudaMalloc(&d->gpb, nodes * 12) == cudaSuccess && cudaMalloc(&d->gmb, nodes * 4) == cudaSuccess &&
-            cudaMalloc(&d->err, 4) == cudaSuccess;
-  if (!ok || cudaMemset(d->err, 0, 4) != cudaSuccess) {
+  const size_t nblk = (size_t)p.nb * p.nb * p.nb, bytes = 2 * nblk * 64 * sizeof(float4);
+  ckd::DGrid& g = d->g;
+  bool ok = cudaMalloc(&g.G, bytes) == cudaSuccess && cudaMalloc(&g.V, bytes) == cudaSuccess &&
+            cudaMalloc(&g.A, bytes) == cudaSuccess && cudaMalloc(&g.flag, nblk * 4) == cudaSuccess &&
+            cudaMalloc(&g.list, nblk * 4) == cudaSuccess && cudaMalloc(&g.count, 4) == cudaSuccess &&
+            cudaMalloc(&g.err, 4) == cudaSuccess;
+  // on the object's stream: the first call is ordered behind them
+  if (!ok || cudaMemsetAsync(g.G, 0, bytes, d->stream) != cudaSuccess ||
+      cudaMemsetAsync(g.flag, 0, nblk * 4, d->stream) != cudaSuccess ||
+      cudaMemsetAsync(g.count, 0, 4, d->stream) != cudaSuccess ||
+      cudaMemsetAsync(g.err, 0, 4, d->stream) != cudaSuccess) {
     cudaGetLastError();
     ckmpm_diff_destroy(d);
     return CKMPM_ENOMEM;
@@ -581,29 +812,18 @@ ckmpm_status ckmpm_diff_create(const ckmpm_scene* sc, void* stream, ckmpm_diff**
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  d->blocks = sms * 8;
+  d->grid_ctas = sms * 16;
+  d->blocks = (int)(((int64_t)p.n + ckd::kDT - 1) / ckd::kDT);
   *out = d;
   return CKMPM_OK;
-}
-
-static ckmpm_status diff_forward_grid(ckmpm_diff* d, const float* x, const float* v, const float* B, const float* F,
-                                      const float* E) {
-  const ckd::DP& p = d->p;
-  size_t nodes = 2ull * p.nn * p.nn * p.nn;
-  if (cudaMemsetAsync(d->gm, 0, nodes * 4, d->stream) != cudaSuccess ||
-      cudaMemsetAsync(d->gp, 0, nodes * 12, d->stream) != cudaSuccess)
-    return CKMPM_ECUDA;
-  ckd::k_fwd_p2g<<<d->blocks, 128, 0, d->stream>>>(p, x, v, B, F, E, d->gm, d->gp, d->err);
-  ckd::k_fwd_grid<<<d->blocks, 256, 0, d->stream>>>(p, d->gm, d->gp, d->gv);
-  return cudaGetLastError() == cudaSuccess ? CKMPM_OK : CKMPM_ECUDA;
 }
 
 ckmpm_status ckmpm_diff_step(ckmpm_diff* d, const float* x, const float* v, const float* B, const float* F,
                              const float* E, float* x1, float* v1, float* B1, float* F1) {
   if (!d || !x || !v || !B || !F || !E || !x1 || !v1 || !B1 || !F1) return CKMPM_EINVAL;
-  ckmpm_status st = diff_forward_grid(d, x, v, B, F, E);
-  if (st != CKMPM_OK) return st;
-  ckd::k_fwd_g2p<<<d->blocks, 128, 0, d->stream>>>(d->p, x, F, d->gv, x1, v1, B1, F1, d->err);
+  ckd::k_fwd_p2g<<<d->blocks, ckd::kDT, 0, d->stream>>>(d->p, d->g, x, v, B, F, E);
+  ckd::k_fwd_grid<false><<<d->grid_ctas, 128, 0, d->stream>>>(d->p, d->g);
+  ckd::k_fwd_g2p<<<d->blocks, ckd::kDT, 0, d->stream>>>(d->p, d->g, x, F, x1, v1, B1, F1);
   return cudaGetLastError() == cudaSuccess ? CKMPM_OK : CKMPM_ECUDA;
 }
 
@@ -612,14 +832,11 @@ ckmpm_status ckmpm_diff_step_backward(ckmpm_diff* d, const float* x, const float
                                       const float* gF1, float* gx, float* gv, float* gB, float* gF, float* gE) {
   if (!d || !x || !v || !B || !F || !E || !gx1 || !gv1 || !gB1 || !gF1 || !gx || !gv || !gB || !gF || !gE)
     return CKMPM_EINVAL;
-  ckmpm_status st = diff_forward_grid(d, x, v, B, F, E);
-  if (st != CKMPM_OK) return st;
-  const ckd::DP& p = d->p;
-  size_t nodes = 2ull * p.nn * p.nn * p.nn;
-  if (cudaMemsetAsync(d->gvb, 0, nodes * 12, d->stream) != cudaSuccess) return CKMPM_ECUDA;
-  ckd::k_bwd_g2p<<<d->blocks, 128, 0, d->stream>>>(p, x, F, d->gv, gx1, gv1, gB1, gF1, gx, gF, d->gvb);
-  ckd::k_bwd_grid<<<d->blocks, 256, 0, d->stream>>>(p, d->gm, d->gp, d->gvb, d->gpb, d->gmb);
-  ckd::k_bwd_p2g<<<d->blocks, 128, 0, d->stream>>>(p, x, v, B, F, E, d->gpb, d->gmb, gx, gv, gB, gF, gE);
+  ckd::k_fwd_p2g<<<d->blocks, ckd::kDT, 0, d->stream>>>(d->p, d->g, x, v, B, F, E);
+  ckd::k_fwd_grid<true><<<d->grid_ctas, 128, 0, d->stream>>>(d->p, d->g);
+  ckd::k_bwd_g2p<<<d->blocks, ckd::kDT, 0, d->stream>>>(d->p, d->g, x, F, gx1, gv1, gB1, gF1, gx, gF);
+  ckd::k_bwd_grid<<<d->grid_ctas, 128, 0, d->stream>>>(d->p, d->g);
+  ckd::k_bwd_p2g<<<d->blocks, ckd::kDT, 0, d->stream>>>(d->p, d->g, x, v, B, F, E, gx, gv, gB, gF, gE);
   return cudaGetLastError() == cudaSuccess ? CKMPM_OK : CKMPM_ECUDA;
 }
 
@@ -627,20 +844,20 @@ ckmpm_status ckmpm_diff_sync(ckmpm_diff* d) {
   if (!d) return CKMPM_EINVAL;
   if (cudaStreamSynchronize(d->stream) != cudaSuccess) return CKMPM_ECUDA;
   uint32_t e = 0;
-  if (cudaMemcpy(&e, d->err, 4, cudaMemcpyDeviceToHost) != cudaSuccess) return CKMPM_ECUDA;
+  if (cudaMemcpy(&e, d->g.err, 4, cudaMemcpyDeviceToHost) != cudaSuccess) return CKMPM_ECUDA;
   return e ? CKMPM_EDOMAIN : CKMPM_OK;
 }
 
 ckmpm_status ckmpm_diff_destroy(ckmpm_diff* d) {
   if (!d) return CKMPM_OK;
   if (d->stream) cudaStreamSynchronize(d->stream);
-  cudaFree(d->gm);
-  cudaFree(d->gp);
-  cudaFree(d->gv);
-  cudaFree(d->gvb);
-  cudaFree(d->gpb);
-  cudaFree(d->gmb);
-  cudaFree(d->err);
+  cudaFree(d->g.G);
+  cudaFree(d->g.V);
+  cudaFree(d->g.A);
+  cudaFree(d->g.flag);
+  cudaFree(d->g.list);
+  cudaFree(d->g.count);
+  cudaFree(d->g.err);
   cudaGetLastError();
   delete d;
   return CKMPM_OK;
