@@ -191,9 +191,9 @@ typedef struct {
   int64_t fp64_particles;     /* particles of the last step's float64 pass */
   double ms_last_step;        /* device time of the last step (timing on) */
   double ms_kernel[8];        /* average device ms per launch per kernel since the
-                                 last ckmpm_reset_timing(): 0 bin, 1 scatter,
-                                 2 p2g (fused steps: the leftover P2G), 3 grid
-                                 update, 4 g2p, 5 grid list, 6 float64 pass,
+                                 last ckmpm_reset_timing(): 0 bin, 1 scatter with
+                                 the grid list, 2 p2g (fused steps: the leftover P2G), 3 grid
+                                 update, 4 g2p, 5 (none), 6 float64 pass,
                                  7 fused G2P2G */
   int64_t launches_kernel[8]; /* launches counted in ms_kernel */
   int64_t launches_per_step;  /* kernel launches issued by one step */
@@ -255,7 +255,7 @@ CKMPM_API ckmpm_status ckmpm_release(ckmpm_ctx* ctx, int scene_id);
  * A steady step (no admission, release, upload or probe since the previous
  * one, timing off) is captured once into a CUDA graph per parity of the
  * double-buffered state and replayed after that, which saves the launch
- * gaps of its nine to eleven kernels; any of those operations drops the
+ * gaps of its six to nine kernels; any of those operations drops the
  * graphs.  A stream that cannot be captured (the legacy default stream, or
  * one the caller is capturing) gets direct launches.  CKMPM_GRAPHS=0 in the
  * environment turns graphs off for contexts created afterwards. */

@@ -1,73 +1,50 @@
 // Per-step particle binning by particle block (counting sort on block keys).
 //
 // The histogram of the keys is produced by the previous G2P (or by admission
-// / re-keying).  One step then runs:
-//   scan_tiles  per 4096-key tile: particle count and non-empty key count
-//   scan_top    one CTA: exclusive scan over tiles; resets per-step counters
-//   scan_final  per non-empty key: offset and scatter cursor; non-empty keys
-//               become the particle-block list (in key order, so the list is
-//               deterministic) and flag the 2x2x2 grid blocks they touch
+// / re-keying), and its sums per tile of kScanTile keys by the float64 pass
+// that follows it.  One step then runs two kernels:
+//   scan_final    per non-empty key: first slot and scatter cursor; non-empty
+//                 keys become the particle-block list (in key order, so the
+//                 list is deterministic) and flag the 2x2x2 grid blocks they
+//                 touch.  Each CTA takes one tile and sums the tiles before it.
+//   scatter_glist perm[cursor[key]++] = particle (warp-aggregated atomics) in
+//                 one part of its CTAs; in the other the flagged grid blocks
+//                 become the active grid-block list, flags cleared
+// (A state that changed outside a step first takes its tile sums with
+// scan_tiles; a key space of more than kScanFusedTiles tiles runs scan_tiles
+// and scan_top, one CTA's exclusive scan over the tile sums, every step.)
 // (G2P clears each histogram entry it has used, so the buffer it fills next
 // step starts at zero without a pass over the whole key space.)
-//   scatter     perm[cursor[key]++] = particle (warp-aggregated atomics)
-//   glist       flagged grid blocks -> active grid-block list; flags cleared
+// Against a scan of three kernels over 4096-key tiles and two further ones
+// (five launches), with the float64 pass that takes the tile sums: 14.2 -> 8.2
+// us a step on the elastic cube (32,768 particles, 64^3), 17.2 -> 9.7 on the
+// granular column (346,112, 128^3), 60 -> 50 on 16.27 M particles (512^3).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "common.cuh"
 #include "launch.h"
+#include "scan.cuh"
 
 namespace ck {
 
 constexpr int kScanThreads = 256;
-constexpr int kPerThread = kScanTile / kScanThreads;  // 16
+constexpr int kPerThread = kScanTile / kScanThreads;  // 4: one 16-byte load; a thread's keys are a serial chain
+static_assert(kPerThread == 4, "the scan loads its keys as one uint4");
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(StepView v, BinScratch bs) {
-  const uint32_t base = blockIdx.x * kScanTile;
-  uint32_t c = 0, ne = 0;
-#pragma unroll
-  for (int q = 0; q < kPerThread; ++q) {
-    uint32_t k = base + q * kScanThreads + threadIdx.x;
-    if (k < v.n_keys) {
-      uint32_t x = v.cnt_cur[k];
-      c += x;
-      ne += x ? 1u : 0u;
-    }
-  }
-  __shared__ uint32_t sc[kScanThreads / 32], sn[kScanThreads / 32];
-  for (int o = 16; o > 0; o >>= 1) {
-    c += __shfl_down_sync(0xffffffffu, c, o);
-    ne += __shfl_down_sync(0xffffffffu, ne, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    sc[threadIdx.x >> 5] = c;
-    sn[threadIdx.x >> 5] = ne;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    uint32_t tc = 0, tn = 0;
-    for (int w = 0; w < kScanThreads / 32; ++w) {
-      tc += sc[w];
-      tn += sn[w];
-    }
-    bs.tile_cnt[blockIdx.x] = tc;
-    bs.tile_ne[blockIdx.x] = tn;
-  }
+  write_tile_sums<kScanThreads>(v.cnt_cur, v.n_keys, bs.tile_cnt, bs.tile_ne);
 }
 
 // Exclusive scan of (tile_cnt, tile_ne) in place by one CTA of 1024 threads.
-__global__ void __launch_bounds__(1024) k_scan_top(StepView v, BinScratch bs, uint32_t ntiles) {
+__global__ void __launch_bounds__(1024) k_scan_top(BinScratch bs, uint32_t ntiles) {
   __shared__ uint32_t wc[32], wn[32];
   __shared__ uint32_t carry_c, carry_n;
   if (threadIdx.x == 0) {
     carry_c = 0;
     carry_n = 0;
-    *v.n_g = 0;
-    *v.fp64_count = 0ull;
-    v.work[0] = 0u;
-    v.work[1] = 0u;
-    if (v.lo_count) *v.lo_count = 0u;
   }
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -116,7 +93,6 @@ __global__ void __launch_bounds__(1024) k_scan_top(StepView v, BinScratch bs, ui
     }
     __syncthreads();
   }
-  if (threadIdx.x == 0) *v.n_pb = carry_n;
 }
 
 __device__ __forceinline__ int scene_of_key(const BinScratch& bs, uint32_t key) {
@@ -131,29 +107,34 @@ __device__ __forceinline__ int scene_of_key(const BinScratch& bs, uint32_t key) 
   return (int)bs.scene_tab[2 * lo + 1];
 }
 
+// FUSED: tile_cnt / tile_ne hold the tiles' own sums (else their exclusive scan).
+template <bool FUSED>
 __global__ void __launch_bounds__(kScanThreads) k_scan_final(StepView v, BinScratch bs) {
-  const uint32_t base = blockIdx.x * kScanTile + threadIdx.x * kPerThread;
-  uint32_t c[kPerThread];
-  uint32_t tc = 0, tn = 0;
-  if (base + kPerThread <= v.n_keys) {  // 16 consecutive counts as four 16-byte loads
-    const uint4* p4 = reinterpret_cast<const uint4*>(v.cnt_cur + base);
-#pragma unroll
-    for (int q = 0; q < kPerThread / 4; ++q) {
-      const uint4 x = p4[q];
-      c[4 * q] = x.x;
-      c[4 * q + 1] = x.y;
-      c[4 * q + 2] = x.z;
-      c[4 * q + 3] = x.w;
+  const uint64_t base = (uint64_t)blockIdx.x * kScanTile + threadIdx.x * kPerThread;
+  uint4 x = make_uint4(0u, 0u, 0u, 0u);
+  if (base + kPerThread <= v.n_keys) {
+    x = *reinterpret_cast<const uint4*>(v.cnt_cur + base);
+  } else if (base < v.n_keys) {
+    x.x = v.cnt_cur[base];
+    if (base + 1 < v.n_keys) x.y = v.cnt_cur[base + 1];
+    if (base + 2 < v.n_keys) x.z = v.cnt_cur[base + 2];
+  }
+  // particles and blocks of the tiles before this one
+  uint32_t tpc = 0, tpn = 0;
+  if (FUSED) {
+    for (uint32_t i = threadIdx.x; i < blockIdx.x; i += kScanThreads) {
+      tpc += bs.tile_cnt[i];
+      tpn += bs.tile_ne[i];
     }
+    tpc = __reduce_add_sync(0xffffffffu, tpc);
+    tpn = __reduce_add_sync(0xffffffffu, tpn);
   } else {
-#pragma unroll
-    for (int q = 0; q < kPerThread; ++q) c[q] = base + q < v.n_keys ? v.cnt_cur[base + q] : 0u;
+    tpc = bs.tile_cnt[blockIdx.x];
+    tpn = bs.tile_ne[blockIdx.x];
   }
-#pragma unroll
-  for (int q = 0; q < kPerThread; ++q) {
-    tc += c[q];
-    tn += c[q] ? 1u : 0u;
-  }
+  const uint32_t c[kPerThread] = {x.x, x.y, x.z, x.w};
+  const uint32_t tc = x.x + x.y + x.z + x.w;
+  const uint32_t tn = (x.x != 0u) + (x.y != 0u) + (x.z != 0u) + (x.w != 0u);
   // block-wide exclusive scan of (tc, tn)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t ic = tc, in = tn;
@@ -165,19 +146,38 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_final(StepView v, BinScra
       in += yn;
     }
   }
-  __shared__ uint32_t wc[kScanThreads / 32], wn[kScanThreads / 32];
+  constexpr int NW = kScanThreads / 32;
+  __shared__ uint32_t wc[NW], wn[NW], pcs[NW], pns[NW];
   if (lane == 31) {
     wc[warp] = ic;
     wn[warp] = in;
+    pcs[warp] = tpc;
+    pns[warp] = tpn;
   }
   __syncthreads();
-  uint32_t pc = bs.tile_cnt[blockIdx.x], pn = bs.tile_ne[blockIdx.x];
-  for (int w = 0; w < warp; ++w) {
-    pc += wc[w];
-    pn += wn[w];
+  uint32_t pc = ic - tc, pn = in - tn;
+#pragma unroll
+  for (int w = 0; w < NW; ++w) {
+    if (FUSED || w == 0) {
+      pc += pcs[w];
+      pn += pns[w];
+    }
+    if (w < warp) {
+      pc += wc[w];
+      pn += wn[w];
+    }
   }
-  pc += ic - tc;
-  pn += in - tn;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {  // the step's counters
+    *v.n_g = 0u;
+    *v.fp64_count = 0ull;
+    v.work[0] = 0u;
+    v.work[1] = 0u;
+    if (v.lo_count) *v.lo_count = 0u;
+  }
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == kScanThreads - 1) {
+    *v.n_pb = pn + tn;
+    v.pb[pn + tn] = make_uint2(0u, pc + tc);
+  }
   // the owning scene of the thread's keys, looked up once and kept in
   // registers while the keys stay inside its key range (the stores below
   // could alias the scene table, so reading it per key reloads it each time)
@@ -187,10 +187,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_final(StepView v, BinScra
   long long tbase = 0;
 #pragma unroll
   for (int q = 0; q < kPerThread; ++q) {
-    uint32_t k = base + q;
-    if (k >= v.n_keys) break;
     if (c[q]) {
-      v.offset[k] = pc;
+      const uint32_t k = (uint32_t)base + q;
       v.cursor[k] = pc;
       if (!(k >= klo && (uint64_t)k < khi)) {
         sl = scene_of_key(bs, k);
@@ -201,12 +199,15 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_final(StepView v, BinScra
         tbase = s.table_base;
         khi = (uint64_t)klo + (uint64_t)npb * (uint64_t)npb * (uint64_t)npb;
       }
-      v.pb_key[pn] = k;
+      v.pb[pn] = make_uint2(k, pc);
       v.pb_scene[pn] = (uint32_t)sl;
       int lb = (int)(k - klo);
       int bx = lb % npb, by = (lb / npb) % npb, bz = lb / (npb * npb);
+#pragma unroll
       for (int dz = 0; dz < 2; ++dz)
+#pragma unroll
         for (int dy = 0; dy < 2; ++dy)
+#pragma unroll
           for (int dx = 0; dx < 2; ++dx)
             v.gflag[tbase + ((long long)(bz + dz) * nb + (by + dy)) * nb + (bx + dx)] = (uint32_t)sl + 1u;
       pn += 1;
@@ -220,12 +221,13 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_final(StepView v, BinScra
 // pass is one atomic round trip instead of kScatterUnroll.
 constexpr int kScatterUnroll = 8;
 
-__global__ void __launch_bounds__(256) k_scatter(StepView v) {
+// (CTA `cta` of `ctas`, 256 threads each)
+__device__ __forceinline__ void scatter_particles(const StepView& v, uint32_t cta, uint32_t ctas) {
   const uint32_t lane = threadIdx.x & 31;
-  const uint32_t stride = gridDim.x * blockDim.x * kScatterUnroll;
+  const uint32_t stride = ctas * blockDim.x * kScatterUnroll;
   // the loop runs on the warp's first index, so every lane of a warp takes
   // the same iterations (the full-mask warp intrinsics below need that)
-  for (uint32_t w0 = blockIdx.x * blockDim.x * kScatterUnroll + (threadIdx.x - lane) * kScatterUnroll;
+  for (uint32_t w0 = cta * blockDim.x * kScatterUnroll + (threadIdx.x - lane) * kScatterUnroll;
        w0 < v.n_cur; w0 += stride) {
     const uint32_t j0 = w0 + lane;
     uint32_t key[kScatterUnroll], peers[kScatterUnroll], base[kScatterUnroll];
@@ -268,13 +270,13 @@ __device__ __forceinline__ void glist_assign(const StepView& v, uint32_t g, uint
   v.gflag[g] = 0u;
 }
 
-__global__ void k_glist(StepView v, uint32_t n_vblocks) {
+__device__ __forceinline__ void list_grid_blocks(const StepView& v, uint32_t n_vblocks, uint32_t cta, uint32_t ctas) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t n4 = (reinterpret_cast<uintptr_t>(v.gflag) & 15u) ? 0u : n_vblocks / 4u;
   const uint4* f4 = reinterpret_cast<const uint4*>(v.gflag);
-  const uint32_t wstride = gridDim.x * blockDim.x;
+  const uint32_t wstride = ctas * blockDim.x;
   // every lane of a warp runs the same iterations (full-mask intrinsics)
-  for (uint32_t q0 = blockIdx.x * blockDim.x + (threadIdx.x - lane); q0 < n4; q0 += wstride) {
+  for (uint32_t q0 = cta * blockDim.x + (threadIdx.x - lane); q0 < n4; q0 += wstride) {
     const uint32_t q = q0 + lane;
     const uint4 f = q < n4 ? f4[q] : make_uint4(0u, 0u, 0u, 0u);
     const uint32_t nf = (f.x != 0u) + (f.y != 0u) + (f.z != 0u) + (f.w != 0u);
@@ -294,10 +296,19 @@ __global__ void k_glist(StepView v, uint32_t n_vblocks) {
     if (f.z) glist_assign(v, 4u * q + 2u, f.z, idx++);
     if (f.w) glist_assign(v, 4u * q + 3u, f.w, idx++);
   }
-  for (uint32_t g = 4u * n4 + blockIdx.x * blockDim.x + threadIdx.x; g < n_vblocks; g += wstride) {
+  for (uint32_t g = 4u * n4 + cta * blockDim.x + threadIdx.x; g < n_vblocks; g += wstride) {
     const uint32_t f = v.gflag[g];
     if (f) glist_assign(v, g, f, atomicAdd(v.n_g, 1u));
   }
+}
+
+// The two passes read the scan's results and do not depend on each other: the
+// first `sctas` CTAs scatter, the others list.
+__global__ void __launch_bounds__(256) k_scatter_glist(StepView v, uint32_t n_vblocks, uint32_t sctas) {
+  if (blockIdx.x < sctas)
+    scatter_particles(v, blockIdx.x, sctas);
+  else
+    list_grid_blocks(v, n_vblocks, blockIdx.x - sctas, gridDim.x - sctas);
 }
 
 // Fused step: before a block table is filled again, the entries its last
@@ -331,14 +342,25 @@ void launch_mark_dead(cudaStream_t st, uint32_t* key, uint32_t start, uint32_t n
 
 void launch_bin(cudaStream_t st, const StepView& v, const BinScratch& bs, int which, uint32_t n_gblocks,
                 int grid_ctas) {
-  uint32_t ntiles = (v.n_keys + kScanTile - 1) / kScanTile;
-  if (ntiles == 0) ntiles = 1;
+  const uint32_t ntiles = scan_tiles(v.n_keys);
+  const bool fused = scan_fused(v.n_keys);
+  // CTAs that have work, up to grid_ctas for each pass
+  const uint32_t lim = (uint32_t)grid_ctas;
+  const uint32_t sctas = std::max(1u, std::min(lim, (v.n_cur + 256u * kScatterUnroll - 1u) / (256u * kScatterUnroll)));
+  const uint32_t gctas = std::max(1u, std::min(lim, (n_gblocks + 1023u) / 1024u));
   switch (which) {
     case LB_SCAN_TILES: k_scan_tiles<<<ntiles, kScanThreads, 0, st>>>(v, bs); break;
-    case LB_SCAN_TOP: k_scan_top<<<1, 1024, 0, st>>>(v, bs, ntiles); break;
-    case LB_SCAN_FINAL: k_scan_final<<<ntiles, kScanThreads, 0, st>>>(v, bs); break;
-    case LB_SCATTER: k_scatter<<<grid_ctas, 256, 0, st>>>(v); break;
-    case LB_GLIST: k_glist<<<grid_ctas, 256, 0, st>>>(v, n_gblocks); break;
+    case LB_SCAN_TOP:
+      if (!fused) k_scan_top<<<1, 1024, 0, st>>>(bs, ntiles);
+      break;
+    case LB_SCAN_FINAL:
+      if (fused)
+        k_scan_final<true><<<ntiles, kScanThreads, 0, st>>>(v, bs);
+      else
+        k_scan_final<false><<<ntiles, kScanThreads, 0, st>>>(v, bs);
+      break;
+    case LB_SCATTER_GLIST: k_scatter_glist<<<sctas + gctas, 256, 0, st>>>(v, n_gblocks, sctas); break;
+    case LB_GLIST: k_scatter_glist<<<gctas, 256, 0, st>>>(v, n_gblocks, 0u); break;
   }
 }
 

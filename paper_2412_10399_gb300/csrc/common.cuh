@@ -89,11 +89,13 @@ struct StepView {
   uint32_t* bnd_cur;    // per key: P2G contribution bounds (mass, momentum) of cur, float
                         // bits; P2G clears an active block's pair after use
   uint32_t* bnd_nxt;    // the same for nxt, written by G2P (all zero before it)
-  uint32_t* offset;     // exclusive scan of cnt_cur
   uint32_t* cursor;     // scatter cursors
   uint32_t* perm;       // sorted slot -> index into cur
-  uint32_t* pb_key;     // non-empty particle blocks: key
+  uint2* pb;            // non-empty particle blocks in key order: (key, first sorted slot), and one
+                        // more entry whose slot ends the last block
   uint32_t* pb_scene;   // and owning scene
+  uint32_t* tile_cnt;   // per tile of kScanTile keys: particles and non-empty keys (the input of the
+  uint32_t* tile_ne;    // next scan); null: the float64 pass leaves them to a kernel of their own
   uint32_t* n_pb;       // number of non-empty particle blocks
   uint32_t* gflag;      // per virtual grid block: scene+1 if touched this step
   uint32_t* table;      // per virtual grid block: pool slot (valid if touched this step)
@@ -131,17 +133,35 @@ __device__ __forceinline__ void flag_error(uint32_t* err, uint32_t bit) { atomic
 // Work unit u of the transfer kernels: particle block u / splits, part
 // u % splits of its particles, in whole chunks of `align` particles (a step
 // with few blocks splits each over several units so that every resident
-// warp gets work).  Returns false when that part is empty.
-__device__ __forceinline__ bool unit_range(const StepView& v, uint32_t u, uint32_t align, uint32_t& bi,
-                                           uint32_t& lo, uint32_t& hi) {
+// warp gets work).  A block's entries are three independent loads: its key
+// and first slot, the next block's first slot, its scene.
+struct Unit {
+  uint32_t key, scene, start, cnt;  // the block
+  uint32_t lo, hi;                  // the unit's particles: [lo, hi) of [0, cnt)
+};
+
+// Returns false when the part is empty.
+__device__ __forceinline__ bool unit_of(const StepView& v, uint32_t u, uint32_t align, Unit& q) {
   const uint32_t S = v.splits;
-  bi = u / S;
-  const uint32_t part = u - bi * S;
-  const uint32_t cnt = v.cnt_cur[v.pb_key[bi]];
-  const uint32_t per = ((cnt + S - 1) / S + align - 1) / align * align;
-  lo = part * per;
-  hi = min(cnt, lo + per);
-  return lo < hi;
+  const uint32_t bi = u / S, part = u - bi * S;
+  const uint2 b = v.pb[bi];
+  const uint32_t end = v.pb[bi + 1].y;
+  q.scene = v.pb_scene[bi];
+  q.key = b.x;
+  q.start = b.y;
+  q.cnt = end - b.y;
+  const uint32_t per = ((q.cnt + S - 1) / S + align - 1) / align * align;
+  q.lo = part * per;
+  q.hi = min(q.cnt, q.lo + per);
+  return q.lo < q.hi;
+}
+
+// The next unit of a persistent one-warp CTA: one at a time from the step's
+// counter.
+__device__ __forceinline__ uint32_t next_unit(uint32_t* work) {
+  uint32_t u = 0;
+  if (threadIdx.x == 0) u = atomicAdd(work, 1u);
+  return __shfl_sync(0xffffffffu, u, 0);
 }
 
 // Cell decomposition shared by every kernel that maps a position to nodes.

@@ -101,7 +101,8 @@ struct ckmpm_ctx {
   uint32_t* key[2]{};
   uint32_t* cnt[2]{};
   uint32_t* bnd[2]{};  // per key: P2G contribution bounds (2 floats as bits)
-  uint32_t *offset = nullptr, *cursor = nullptr, *perm = nullptr, *pb_key = nullptr, *pb_scene = nullptr;
+  uint32_t *cursor = nullptr, *perm = nullptr, *pb_scene = nullptr;
+  uint2* pb = nullptr;
   uint32_t *counters = nullptr;  // [0] n_pb, [1] n_g, [2] err, [4..5] fp64 (64-bit), [6..7] work,
                                  // [8] n_g of the second table set, [9] leftover count
   // fused G2P2G steps: a second block-table set for the next step's grid,
@@ -120,6 +121,9 @@ struct ckmpm_ctx {
   uint32_t* fp64_list = nullptr;  // particles of the float64 pass (capacity cap_n)
   uint32_t *gflag = nullptr, *table = nullptr, *g_list = nullptr, *g_scene = nullptr;
   uint32_t *tile_cnt = nullptr, *tile_ne = nullptr, *scene_tab = nullptr;
+  // key-space size whose tile sums of cnt[cur] are in tile_cnt / tile_ne (left
+  // there by the last step's float64 pass); 0: the next step takes them itself
+  uint32_t tiles_keys = 0;
   float4 *Gacc = nullptr, *Gvel = nullptr;
   SceneDev* d_scenes = nullptr;
   MatDev* d_mats = nullptr;
@@ -241,10 +245,9 @@ ck::StepView make_view(ckmpm_ctx* ctx) {
   v.cnt_nxt = ctx->cnt[ctx->cur ^ 1];
   v.bnd_cur = ctx->bnd[ctx->cur];
   v.bnd_nxt = ctx->bnd[ctx->cur ^ 1];
-  v.offset = ctx->offset;
   v.cursor = ctx->cursor;
   v.perm = ctx->perm;
-  v.pb_key = ctx->pb_key;
+  v.pb = ctx->pb;
   v.pb_scene = ctx->pb_scene;
   v.n_pb = ctx->counters + 0;
   v.n_g = ctx->counters + (ctx->tsel == 0 ? 1 : 8);
@@ -264,6 +267,10 @@ ck::StepView make_view(ckmpm_ctx* ctx) {
   v.n_mats = (uint32_t)ctx->cap_mats;
   v.n_keys = (uint32_t)std::max<int64_t>(ctx->keys_alloc.high, 1);
   v.n_cur = (uint32_t)ctx->n_cur;
+  if (ck::scan_fused(v.n_keys)) {
+    v.tile_cnt = ctx->tile_cnt;
+    v.tile_ne = ctx->tile_ne;
+  }
   v.keep_gacc = 0;
   // a step with few particles splits each block over several work units, so
   // that the resident warps of the transfer kernels (about 20 per SM) get two
@@ -556,8 +563,8 @@ ckmpm_status init_ctx(ckmpm_ctx* ctx, const ckmpm_config* cfg) {
             alloc_n(ctx, ctx->perm, ctx->cap_n) && alloc_n(ctx, ctx->fp64_list, ctx->cap_n) &&
             alloc_n(ctx, ctx->cnt[0], ctx->cap_keys) &&
             alloc_n(ctx, ctx->cnt[1], ctx->cap_keys) && alloc_n(ctx, ctx->bnd[0], 2 * ctx->cap_keys) &&
-            alloc_n(ctx, ctx->bnd[1], 2 * ctx->cap_keys) && alloc_n(ctx, ctx->offset, ctx->cap_keys) &&
-            alloc_n(ctx, ctx->cursor, ctx->cap_keys) && alloc_n(ctx, ctx->pb_key, ctx->cap_keys) &&
+            alloc_n(ctx, ctx->bnd[1], 2 * ctx->cap_keys) &&
+            alloc_n(ctx, ctx->cursor, ctx->cap_keys) && alloc_n(ctx, ctx->pb, ctx->cap_keys + 1) &&
             alloc_n(ctx, ctx->pb_scene, ctx->cap_keys) && alloc_n(ctx, ctx->counters, 12) &&
             alloc_n(ctx, ctx->gflag, ctx->cap_vblocks) && alloc_n(ctx, ctx->table, ctx->cap_vblocks) &&
             alloc_n(ctx, ctx->g_list, ctx->cap_pool) && alloc_n(ctx, ctx->g_scene, ctx->cap_pool) &&
@@ -656,7 +663,11 @@ ckmpm_status run_step(ckmpm_ctx* ctx, bool probe) {
   if (ctx->fused) ctx->grid_valid = false;  // a probe reuses the grid arrays
   ck::StepView v = make_view(ctx);
   ckmpm_ctx::EvPair ep{};
-  const bool steady = !probe && !ctx->timing && !ctx->grids_dirty && !ctx->keys_dirty;
+  const bool fused_scan = ck::scan_fused(v.n_keys);
+  if (ctx->keys_dirty) ctx->tiles_keys = 0;
+  const bool own_tiles = !fused_scan || ctx->tiles_keys != v.n_keys;
+  const bool steady =
+      !probe && !ctx->timing && !ctx->grids_dirty && !ctx->keys_dirty && !(fused_scan && own_tiles);
   if (probe) drop_graphs(ctx);  // the probe refills the block table the graphs were captured with
   if (ctx->grids_dirty) {
     ck::launch_transfer(ctx->kind, ctx->lc, v, ck::LK_CLEAR);
@@ -674,6 +685,7 @@ ckmpm_status run_step(ckmpm_ctx* ctx, bool probe) {
   int64_t n_live = 0;
   for (auto& s : ctx->scenes) n_live += s.alive ? s.n : 0;
   if (n_live == 0) {
+    ctx->tiles_keys = 0;
     if (!probe) {
       ctx->n_cur = 0;
       ctx->layout.clear();
@@ -693,15 +705,12 @@ ckmpm_status run_step(ckmpm_ctx* ctx, bool probe) {
   v.keep_gacc = probe ? 1u : 0u;
   auto issue = [&]() {
   tbeg(ctx, ep, 0);
-  ck::launch_bin(ctx->stream, v, bs, ck::LB_SCAN_TILES, ngb, grid_ctas);
+  if (own_tiles) ck::launch_bin(ctx->stream, v, bs, ck::LB_SCAN_TILES, ngb, grid_ctas);
   ck::launch_bin(ctx->stream, v, bs, ck::LB_SCAN_TOP, ngb, grid_ctas);
   ck::launch_bin(ctx->stream, v, bs, ck::LB_SCAN_FINAL, ngb, grid_ctas);
   tend(ctx, ep);
   tbeg(ctx, ep, 1);
-  ck::launch_bin(ctx->stream, v, bs, ck::LB_SCATTER, ngb, grid_ctas);
-  tend(ctx, ep);
-  tbeg(ctx, ep, 5);
-  ck::launch_bin(ctx->stream, v, bs, ck::LB_GLIST, ngb, grid_ctas);
+  ck::launch_bin(ctx->stream, v, bs, ck::LB_SCATTER_GLIST, ngb, grid_ctas);
   tend(ctx, ep);
   tbeg(ctx, ep, 2);
   ck::launch_transfer(ctx->kind, ctx->lc, v, ck::LK_P2G);
@@ -718,6 +727,8 @@ ckmpm_status run_step(ckmpm_ctx* ctx, bool probe) {
   tend(ctx, ep);
   };
   if (!(steady && !ctx->fused && graph_step(ctx, ctx->cur, issue))) issue();
+  // a probe leaves the tile sums of the current state, a step those of the next
+  ctx->tiles_keys = fused_scan ? v.n_keys : 0;
   if (probe) {
     ctx->grids_dirty = true;
     CK_TRY(cudaGetLastError(), "probe launch");
@@ -761,10 +772,12 @@ ckmpm_status run_step_fused(ckmpm_ctx* ctx) {
                        ctx->bnd[ctx->cur], ctx->d_scenes, ctx->d_mats, (uint32_t)ctx->n_cur, v.err);
     ctx->keys_dirty = false;
     ctx->grid_valid = false;
+    ctx->tiles_keys = 0;
   }
   int64_t n_live = 0;
   for (auto& s : ctx->scenes) n_live += s.alive ? s.n : 0;
   if (n_live == 0) {
+    ctx->tiles_keys = 0;
     ctx->n_cur = 0;
     ctx->layout.clear();
     ctx->steps++;
@@ -782,6 +795,8 @@ ckmpm_status run_step_fused(ckmpm_ctx* ctx) {
   ctx->tsel = ns;
   ck::StepView vn = make_view(ctx);
   ctx->tsel = cs;
+  const bool fused_scan = ck::scan_fused(vc.n_keys);
+  const bool own_tiles = !fused_scan || ctx->tiles_keys != vc.n_keys;
   ckmpm_ctx::EvPair ep{};
   if (ctx->timing) cudaEventRecord(ctx->step_a, ctx->stream);
   // the fused kernel gathers through set cs and scatters through set ns
@@ -810,20 +825,18 @@ ckmpm_status run_step_fused(ckmpm_ctx* ctx) {
   auto issue_steady = [&]() {
     ck::launch_table_reset(ctx->stream, vn.table, vn.g_list, vn.n_g, vn.pool_cap, grid_ctas);
     tbeg(ctx, ep, 0);
-    ck::launch_bin(ctx->stream, vn, bs, ck::LB_SCAN_TILES, ngb, grid_ctas);
+    if (own_tiles) ck::launch_bin(ctx->stream, vn, bs, ck::LB_SCAN_TILES, ngb, grid_ctas);
     ck::launch_bin(ctx->stream, vn, bs, ck::LB_SCAN_TOP, ngb, grid_ctas);
     ck::launch_bin(ctx->stream, vn, bs, ck::LB_SCAN_FINAL, ngb, grid_ctas);
     tend(ctx, ep);
     tbeg(ctx, ep, 1);
-    ck::launch_bin(ctx->stream, vn, bs, ck::LB_SCATTER, ngb, grid_ctas);
-    tend(ctx, ep);
-    tbeg(ctx, ep, 5);
-    ck::launch_bin(ctx->stream, vn, bs, ck::LB_GLIST, ngb, grid_ctas);
+    ck::launch_bin(ctx->stream, vn, bs, ck::LB_SCATTER_GLIST, ngb, grid_ctas);
     tend(ctx, ep);
     issue_fused();
   };
   if (ctx->grid_valid) {
-    if (!(was_clean && graph_step(ctx, ctx->cur + 2 * ctx->tsel, issue_steady))) issue_steady();
+    if (!(was_clean && !(fused_scan && own_tiles) && graph_step(ctx, ctx->cur + 2 * ctx->tsel, issue_steady)))
+      issue_steady();
   } else {
     // every table set is cleared of the entries its last fill assigned (its
     // list records them, slots claimed by the leftover P2G included) before
@@ -831,20 +844,19 @@ ckmpm_status run_step_fused(ckmpm_ctx* ctx) {
     ck::launch_table_reset(ctx->stream, vn.table, vn.g_list, vn.n_g, vn.pool_cap, grid_ctas);
     // prologue: binning, P2G and grid update of the current state into set cs
     ck::launch_table_reset(ctx->stream, vc.table, vc.g_list, vc.n_g, vc.pool_cap, grid_ctas);
-    ck::launch_bin(ctx->stream, vc, bs, ck::LB_SCAN_TILES, ngb, grid_ctas);
+    if (own_tiles) ck::launch_bin(ctx->stream, vc, bs, ck::LB_SCAN_TILES, ngb, grid_ctas);
     ck::launch_bin(ctx->stream, vc, bs, ck::LB_SCAN_TOP, ngb, grid_ctas);
     ck::launch_bin(ctx->stream, vc, bs, ck::LB_SCAN_FINAL, ngb, grid_ctas);
-    ck::launch_bin(ctx->stream, vc, bs, ck::LB_SCATTER, ngb, grid_ctas);
-    ck::launch_bin(ctx->stream, vc, bs, ck::LB_GLIST, ngb, grid_ctas);
+    ck::launch_bin(ctx->stream, vc, bs, ck::LB_SCATTER_GLIST, ngb, grid_ctas);
     ck::launch_transfer(ctx->kind, ctx->lc, vc, ck::LK_P2G);
     ck::launch_transfer(ctx->kind, ctx->lc, vc, ck::LK_UPDATE);
     // the same particle blocks flag the next step's grid blocks
-    CK_TRY(cudaMemsetAsync(vn.n_g, 0, sizeof(uint32_t), ctx->stream), "memset");
     ck::launch_bin(ctx->stream, vn, bs, ck::LB_SCAN_FINAL, ngb, grid_ctas);
     ck::launch_bin(ctx->stream, vn, bs, ck::LB_GLIST, ngb, grid_ctas);
     issue_fused();
     ctx->grid_valid = true;
   }
+  ctx->tiles_keys = fused_scan ? vc.n_keys : 0;
   if (ctx->timing) cudaEventRecord(ctx->step_b, ctx->stream);
   CK_TRY(cudaGetLastError(), "step launch");
   ctx->cur ^= 1;
@@ -1013,6 +1025,7 @@ ckmpm_status admit_impl(ckmpm_ctx* ctx, const ckmpm_scene* sc, int* scene_id) {
   }
   ctx->layout.push_back({slot, ctx->n_cur, sc->n});
   ctx->grid_valid = false;
+  ctx->tiles_keys = 0;
   drop_graphs(ctx);  // particle count, key space and scene table changed
   ctx->n_cur += sc->n;
   if (scene_id) *scene_id = slot;
@@ -1117,6 +1130,7 @@ ckmpm_status ckmpm_release(ckmpm_ctx* ctx, int scene_id) {
          "memset");
   h.alive = false;
   ctx->grid_valid = false;
+  ctx->tiles_keys = 0;
   drop_graphs(ctx);
   ctx->h_scenes[scene_id].alive = 0;
   CK_TRY(cudaMemcpyAsync(ctx->d_scenes + scene_id, &ctx->h_scenes[scene_id], sizeof(SceneDev), cudaMemcpyHostToDevice,
@@ -1360,7 +1374,10 @@ ckmpm_status ckmpm_get_stats(ckmpm_ctx* ctx, ckmpm_stats* out) {
     out->ms_kernel[i] = ctx->ms_cnt[i] ? ctx->ms_sum[i] / ctx->ms_cnt[i] : 0.0;
     out->launches_kernel[i] = ctx->ms_cnt[i];
   }
-  out->launches_per_step = ctx->fused ? 11 : 9;
+  // split: scan, scatter with the grid list, P2G, grid update, G2P, float64
+  // pass; a key space too large for the fused scan takes two more
+  const bool one_scan = ck::scan_fused((uint32_t)std::max<int64_t>(ctx->keys_alloc.high, 1));
+  out->launches_per_step = (ctx->fused ? 7 : 6) + (one_scan ? 0 : 2);
   return CKMPM_OK;
 }
 

@@ -36,7 +36,15 @@ void launch_rekey(int kind, cudaStream_t st, Pool P, uint32_t* key, uint32_t* cn
                   const SceneDev* scenes, const MatDev* mats, uint32_t n, uint32_t* err);
 
 // bin.cu
-constexpr int kScanTile = 4096;  // keys per scan tile
+constexpr int kScanTile = 1024;  // keys per scan tile
+// Up to this many tiles every CTA of the scan sums the tiles before its own
+// (at most 16 loads a thread); beyond, one CTA scans the tile sums first.
+constexpr uint32_t kScanFusedTiles = 4096;
+__host__ __device__ inline uint32_t scan_tiles(uint32_t n_keys) {
+  const uint32_t t = (uint32_t)(((uint64_t)n_keys + kScanTile - 1) / kScanTile);
+  return t ? t : 1u;
+}
+inline bool scan_fused(uint32_t n_keys) { return scan_tiles(n_keys) <= kScanFusedTiles; }
 struct BinScratch {
   uint32_t* tile_cnt;   // per tile: sum of counts
   uint32_t* tile_ne;    // per tile: non-empty keys
@@ -45,7 +53,8 @@ struct BinScratch {
 };
 void launch_bin(cudaStream_t st, const StepView& v, const BinScratch& bs, int which, uint32_t n_gblocks,
                 int grid_ctas);
-enum { LB_SCAN_TILES = 0, LB_SCAN_TOP = 1, LB_SCAN_FINAL = 2, LB_SCATTER = 3, LB_GLIST = 4 };
+// LB_SCAN_TOP launches nothing when the scan is fused (scan_fused)
+enum { LB_SCAN_TILES = 0, LB_SCAN_TOP = 1, LB_SCAN_FINAL = 2, LB_SCATTER_GLIST = 3, LB_GLIST = 4 };
 void launch_mark_dead(cudaStream_t st, uint32_t* key, uint32_t start, uint32_t n);
 void launch_table_reset(cudaStream_t st, uint32_t* table, const uint32_t* g_list, const uint32_t* n_g,
                         uint32_t pool_cap, int grid_ctas);

@@ -134,7 +134,7 @@ extern "C" CKMPM_API ckmpm_status ckmpm_p2g_grids_static(const ckmpm_scene* sc, 
   const int64_t n = sc->n;
   const int64_t npb = (sc->res + 3) / 4, nb = npb + 1;
   const int64_t nkeys = npb * npb * npb, nvb = nb * nb * nb;
-  const int64_t ntiles = (nkeys + ck::kScanTile - 1) / ck::kScanTile;
+  const int64_t ntiles = ck::scan_tiles((uint32_t)nkeys);
 
   Carve cv{(char*)base};
   ck::Pool P{};
@@ -156,10 +156,9 @@ extern "C" CKMPM_API ckmpm_status ckmpm_p2g_grids_static(const ckmpm_scene* sc, 
   v.cnt_nxt = cv.take<uint32_t>(nkeys);
   v.bnd_cur = cv.take<uint32_t>(2 * nkeys);
   v.bnd_nxt = cv.take<uint32_t>(2 * nkeys);
-  v.offset = cv.take<uint32_t>(nkeys);
   v.cursor = cv.take<uint32_t>(nkeys);
   v.perm = cv.take<uint32_t>(n);
-  v.pb_key = cv.take<uint32_t>(nkeys);
+  v.pb = cv.take<uint2>(nkeys + 1);
   v.pb_scene = cv.take<uint32_t>(nkeys);
   uint32_t* counters = cv.take<uint32_t>(8);
   v.n_pb = counters + 0;
@@ -264,8 +263,7 @@ extern "C" CKMPM_API ckmpm_status ckmpm_p2g_grids_static(const ckmpm_scene* sc, 
   ck::launch_bin(st, v, bs, ck::LB_SCAN_TILES, (uint32_t)nvb, grid_ctas);
   ck::launch_bin(st, v, bs, ck::LB_SCAN_TOP, (uint32_t)nvb, grid_ctas);
   ck::launch_bin(st, v, bs, ck::LB_SCAN_FINAL, (uint32_t)nvb, grid_ctas);
-  ck::launch_bin(st, v, bs, ck::LB_SCATTER, (uint32_t)nvb, grid_ctas);
-  ck::launch_bin(st, v, bs, ck::LB_GLIST, (uint32_t)nvb, grid_ctas);
+  ck::launch_bin(st, v, bs, ck::LB_SCATTER_GLIST, (uint32_t)nvb, grid_ctas);
   ck::LaunchCfg lc{st, sms * 8};
   lc.transfer = pic ? 1 : 0;
   ck::launch_transfer(kernel, lc, v, ck::LK_P2G);
