@@ -2,8 +2,9 @@
 //
 // Particle pool (structure of arrays, double-buffered, 16-byte vectors):
 //   X   float4 (x, y, z, material index as bits)
-//   VM0 float4 (vx, vy, vz, M00)   VM1 (M01, M02, M10, M11)   VM2 (M12, M20, M21, M22)
-//   F0  float4 (F00, F01, F02, F10)  F1 (F11, F12, F20, F21)  F2 float F22
+//   VM0 float4 (vx, vy, vz, M22)   VM1 (M00, M10, M01, M11)   VM2 (M02, M12, M20, M21)
+//   F0  float4 (F00, F10, F01, F11)  F1 (F02, F12, F20, F21)  F2 float F22
+// (rows 0 and 1 of a matrix side by side: the pairs of the packed arithmetic)
 //   ID  uint32 scene-local particle index
 // M = m B - dt V0 tau(F) is the per-particle matrix that P2G multiplies by
 // D(x)^-1: it carries both the APIC affine momentum (Sec. 4.4) and the MLS
@@ -49,15 +50,17 @@ struct SceneDev {
   int alive;
 };
 
-struct MatDev {
-  int model;      // 0 fixed-corotated, 1 Drucker-Prager, 2 J-based fluid
-  int scene;      // owning scene slot
-  float mu, lam;  // Lame parameters
+// Two 16-byte groups of what the update reads together, then the indices.
+struct alignas(16) MatDev {
   float mass;     // rho * V0
-  float alpha;    // Drucker-Prager cone coefficient
+  float mu, lam;  // Lame parameters
   float dpc;      // Drucker-Prager: (3 lam + 2 mu) / (2 mu) alpha = alpha (1 + nu) / (1 - 2 nu), any E
+  float alpha;    // Drucker-Prager cone coefficient
   float E, nu;    // for per-particle E; the fluid's equation-of-state constant B is E
   float gamma;    // fluid equation-of-state exponent
+  int model;      // 0 fixed-corotated, 1 Drucker-Prager, 2 J-based fluid
+  int scene;      // owning scene slot
+  int pad_[2];
 };
 
 // Pointers to one buffer of the particle pool.
@@ -71,9 +74,8 @@ struct Pool {
   float* F2;
   uint32_t* ID;
   float* E;  // optional per-particle Young's modulus (may be null)
-  // APIC with the kernel gradient only (else null): T = -dt V0 tau, row-major
-  // in T0 (T00, T01, T02, T10), T1 (T11, T12, T20, T21), T2 T22; VM then
-  // holds m B without the stress
+  // APIC with the kernel gradient only (else null): T = -dt V0 tau in the
+  // order of F (T0, T1, T2); VM then holds m B without the stress
   float4* T0;
   float4* T1;
   float* T2;
@@ -210,8 +212,8 @@ __device__ __forceinline__ bool in_domain(float u, int res) {
   return u >= 0.5f && u < (float)res - 0.5f;
 }
 
-template <int KIND>
-__device__ __forceinline__ uint32_t particle_key(const SceneDev& s, float ux, float uy, float uz) {
+template <int KIND, typename SceneT>
+__device__ __forceinline__ uint32_t particle_key(const SceneT& s, float ux, float uy, float uz) {
   Cell<KIND> cx, cy, cz;
   cx.set(ux);
   cy.set(uy);

@@ -15,6 +15,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "pack.cuh"
+
 namespace ck {
 
 template <typename T>
@@ -384,32 +386,22 @@ __device__ __forceinline__ void constitutive_left(int model, T* F, T mu, T lam, 
 }
 
 // ------------------------------------------- Drucker-Prager for small stretches
-//
-// Symmetric 3x3 matrices as (00, 11, 22, 01, 02, 12).  sym_mul forms A B for
-// commuting symmetric A and B (polynomials in one matrix), which is symmetric.
-__device__ __forceinline__ void sym_mul(const float* a, const float* b, float* c) {
-  c[0] = a[0] * b[0] + a[3] * b[3] + a[4] * b[4];
-  c[1] = a[3] * b[3] + a[1] * b[1] + a[5] * b[5];
-  c[2] = a[4] * b[4] + a[5] * b[5] + a[2] * b[2];
-  c[3] = a[0] * b[3] + a[3] * b[1] + a[4] * b[5];
-  c[4] = a[0] * b[4] + a[3] * b[5] + a[4] * b[2];
-  c[5] = a[3] * b[4] + a[1] * b[5] + a[5] * b[2];
-}
 
 // X = F F^T - I from D = F - I as D + D^T + D D^T (no cancellation against the
-// identity), and its largest row abs-sum.
-__device__ __forceinline__ float left_strain(const float* F, float* X) {
-  const float d[9] = {F[0] - 1.f, F[1], F[2], F[3], F[4] - 1.f, F[5], F[6], F[7], F[8] - 1.f};
-  X[0] = 2.f * d[0] + (d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-  X[1] = 2.f * d[4] + (d[3] * d[3] + d[4] * d[4] + d[5] * d[5]);
-  X[2] = 2.f * d[8] + (d[6] * d[6] + d[7] * d[7] + d[8] * d[8]);
-  X[3] = d[1] + d[3] + (d[0] * d[3] + d[1] * d[4] + d[2] * d[5]);
-  X[4] = d[2] + d[6] + (d[0] * d[6] + d[1] * d[7] + d[2] * d[8]);
-  X[5] = d[5] + d[7] + (d[3] * d[6] + d[4] * d[7] + d[5] * d[8]);
-  const float r0 = fabsf(X[0]) + fabsf(X[3]) + fabsf(X[4]);
-  const float r1 = fabsf(X[3]) + fabsf(X[1]) + fabsf(X[5]);
-  const float r2 = fabsf(X[4]) + fabsf(X[5]) + fabsf(X[2]);
-  return fmaxf(r0, fmaxf(r1, r2));
+// identity); returns its largest row abs-sum.
+__device__ __forceinline__ float left_strain(const M3& F, Sym& X) {
+  const float d00 = F.c[0].p.x - 1.f, d11 = F.c[1].p.y - 1.f, d22 = F.c[2].z - 1.f;
+  const f2 c0 = pk(d00, F.c[0].p.y), c1 = pk(F.c[1].p.x, d11), c2 = F.c[2].p;  // columns' rows 0, 1
+  const float r0 = F.c[0].z, r1 = F.c[1].z;                                     // row 2
+  const f2 s = fma2(c0, c0, fma2(c1, c1, mul2(c2, c2)));
+  X.d = pk(fmaf(2.f, d00, s.x), fmaf(2.f, d11, s.y));
+  X.o = fma2(c0, dup(r0), fma2(c1, dup(r1), fma2(c2, dup(d22), add2(c2, pk(r0, r1)))));
+  X.c = fmaf(2.f, d22, fmaf(r0, r0, fmaf(r1, r1, d22 * d22)));
+  X.e = c1.x + c0.y + fmaf(c0.x, c0.y, fmaf(c1.x, c1.y, c2.x * c2.y));
+  const float a = fabsf(X.d.x) + fabsf(X.e) + fabsf(X.o.x);
+  const float b = fabsf(X.e) + fabsf(X.d.y) + fabsf(X.o.y);
+  const float c = fabsf(X.o.x) + fabsf(X.o.y) + fabsf(X.c);
+  return fmaxf(a, fmaxf(b, c));
 }
 
 // The Drucker-Prager update of Sec. 3.2 step 4 (klar2016 return map, Hencky
@@ -431,96 +423,39 @@ __device__ __forceinline__ float left_strain(const float* F, float* X) {
 // do not diverge; the degree-4 case is the one this update always used.
 __device__ __forceinline__ int dp_lane_degree(float xr) { return xr <= 3.4e-4f ? 2 : xr <= 5.4e-3f ? 3 : 4; }
 
-// lane_deg: dp_lane_degree of the particle's xr
-__device__ __forceinline__ void dp_small_strain(float* F, const float* X, int lane_deg, float mu, float lam,
-                                                float dpc, float* tau) {
+// lane_deg: dp_lane_degree of the particle's xr; tau comes out times ts.
+__device__ __forceinline__ void dp_small_strain(M3& F, const Sym& X, int lane_deg, float mu, float lam, float dpc,
+                                                float ts, Sym& tau) {
   const int deg = __reduce_max_sync(__activemask(), lane_deg);
-  float Z[6], W[6];
   // log(I + X) = X Q(X), Q = I - X/2 + X^2/3 - X^3/4 through degree deg:
   // Z = I/(deg-1) - X/deg, then Z = I/k - X Z for k = deg-2 .. 1
-  const float za = deg == 4 ? 1.f / 3.f : deg == 3 ? 0.5f : 1.f;
-  const float zb = deg == 4 ? 0.25f : deg == 3 ? 1.f / 3.f : 0.5f;
-#pragma unroll
-  for (int q = 0; q < 6; ++q) Z[q] = -zb * X[q] + (q < 3 ? za : 0.f);
-  if (deg == 4) {
-    sym_mul(X, Z, W);
-#pragma unroll
-    for (int q = 0; q < 6; ++q) Z[q] = -W[q] + (q < 3 ? 0.5f : 0.f);
-  }
-  if (deg >= 3) {
-    sym_mul(X, Z, W);
-#pragma unroll
-    for (int q = 0; q < 6; ++q) Z[q] = -W[q] + (q < 3 ? 1.f : 0.f);
-  }
-  float L[6];
-  sym_mul(X, Z, L);
-#pragma unroll
-  for (int q = 0; q < 6; ++q) L[q] *= 0.5f;
-  const float tr = L[0] + L[1] + L[2];
-  const float h[6] = {L[0] - tr * (1.f / 3.f), L[1] - tr * (1.f / 3.f), L[2] - tr * (1.f / 3.f), L[3], L[4], L[5]};
-  const float nrm = sqrtf(h[0] * h[0] + h[1] * h[1] + h[2] * h[2] + 2.f * (h[3] * h[3] + h[4] * h[4] + h[5] * h[5]));
-  float Ln[6] = {L[0], L[1], L[2], L[3], L[4], L[5]};
-  float Y[6];
-  bool moved = false;
-  if (tr >= 0.f) {  // tension: the tip
-#pragma unroll
-    for (int q = 0; q < 6; ++q) {
-      Ln[q] = 0.f;
-      Y[q] = -L[q];
-    }
-    moved = true;
-  } else {
-    const float dg = nrm + dpc * tr;
-    if (dg > 0.f && nrm > 0.f) {
-      const float k = dg / nrm;
-#pragma unroll
-      for (int q = 0; q < 6; ++q) {
-        Y[q] = -k * h[q];
-        Ln[q] = L[q] + Y[q];
-      }
-      moved = true;
-    }
-  }
-  if (moved) {
-    // exp(Y) = I + Y P(Y), P = I + Y/2 + Y^2/6 + Y^3/24 through degree deg:
+  const Sym N = scale(-1.f, X);
+  Sym Z = add_diag(deg == 4 ? 1.f / 3.f : deg == 3 ? 0.5f : 1.f, scale(deg == 4 ? 0.25f : deg == 3 ? 1.f / 3.f : 0.5f, N));
+  if (deg == 4) Z = sym_mul(Z, N, 0.5f);
+  if (deg >= 3) Z = sym_mul(Z, N, 1.f);
+  const Sym L = sym_mul(Z, scale(0.5f, X), 0.f);
+  const float tr = L.d.x + L.d.y + L.c;
+  // the tip (tension): eps moves by all of L; else along dev L by the factor
+  // k = dgamma / |dev L| = 1 + dpc tr / |dev L|, where it is positive
+  const bool tip = tr >= 0.f;
+  const Sym h = add_diag(tip ? 0.f : tr * (-1.f / 3.f), L);
+  const f2 q = fma2(h.d, h.d, mul2(dup(2.f), mul2(h.o, h.o)));
+  const float n2 = q.x + q.y + fmaf(h.c, h.c, 2.f * (h.e * h.e));
+  const float k = tip ? 1.f : fmaf(dpc * tr, Num<float>::rsqrt_(n2), 1.f);
+  Sym Ln = L;
+  if (tip || (n2 > 0.f && k > 0.f)) {
+    const Sym Y = scale(-k, h);
+    Ln = {add2(L.d, Y.d), add2(L.o, Y.o), L.c + Y.c, L.e + Y.e};
+    // exp(Y) - I = Y P(Y), P = I + Y/2 + Y^2/6 + Y^3/24 through degree deg:
     // Z = I/(deg-1)! + Y/deg!, then Z = I/k! + Y Z for k = deg-2 .. 1
-    const float ea = deg == 4 ? 1.f / 6.f : deg == 3 ? 0.5f : 1.f;
-    const float eb = deg == 4 ? 1.f / 24.f : deg == 3 ? 1.f / 6.f : 0.5f;
-#pragma unroll
-    for (int q = 0; q < 6; ++q) Z[q] = Y[q] * eb + (q < 3 ? ea : 0.f);
-    if (deg == 4) {
-      sym_mul(Y, Z, W);
-#pragma unroll
-      for (int q = 0; q < 6; ++q) Z[q] = W[q] + (q < 3 ? 0.5f : 0.f);
-    }
-    if (deg >= 3) {
-      sym_mul(Y, Z, W);
-#pragma unroll
-      for (int q = 0; q < 6; ++q) Z[q] = W[q] + (q < 3 ? 1.f : 0.f);
-    }
-    float Ex[6];
-    sym_mul(Y, Z, Ex);
-    Ex[0] += 1.f;
-    Ex[1] += 1.f;
-    Ex[2] += 1.f;
-    const float Em[9] = {Ex[0], Ex[3], Ex[4], Ex[3], Ex[1], Ex[5], Ex[4], Ex[5], Ex[2]};
-    float Fn[9];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int j = 0; j < 3; ++j)
-        CK_M(Fn, i, j) = CK_M(Em, i, 0) * CK_M(F, 0, j) + CK_M(Em, i, 1) * CK_M(F, 1, j) + CK_M(Em, i, 2) * CK_M(F, 2, j);
-#pragma unroll
-    for (int q = 0; q < 9; ++q) F[q] = Fn[q];
+    Sym P = add_diag(deg == 4 ? 1.f / 6.f : deg == 3 ? 0.5f : 1.f,
+                     scale(deg == 4 ? 1.f / 24.f : deg == 3 ? 1.f / 6.f : 0.5f, Y));
+    if (deg == 4) P = sym_mul(P, Y, 0.5f);
+    if (deg >= 3) P = sym_mul(P, Y, 1.f);
+    F = mul_add(sym_m3(sym_mul(P, Y, 0.f)), F, F);
   }
-  const float trn = Ln[0] + Ln[1] + Ln[2];
-  const float m2 = 2.f * mu, vol = lam * trn;
-  tau[0] = m2 * Ln[0] + vol;
-  tau[4] = m2 * Ln[1] + vol;
-  tau[8] = m2 * Ln[2] + vol;
-  tau[1] = tau[3] = m2 * Ln[3];
-  tau[2] = tau[6] = m2 * Ln[4];
-  tau[5] = tau[7] = m2 * Ln[5];
+  const float m2 = 2.f * mu * ts, vol = lam * (Ln.d.x + Ln.d.y + Ln.c) * ts;
+  tau = add_diag(vol, scale(m2, Ln));
 }
 
 // J-based fluid (the equation of state of the dam-break scenes): J = det F,

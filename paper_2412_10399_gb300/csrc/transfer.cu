@@ -17,6 +17,7 @@
 
 #include "common.cuh"
 #include "launch.h"
+#include "pack.cuh"
 #include "scan.cuh"
 #include "svd3.cuh"
 
@@ -31,6 +32,10 @@ constexpr float kInv2Pi = 0.15915494309189535f;
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
@@ -50,34 +55,38 @@ __device__ __forceinline__ void cp_async_wait() {
 // the transfer kernels (one copy per CTA).
 constexpr int kSmemMats = 8;
 
-// sin(2 pi f) for f in [0, 1): reduce to t = f - rint(f) in [-1/2, 1/2], fold
-// |t| > 1/4 with sin(2 pi t) = sin(2 pi (sign(t)/2 - t)) (both steps exact in
-// float), then the Taylor series of sin x at x = 2 pi t, |x| <= pi/2, through
-// x^11: coefficients (-1)^k (2 pi)^(2k+1) / (2k+1)!, truncation error below
-// (pi/2)^13 / 13! = 1.5e-8, about 1.6e-7 after float rounding.
-__device__ __forceinline__ float sin_2pi(float f) {
-  float t = f - rintf(f);
+// The reduction of sin(2 pi f) and cos(2 pi f), f in [0, 1): t = f - rint(f) in
+// [-1/2, 1/2], then |t| > 1/4 folds by t -> sign(t)/2 - t (both steps exact in
+// float), which keeps the sine and flips the cosine's sign.
+__device__ __forceinline__ float fold_2pi(float t) {
   const float h = copysignf(0.5f, t) - t;
-  t = fabsf(t) > 0.25f ? h : t;
-  const float t2 = t * t;
-  float p = -15.094642576822984f;
-  p = fmaf(p, t2, 42.058693944897634f);
-  p = fmaf(p, t2, -76.70585975306136f);
-  p = fmaf(p, t2, 81.60524927607504f);
-  p = fmaf(p, t2, -41.341702240399755f);
-  p = fmaf(p, t2, 6.283185307179586f);
+  return fabsf(t) > 0.25f ? h : t;
+}
+
+// sin(2 pi f) per axis, f in [0, 1): the Taylor series of sin x at x = 2 pi t,
+// |x| <= pi/2, through x^11: coefficients (-1)^k (2 pi)^(2k+1) / (2k+1)!,
+// truncation error below (pi/2)^13 / 13! = 1.5e-8, about 1.6e-7 after float
+// rounding.
+__device__ __forceinline__ V3 sin_2pi(const V3& f) {
+  V3 t = f - V3{pk(rintf(f.p.x), rintf(f.p.y)), rintf(f.z)};
+  t = {pk(fold_2pi(t.p.x), fold_2pi(t.p.y)), fold_2pi(t.z)};
+  const V3 t2 = t * t;
+  V3 p = v3(-15.094642576822984f);
+  p = fma3(p, t2, v3(42.058693944897634f));
+  p = fma3(p, t2, v3(-76.70585975306136f));
+  p = fma3(p, t2, v3(81.60524927607504f));
+  p = fma3(p, t2, v3(-41.341702240399755f));
+  p = fma3(p, t2, v3(6.283185307179586f));
   return t * p;
 }
 
-// cos(2 pi f) for f in [0, 1): the reduction of sin_2pi, where the fold
-// t -> sign(t)/2 - t flips the cosine's sign, then the Taylor series of cos x
-// at x = 2 pi t, |x| <= pi/2, through x^12: coefficients
-// (-1)^k (2 pi)^(2k) / (2k)!, truncation error below (pi/2)^14 / 14! = 6.4e-9.
+// cos(2 pi f) for f in [0, 1): the Taylor series of cos x at x = 2 pi t,
+// |x| <= pi/2, through x^12: coefficients (-1)^k (2 pi)^(2k) / (2k)!,
+// truncation error below (pi/2)^14 / 14! = 6.4e-9.
 __device__ __forceinline__ float cos_2pi(float f) {
   float t = f - rintf(f);
-  const float h = copysignf(0.5f, t) - t;
   const bool fold = fabsf(t) > 0.25f;
-  t = fold ? h : t;
+  t = fold_2pi(t);
   const float t2 = t * t;
   float p = 7.903536371318465f;
   p = fmaf(p, t2, -26.426256783374388f);
@@ -87,6 +96,20 @@ __device__ __forceinline__ float cos_2pi(float f) {
   p = fmaf(p, t2, -19.739208802178716f);
   p = fmaf(p, t2, 1.0f);
   return fold ? -p : p;
+}
+// per axis: x and y packed, by the same steps
+__device__ __forceinline__ V3 cos_2pi(const V3& f) {
+  const f2 t = add2(f.p, pk(-rintf(f.p.x), -rintf(f.p.y)));
+  const bool fx = fabsf(t.x) > 0.25f, fy = fabsf(t.y) > 0.25f;
+  const f2 u = pk(fold_2pi(t.x), fold_2pi(t.y)), t2 = mul2(u, u);
+  f2 p = dup(7.903536371318465f);
+  p = fma2(p, t2, dup(-26.426256783374388f));
+  p = fma2(p, t2, dup(60.24464137187664f));
+  p = fma2(p, t2, dup(-85.45681720669371f));
+  p = fma2(p, t2, dup(64.93939402266828f));
+  p = fma2(p, t2, dup(-19.739208802178716f));
+  p = fma2(p, t2, dup(1.0f));
+  return {pk(fx ? -p.x : p.x, fy ? -p.y : p.y), cos_2pi(f.z)};
 }
 
 // 1/x for a normal float x: the hardware approximation refined by one
@@ -100,12 +123,20 @@ __device__ __forceinline__ float rcp_nr(float x) {
   const float e = fmaf(-x, y, 1.0f);
   return fmaf(y, e, y);
 }
+__device__ __forceinline__ V3 rcp_nr(const V3& x) {
+  V3 y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y.p.x) : "f"(x.p.x));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y.p.y) : "f"(x.p.y));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y.z) : "f"(x.z));
+  return fma3(y, fma3(neg3(x), y, v3(1.0f)), y);
+}
 
 template <int KIND>
 struct Geo;
 template <>
 struct Geo<0> {
   static constexpr int NG = 2;
+  static constexpr int N = 2;  // nodes per axis of a stencil
   static constexpr int E0 = 5, E1 = 6;
   static constexpr int N0 = 125;
   static constexpr int NS = 341;
@@ -114,6 +145,7 @@ struct Geo<0> {
 template <>
 struct Geo<1> {
   static constexpr int NG = 1;
+  static constexpr int N = 3;
   static constexpr int E0 = 6, E1 = 6;
   static constexpr int N0 = 216;
   static constexpr int NS = 216;
@@ -162,8 +194,9 @@ __device__ __forceinline__ void load_block_slots(const StepView& v, const SceneD
 // ------------------------------------------------------------------ stencils
 
 // Weights, node offsets (x_i - x_p in cells) and D^-1 (cells^-2) of one
-// particle.  CK: K1 weights on both grids from one sine per axis
-// (sin 2 pi f- = -sin 2 pi f+), D = Lambda + s s^T with the closed form
+// particle, per axis in a V3, computed from the fractions where they are used
+// (a kernel holds one grid's weights at a time).  CK: K1 weights on both grids from one sine per
+// axis (sin 2 pi f- = -sin 2 pi f+), D = Lambda + s s^T with the closed form
 // Lambda_a = (m2(f+) + m2(f-))/2 - s_a^2, s_a = sin(2 pi f+_a)/(2 pi),
 // inverted by Sherman-Morrison.  Quadratic: B-spline weights, D^-1 = 4 I.
 template <int KIND>
@@ -171,357 +204,266 @@ struct Sten;
 
 template <>
 struct Sten<0> {
-  int r[2][3];        // base node of each slot relative to the block origin
-  float w[2][3][2];   // per slot, axis, node
-  float d[2][3][2];
-  float li[3], y[3], den;  // D^-1 = diag(li) - den y y^T (cells^-2)
-  float k[2][3][2];        // PIC transfer: K1'(d) per slot, axis, node (set_grad)
+  int r[2][3];     // base node of each grid relative to the block origin
+  V3 f[2];         // fractions on G- and G+
+  V3 sg;           // sin(2 pi f+) / (2 pi)
+  V3 c;            // kernel-gradient transfers: cos(2 pi f+) (set_grad)
   __device__ __forceinline__ bool set(float ux, float uy, float uz, int ox, int oy, int oz) {
-    float u[3] = {ux, uy, uz};
-    int o[3] = {ox, oy, oz};
-    float s[3], lam[3];
+    const int o[3] = {ox, oy, oz};
     bool ok = true;
+    const V3 t = V3{pk(ux, uy), uz} + v3(0.25f);
+    const float fb[3] = {floorf(t.p.x), floorf(t.p.y), floorf(t.z)};
+    f[1] = t - V3{pk(fb[0], fb[1]), fb[2]};
+    const float fp[3] = {f[1].p.x, f[1].p.y, f[1].z};
+    float sh[3];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      Cell<0> c;
-      c.set(u[a]);
-      r[0][a] = c.bm - o[a];
-      r[1][a] = c.bp - o[a];
+    for (int a = 0; a < 3; ++a) {  // Cell<0>: b- = b+ or b+ - 1, f- = f+ -+ 1/2
+      const int bp = (int)fb[a];
+      const bool up = fp[a] >= 0.5f;
+      const int bm = up ? bp : bp - 1;
+      sh[a] = up ? -0.5f : 0.5f;
+      r[0][a] = bm - o[a];
+      r[1][a] = bp - o[a];
       ok = ok && (unsigned)r[0][a] <= 3u;  // then the G+ base, r[0][a] or r[0][a] + 1, is in [0, 4]
-      float sg = sin_2pi(c.fp) * kInv2Pi;
-      w[1][a][0] = 1.0f - c.fp + sg;
-      w[1][a][1] = c.fp - sg;
-      d[1][a][0] = -c.fp;
-      d[1][a][1] = 1.0f - c.fp;
-      w[0][a][0] = 1.0f - c.fm - sg;
-      w[0][a][1] = c.fm + sg;
-      d[0][a][0] = -c.fm;
-      d[0][a][1] = 1.0f - c.fm;
-      float m2p = c.fp * (1.0f - c.fp) - sg * (1.0f - 2.0f * c.fp);
-      float m2m = c.fm * (1.0f - c.fm) + sg * (1.0f - 2.0f * c.fm);
-      lam[a] = 0.5f * (m2p + m2m) - sg * sg;
-      s[a] = sg;
     }
-    // Lambda_a in [0.0826, 0.1586] and 1 + s^T Lambda^-1 s in [1, 1.3]
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      li[a] = rcp_nr(lam[a]);
-      y[a] = li[a] * s[a];
-    }
-    den = rcp_nr(1.0f + s[0] * y[0] + s[1] * y[1] + s[2] * y[2]);
+    f[0] = f[1] + V3{pk(sh[0], sh[1]), sh[2]};
+    sg = kInv2Pi * sin_2pi(f[1]);
     return ok;
   }
+  // K1 weights: 1 - f+ + s and f+ - s on G+, with -s on G-
+  __device__ __forceinline__ V3 w(int g, int n) const {
+    const V3 h = n == 0 ? v3(1.0f) - f[g] : f[g];
+    return (g == 1) == (n == 0) ? h + sg : h - sg;
+  }
+  __device__ __forceinline__ V3 d(int g, int n) const { return n == 0 ? neg3(f[g]) : v3(1.0f) - f[g]; }
   // K1'(x) = sgn(x) (cos(2 pi |x|) - 1) at the node offsets d = -f, 1 - f:
   // with c = cos(2 pi f+), 1 - c and c - 1 on G+; cos(2 pi f-) = -c, so
   // 1 + c and -1 - c on G-.  Each pair sums to 0 (the weights sum to 1).
-  __device__ __forceinline__ void set_grad() {
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const float c = cos_2pi(-d[1][a][0]);
-      k[1][a][0] = 1.0f - c;
-      k[1][a][1] = c - 1.0f;
-      k[0][a][0] = 1.0f + c;
-      k[0][a][1] = -1.0f - c;
-    }
+  __device__ __forceinline__ void set_grad() { c = cos_2pi(f[1]); }
+  __device__ __forceinline__ V3 k(int g, int n) const {
+    const V3 h = g == 1 ? v3(1.0f) - c : v3(1.0f) + c;
+    return n == 0 ? h : neg3(h);
+  }
+  // D^-1 = diag(li) - den y y^T (cells^-2)
+  __device__ __forceinline__ void dinv(V3& li, V3& y, float& den) const {
+    const V3 one = v3(1.0f);
+    const V3 m2p = fma3(f[1], one - f[1], neg3(sg * fma3(-2.0f, f[1], one)));
+    const V3 m2m = fma3(f[0], one - f[0], sg * fma3(-2.0f, f[0], one));
+    const V3 lam = fma3(0.5f, m2p + m2m, neg3(sg * sg));
+    // Lambda_a in [0.0826, 0.1586] and 1 + s^T Lambda^-1 s in [1, 1.3]
+    li = rcp_nr(lam);
+    y = li * sg;
+    den = rcp_nr(1.0f + sg.p.x * y.p.x + sg.p.y * y.p.y + sg.z * y.z);
   }
 };
 
 template <>
 struct Sten<1> {
-  int r[3];
-  float w[3][3];
-  float d[3][3];
-  float k[3][3];  // PIC transfer: N'(d) per axis, node (set_grad)
+  int r[1][3];
+  V3 f[1];  // in [0.5, 1.5)
   __device__ __forceinline__ bool set(float ux, float uy, float uz, int ox, int oy, int oz) {
-    float u[3] = {ux, uy, uz};
-    int o[3] = {ox, oy, oz};
+    const float u[3] = {ux, uy, uz};
+    const int o[3] = {ox, oy, oz};
+    float fa[3];
     bool ok = true;
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       Cell<1> c;
       c.set(u[a]);
-      r[a] = c.b - o[a];
-      ok = ok && (unsigned)r[a] <= 3u;
-      float f = c.f;
-      w[a][0] = 0.5f * (1.5f - f) * (1.5f - f);
-      w[a][1] = 0.75f - (f - 1.0f) * (f - 1.0f);
-      w[a][2] = 0.5f * (f - 0.5f) * (f - 0.5f);
-      d[a][0] = -f;
-      d[a][1] = 1.0f - f;
-      d[a][2] = 2.0f - f;
+      r[0][a] = c.b - o[a];
+      ok = ok && (unsigned)r[0][a] <= 3u;
+      fa[a] = c.f;
     }
+    f[0] = {pk(fa[0], fa[1]), fa[2]};
     return ok;
   }
-  // N'(x) of the quadratic B-spline at d = -f, 1 - f, 2 - f (f in [1/2, 3/2)):
-  // 3/2 - f, 2 (f - 1), 1/2 - f.
-  __device__ __forceinline__ void set_grad() {
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const float f = -d[a][0];
-      k[a][0] = 1.5f - f;
-      k[a][1] = 2.0f * (f - 1.0f);
-      k[a][2] = 0.5f - f;
-    }
+  __device__ __forceinline__ V3 w(int, int n) const {
+    const V3 p = n == 0 ? v3(1.5f) - f[0] : n == 1 ? v3(1.0f) - f[0] : f[0] - v3(0.5f);
+    return n == 1 ? v3(0.75f) - p * p : 0.5f * (p * p);
+  }
+  __device__ __forceinline__ V3 d(int, int n) const { return n == 0 ? neg3(f[0]) : v3((float)n) - f[0]; }
+  __device__ __forceinline__ void set_grad() {}
+  // N'(x) of the quadratic B-spline at d = -f, 1 - f, 2 - f: 3/2 - f, 2 (f - 1), 1/2 - f
+  __device__ __forceinline__ V3 k(int, int n) const {
+    return n == 0 ? v3(1.5f) - f[0] : n == 1 ? 2.0f * (f[0] - v3(1.0f)) : v3(0.5f) - f[0];
   }
 };
 
+// Staged nodes of grid g: row pitch, first index, and a stencil's first node.
+template <int KIND>
+__device__ __forceinline__ constexpr int pitch(int g) {
+  return KIND == 0 && g == 0 ? 5 : 6;
+}
+template <int KIND>
+__device__ __forceinline__ int first_node(const Sten<KIND>& st, int g) {
+  const int E = pitch<KIND>(g);
+  return (g == 0 ? 0 : 125) + (st.r[g][2] * E + st.r[g][1]) * E + st.r[g][0];
+}
+
 // Visit every (node, weight, offset) of a stencil: fn(staged_index, w, dx, dy, dz).
-template <typename Fn>
-__device__ __forceinline__ void for_nodes(const Sten<0>& st, Fn&& fn) {
+template <int KIND, typename Fn>
+__device__ __forceinline__ void for_nodes(const Sten<KIND>& st, Fn&& fn) {
+  constexpr int N = Geo<KIND>::N;
 #pragma unroll
-  for (int slot = 0; slot < 2; ++slot) {
-    const int E = slot == 0 ? 5 : 6;
-    const int base = slot == 0 ? 0 : 125;
+  for (int g = 0; g < Geo<KIND>::NG; ++g) {
+    const int E = pitch<KIND>(g), base = first_node<KIND>(st, g);
 #pragma unroll
-    for (int sz = 0; sz < 2; ++sz)
+    for (int sz = 0; sz < N; ++sz)
 #pragma unroll
-      for (int sy = 0; sy < 2; ++sy) {
-        float wyz = st.w[slot][1][sy] * st.w[slot][2][sz];
-        int row = base + ((st.r[slot][2] + sz) * E + (st.r[slot][1] + sy)) * E + st.r[slot][0];
+      for (int sy = 0; sy < N; ++sy) {
+        const float wyz = st.w(g, sy).p.y * st.w(g, sz).z;
 #pragma unroll
-        for (int sx = 0; sx < 2; ++sx)
-          fn(row + sx, st.w[slot][0][sx] * wyz, st.d[slot][0][sx], st.d[slot][1][sy], st.d[slot][2][sz]);
+        for (int sx = 0; sx < N; ++sx)
+          fn(base + (sz * E + sy) * E + sx, st.w(g, sx).p.x * wyz, st.d(g, sx).p.x, st.d(g, sy).p.y, st.d(g, sz).z);
       }
   }
 }
 
-template <typename Fn>
-__device__ __forceinline__ void for_nodes(const Sten<1>& st, Fn&& fn) {
-#pragma unroll
-  for (int sz = 0; sz < 3; ++sz)
-#pragma unroll
-    for (int sy = 0; sy < 3; ++sy) {
-      float wyz = st.w[1][sy] * st.w[2][sz];
-      int row = ((st.r[2] + sz) * 6 + (st.r[1] + sy)) * 6 + st.r[0];
-#pragma unroll
-      for (int sx = 0; sx < 3; ++sx) fn(row + sx, st.w[0][sx] * wyz, st.d[0][sx], st.d[1][sy], st.d[2][sz]);
-    }
+// Staged grid velocities: (x, y) and z apart, so that a node is an 8- and a
+// 4-byte shared load (three wavefronts) instead of a 16-byte one (four).
+template <int NS>
+struct NodeVel {
+  float2 xy[NS];
+  float z[NS];
+};
+template <int NS>
+__device__ __forceinline__ void stage_node(NodeVel<NS>& s, int j, const float4* g) {
+  cp_async8(&s.xy[j], g);
+  cp_async4(&s.z[j], reinterpret_cast<const float*>(g) + 2);
 }
-
-// Kernel-gradient transfers: visit every (node, weight, kernel-derivative
-// products, offsets) of a stencil, fn(staged_index, w, gx, gy, gz, dx, dy, dz)
-// with w = Kx Ky Kz and g = (K'x Ky Kz, Kx K'y Kz, Kx Ky K'z), so that
-// grad w = -g / dx (the gradient with respect to the particle position), and
-// d the node offset in cells.  Needs set_grad().
-template <typename Fn>
-__device__ __forceinline__ void for_nodes_grad(const Sten<0>& st, Fn&& fn) {
-#pragma unroll
-  for (int slot = 0; slot < 2; ++slot) {
-    const int E = slot == 0 ? 5 : 6;
-    const int base = slot == 0 ? 0 : 125;
-#pragma unroll
-    for (int sz = 0; sz < 2; ++sz)
-#pragma unroll
-      for (int sy = 0; sy < 2; ++sy) {
-        const float wyz = st.w[slot][1][sy] * st.w[slot][2][sz];
-        const float kyz = st.k[slot][1][sy] * st.w[slot][2][sz];
-        const float ykz = st.w[slot][1][sy] * st.k[slot][2][sz];
-        const int row = base + ((st.r[slot][2] + sz) * E + (st.r[slot][1] + sy)) * E + st.r[slot][0];
-#pragma unroll
-        for (int sx = 0; sx < 2; ++sx) {
-          const float wx = st.w[slot][0][sx];
-          fn(row + sx, wx * wyz, st.k[slot][0][sx] * wyz, wx * kyz, wx * ykz, st.d[slot][0][sx], st.d[slot][1][sy],
-             st.d[slot][2][sz]);
-        }
-      }
-  }
-}
-
-template <typename Fn>
-__device__ __forceinline__ void for_nodes_grad(const Sten<1>& st, Fn&& fn) {
-#pragma unroll
-  for (int sz = 0; sz < 3; ++sz)
-#pragma unroll
-    for (int sy = 0; sy < 3; ++sy) {
-      const float wyz = st.w[1][sy] * st.w[2][sz];
-      const float kyz = st.k[1][sy] * st.w[2][sz];
-      const float ykz = st.w[1][sy] * st.k[2][sz];
-      const int row = ((st.r[2] + sz) * 6 + (st.r[1] + sy)) * 6 + st.r[0];
-#pragma unroll
-      for (int sx = 0; sx < 3; ++sx) {
-        const float wx = st.w[0][sx];
-        fn(row + sx, wx * wyz, st.k[0][sx] * wyz, wx * kyz, wx * ykz, st.d[0][sx], st.d[1][sy], st.d[2][sz]);
-      }
-    }
-}
+struct Nodes {
+  const float2* xy;
+  const float* z;
+  __device__ __forceinline__ V3 operator[](int i) const { return {xy[i], z[i]}; }
+  __device__ __forceinline__ Nodes operator+(int i) const { return {xy + i, z + i}; }
+};
 
 // G2P gather as a tensor-product contraction (a node's weight is the product
 // of per-axis weights): over one grid's N^3 stencil, S = sum w v~ and the
 // first moments M_a = sum w v~ s_a (s_a in 0..N-1: the node's offset in the
 // stencil along axis a), reducing x, then y, then z.  With x_i - x_p =
-// (s - f) dx per axis, sum w v~ (x_i - x_p)_a / dx = M_a - f_a S.  sv holds
-// the staged nodes with row pitch E; base is the stencil's first node.
-template <int N, int E>
-__device__ __forceinline__ void gather_moments(const float4* sv, int base, const float* wx, const float* wy,
-                                               const float* wz, float* S, float* Mx, float* My, float* Mz) {
+// (s - f) dx per axis, sum w v~ (x_i - x_p)_a / dx = M_a - f_a S.  FIRST: M
+// starts here (else it adds to the grid before).  wz carries the factor 1/2
+// that averages the two CK grids: every sum is linear in the z weights, and
+// scaling by a power of two is exact.
+template <int KIND, bool FIRST>
+__device__ __forceinline__ void gather_moments(const Nodes& sv, const Sten<KIND>& st, int g, V3& S, V3* M) {
+  constexpr int N = Geo<KIND>::N;
+  const int E = pitch<KIND>(g), base = first_node<KIND>(st, g);
 #pragma unroll
   for (int sz = 0; sz < N; ++sz) {
-    float Ps[3], Px[3], Py[3];
+    V3 Ps, Px, Py;
 #pragma unroll
     for (int sy = 0; sy < N; ++sy) {
-      float Rs[3], Rx[3];
-      const int row = base + (sz * E + sy) * E;
-#pragma unroll
-      for (int sx = N - 1; sx >= 0; --sx) {
-        const float4 a = sv[row + sx];
-        const float t[3] = {wx[sx] * a.x, wx[sx] * a.y, wx[sx] * a.z};
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          if (sx == N - 1) {
-            Rs[c] = t[c];
-            Rx[c] = (float)sx * t[c];
-          } else {
-            Rs[c] += t[c];
-            if (sx > 0) Rx[c] = fmaf((float)sx, t[c], Rx[c]);
-          }
-        }
+      const Nodes row = sv + base + (sz * E + sy) * E;
+      V3 Rs, Rx;
+      Rx = st.w(g, 1).p.x * row[1];
+      Rs = fma3(st.w(g, 0).p.x, row[0], Rx);
+      if constexpr (N == 3) {
+        const V3 t = st.w(g, 2).p.x * row[2];
+        Rs = Rs + t;
+        Rx = fma3(2.0f, t, Rx);
       }
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const float u = wy[sy] * Rs[c];
-        if (sy == 0) {
-          Ps[c] = u;
-          Px[c] = wy[sy] * Rx[c];
-        } else {
-          Ps[c] += u;
-          Px[c] = fmaf(wy[sy], Rx[c], Px[c]);
-          Py[c] = sy == 1 ? u : fmaf((float)sy, u, Py[c]);
-        }
-      }
-    }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const float u = wz[sz] * Ps[c];
-      if (sz == 0) {
-        S[c] = u;
-        Mx[c] = wz[sz] * Px[c];
-        My[c] = wz[sz] * Py[c];
+      const float wy = st.w(g, sy).p.y;
+      if (sy == 0) {
+        Ps = wy * Rs;
+        Px = wy * Rx;
       } else {
-        S[c] += u;
-        Mx[c] = fmaf(wz[sz], Px[c], Mx[c]);
-        My[c] = fmaf(wz[sz], Py[c], My[c]);
-        Mz[c] = sz == 1 ? u : fmaf((float)sz, u, Mz[c]);
+        const V3 u = wy * Rs;
+        Ps = Ps + u;
+        Px = fma3(wy, Rx, Px);
+        Py = sy == 1 ? u : fma3(2.0f, u, Py);
       }
+    }
+    const float wz = st.w(g, sz).z * (KIND == 0 ? 0.5f : 1.0f);
+    if (sz == 0) {
+      S = wz * Ps;
+      M[0] = FIRST ? wz * Px : fma3(wz, Px, M[0]);
+      M[1] = FIRST ? wz * Py : fma3(wz, Py, M[1]);
+    } else {
+      S = fma3(wz, Ps, S);
+      M[0] = fma3(wz, Px, M[0]);
+      M[1] = fma3(wz, Py, M[1]);
+      M[2] = FIRST && sz == 1 ? wz * Ps : fma3((float)sz * wz, Ps, M[2]);
     }
   }
 }
 
-// v = h sum w v~ and Bh = h sum w v~ (x_i - x_p)^T / dx (row c, column a) over
-// the particle's stencil; h = 1/2 averages the two CK grids.  Every sum is
-// linear in the z weights, so h is applied to those (four products) instead
-// of to the twelve results; scaling by a power of two is exact, so the
-// results are the same bits.
-__device__ __forceinline__ void g2p_gather(const Sten<0>& st, const float4* sv, float* vel, float* Bh) {
-  float S[2][3], M[2][3][3];
-  const float hz0[2] = {0.5f * st.w[0][2][0], 0.5f * st.w[0][2][1]};
-  const float hz1[2] = {0.5f * st.w[1][2][0], 0.5f * st.w[1][2][1]};
-  gather_moments<2, 5>(sv, (st.r[0][2] * 5 + st.r[0][1]) * 5 + st.r[0][0], st.w[0][0], st.w[0][1], hz0, S[0],
-                       M[0][0], M[0][1], M[0][2]);
-  gather_moments<2, 6>(sv, 125 + (st.r[1][2] * 6 + st.r[1][1]) * 6 + st.r[1][0], st.w[1][0], st.w[1][1], hz1,
-                       S[1], M[1][0], M[1][1], M[1][2]);
+// v = h sum w v~ and Bh = h sum w v~ (x_i - x_p)^T / dx (column a: axis a) over
+// the particle's stencil; h = 1/2 averages the two CK grids.
+template <int KIND>
+__device__ __forceinline__ void g2p_gather(const Sten<KIND>& st, const Nodes& sv, V3& vel, M3& Bh) {
+  V3 S[Geo<KIND>::NG];
+  gather_moments<KIND, true>(sv, st, 0, S[0], Bh.c);
+  if constexpr (KIND == 0) gather_moments<KIND, false>(sv, st, 1, S[1], Bh.c);
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    vel[c] = S[0][c] + S[1][c];
-#pragma unroll
-    for (int a = 0; a < 3; ++a)  // f_a = -d[g][a][0]
-      Bh[c * 3 + a] = fmaf(st.d[0][a][0], S[0][c], M[0][a][c]) + fmaf(st.d[1][a][0], S[1][c], M[1][a][c]);
+  for (int a = 0; a < 3; ++a) {  // f_a = -d[g][0]
+    if constexpr (KIND == 0) Bh.c[a] = fma3(at3(st.d(1, 0), a), S[1], Bh.c[a]);
+    Bh.c[a] = fma3(at3(st.d(0, 0), a), S[0], Bh.c[a]);
   }
+  vel = S[0];
+  if constexpr (KIND == 0) vel = vel + S[1];
 }
 
-__device__ __forceinline__ void g2p_gather(const Sten<1>& st, const float4* sv, float* vel, float* Bh) {
-  float S[3], M[3][3];
-  gather_moments<3, 6>(sv, (st.r[2] * 6 + st.r[1]) * 6 + st.r[0], st.w[0], st.w[1], st.w[2], S, M[0], M[1], M[2]);
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    vel[c] = S[c];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) Bh[c * 3 + a] = fmaf(st.d[a][0], S[c], M[a][c]);
-  }
-}
-
-// PIC transfer: S = sum w v~ and the derivative sums G_a = sum g_a v~ over one
-// grid's N^3 stencil (g as in for_nodes_grad), by the same x, y, z reduction
-// as gather_moments with the kernel derivative in place of the offset.
-template <int N, int E>
-__device__ __forceinline__ void gather_grad(const float4* sv, int base, const float* wx, const float* wy,
-                                            const float* wz, const float* kx, const float* ky, const float* kz,
-                                            float* S, float* Gx, float* Gy, float* Gz) {
+// Kernel-gradient transfers: S = sum w v~ and the derivative sums G_a = sum
+// g_a v~ over one grid's N^3 stencil, g = (K'x Ky Kz, Kx K'y Kz, Kx Ky K'z)
+// (so that grad w = -g / dx with respect to the particle position), by the
+// same x, y, z reduction with the kernel derivative in place of the offset.
+template <int KIND, bool FIRST>
+__device__ __forceinline__ void gather_grad(const Nodes& sv, const Sten<KIND>& st, int g, V3& S, V3* G) {
+  constexpr int N = Geo<KIND>::N;
+  const int E = pitch<KIND>(g), base = first_node<KIND>(st, g);
+  constexpr float h = KIND == 0 ? 0.5f : 1.0f;
 #pragma unroll
   for (int sz = 0; sz < N; ++sz) {
-    float Ps[3], Px[3], Py[3];
+    V3 Ps, Px, Py;
 #pragma unroll
     for (int sy = 0; sy < N; ++sy) {
-      float Rs[3], Rx[3];
-      const int row = base + (sz * E + sy) * E;
+      const Nodes row = sv + base + (sz * E + sy) * E;
+      V3 Rs, Rx;
 #pragma unroll
       for (int sx = 0; sx < N; ++sx) {
-        const float4 a = sv[row + sx];
-        const float t[3] = {a.x, a.y, a.z};
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          Rs[c] = sx == 0 ? wx[sx] * t[c] : fmaf(wx[sx], t[c], Rs[c]);
-          Rx[c] = sx == 0 ? kx[sx] * t[c] : fmaf(kx[sx], t[c], Rx[c]);
-        }
+        const V3 a = row[sx];
+        Rs = sx == 0 ? st.w(g, sx).p.x * a : fma3(st.w(g, sx).p.x, a, Rs);
+        Rx = sx == 0 ? st.k(g, sx).p.x * a : fma3(st.k(g, sx).p.x, a, Rx);
       }
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        Ps[c] = sy == 0 ? wy[sy] * Rs[c] : fmaf(wy[sy], Rs[c], Ps[c]);
-        Px[c] = sy == 0 ? wy[sy] * Rx[c] : fmaf(wy[sy], Rx[c], Px[c]);
-        Py[c] = sy == 0 ? ky[sy] * Rs[c] : fmaf(ky[sy], Rs[c], Py[c]);
-      }
+      const float wy = st.w(g, sy).p.y, ky = st.k(g, sy).p.y;
+      Ps = sy == 0 ? wy * Rs : fma3(wy, Rs, Ps);
+      Px = sy == 0 ? wy * Rx : fma3(wy, Rx, Px);
+      Py = sy == 0 ? ky * Rs : fma3(ky, Rs, Py);
     }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      S[c] = sz == 0 ? wz[sz] * Ps[c] : fmaf(wz[sz], Ps[c], S[c]);
-      Gx[c] = sz == 0 ? wz[sz] * Px[c] : fmaf(wz[sz], Px[c], Gx[c]);
-      Gy[c] = sz == 0 ? wz[sz] * Py[c] : fmaf(wz[sz], Py[c], Gy[c]);
-      Gz[c] = sz == 0 ? kz[sz] * Ps[c] : fmaf(kz[sz], Ps[c], Gz[c]);
-    }
+    const float wz = h * st.w(g, sz).z, kz = h * st.k(g, sz).z;
+    const bool first = FIRST && sz == 0;
+    S = first ? wz * Ps : fma3(wz, Ps, S);
+    G[0] = first ? wz * Px : fma3(wz, Px, G[0]);
+    G[1] = first ? wz * Py : fma3(wz, Py, G[1]);
+    G[2] = first ? kz * Ps : fma3(kz, Ps, G[2]);
   }
 }
 
-// PIC transfer: v = h sum w v~ and Gr = h sum v~ g^T (row c, column a), so
-// that grad v = -Gr / dx; h = 1/2 averages the two CK grids.  Needs set_grad().
-__device__ __forceinline__ void g2p_gather_grad(const Sten<0>& st, const float4* sv, float* vel, float* Gr) {
-  float S[2][3], D[2][3][3];
-  gather_grad<2, 5>(sv, (st.r[0][2] * 5 + st.r[0][1]) * 5 + st.r[0][0], st.w[0][0], st.w[0][1], st.w[0][2],
-                    st.k[0][0], st.k[0][1], st.k[0][2], S[0], D[0][0], D[0][1], D[0][2]);
-  gather_grad<2, 6>(sv, 125 + (st.r[1][2] * 6 + st.r[1][1]) * 6 + st.r[1][0], st.w[1][0], st.w[1][1], st.w[1][2],
-                    st.k[1][0], st.k[1][1], st.k[1][2], S[1], D[1][0], D[1][1], D[1][2]);
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    vel[c] = 0.5f * (S[0][c] + S[1][c]);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) Gr[c * 3 + a] = 0.5f * (D[0][a][c] + D[1][a][c]);
-  }
+// v = h sum w v~ and Gr = h sum v~ g^T (column a: axis a), so that grad v =
+// -Gr / dx; h = 1/2 averages the two CK grids.  Needs set_grad().
+template <int KIND>
+__device__ __forceinline__ void g2p_gather_grad(const Sten<KIND>& st, const Nodes& sv, V3& vel, M3& Gr) {
+  gather_grad<KIND, true>(sv, st, 0, vel, Gr.c);
+  if constexpr (KIND == 0) gather_grad<KIND, false>(sv, st, 1, vel, Gr.c);
 }
 
-__device__ __forceinline__ void g2p_gather_grad(const Sten<1>& st, const float4* sv, float* vel, float* Gr) {
-  float S[3], D[3][3];
-  gather_grad<3, 6>(sv, (st.r[2] * 6 + st.r[1]) * 6 + st.r[0], st.w[0], st.w[1], st.w[2], st.k[0], st.k[1],
-                    st.k[2], S, D[0], D[1], D[2]);
+// R = scale Q D^-1.  CK: D^-1 = diag(li) - den y y^T, so with t = Q y a column
+// costs one product and one fused update; quadratic: D^-1 = 4 I.
+__device__ __forceinline__ M3 mul_dinv(const Sten<0>& st, const M3& Q, float scale) {
+  V3 li, y;
+  float den;
+  st.dinv(li, y, den);
+  const V3 t = fma3(y.z, Q.c[2], fma3(y.p.y, Q.c[1], y.p.x * Q.c[0]));
+  const V3 ls = scale * li, ys = neg3((scale * den) * y);
+  M3 R;
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    vel[c] = S[c];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) Gr[c * 3 + a] = D[a][c];
-  }
+  for (int q = 0; q < 3; ++q) R.c[q] = fma3(at3(ys, q), t, at3(ls, q) * Q.c[q]);
+  return R;
 }
-
-// R = scale Q D^-1 for a row-major 3x3 Q.  CK: D^-1 = diag(li) - den y y^T,
-// so each row costs one dot product with y and three fused updates instead of
-// a full 3x3 product; quadratic: D^-1 = 4 I.
-__device__ __forceinline__ void mul_dinv(const Sten<0>& st, const float* Q, float scale, float* R) {
-#pragma unroll
-  for (int r = 0; r < 3; ++r) {
-    const float t = (Q[r * 3] * st.y[0] + Q[r * 3 + 1] * st.y[1] + Q[r * 3 + 2] * st.y[2]) * st.den;
-#pragma unroll
-    for (int q = 0; q < 3; ++q) R[r * 3 + q] = scale * (Q[r * 3 + q] * st.li[q] - t * st.y[q]);
-  }
-}
-__device__ __forceinline__ void mul_dinv(const Sten<1>&, const float* Q, float scale, float* R) {
-#pragma unroll
-  for (int q = 0; q < 9; ++q) R[q] = (4.0f * scale) * Q[q];
+__device__ __forceinline__ M3 mul_dinv(const Sten<1>&, const M3& Q, float scale) {
+  return {{(4.0f * scale) * Q.c[0], (4.0f * scale) * Q.c[1], (4.0f * scale) * Q.c[2]}};
 }
 
 __device__ __forceinline__ void decode_block(const SceneDev& s, uint32_t key, int& ox, int& oy, int& oz) {
@@ -596,14 +538,14 @@ struct P2GBound<1> {
 // and re-keying otherwise), so P2G reads a block's bounds without a pass over
 // its particles.
 template <int KIND>
-__device__ __forceinline__ void p2g_bounds(float inv_dx, float mass, float vx, float vy, float vz, const float* M,
-                                           float& bmass, float& bmom) {
-  const float r0 = fabsf(M[0]) + fabsf(M[1]) + fabsf(M[2]);
-  const float r1 = fabsf(M[3]) + fabsf(M[4]) + fabsf(M[5]);
-  const float r2 = fabsf(M[6]) + fabsf(M[7]) + fabsf(M[8]);
+__device__ __forceinline__ void p2g_bounds(float inv_dx, float mass, const V3& v, const M3& M, float& bmass,
+                                           float& bmom) {
+  const float r0 = fabsf(M.c[0].p.x) + fabsf(M.c[1].p.x) + fabsf(M.c[2].p.x);
+  const float r1 = fabsf(M.c[0].p.y) + fabsf(M.c[1].p.y) + fabsf(M.c[2].p.y);
+  const float r2 = fabsf(M.c[0].z) + fabsf(M.c[1].z) + fabsf(M.c[2].z);
   const float rm = fmaxf(r0, fmaxf(r1, r2));
   bmass = P2GBound<KIND>::wmax * mass;
-  bmom = bmass * fmaxf(fabsf(vx), fmaxf(fabsf(vy), fabsf(vz))) +
+  bmom = bmass * fmaxf(fabsf(v.p.x), fmaxf(fabsf(v.p.y), fabsf(v.z))) +
          P2GBound<KIND>::wd * P2GBound<KIND>::dinv * rm * inv_dx;
 }
 
@@ -615,200 +557,138 @@ __device__ __forceinline__ void p2g_bounds(float inv_dx, float mass, float vx, f
 // conversion off the XU pipe; smaller blocks convert with __float2int_rn.
 constexpr uint32_t kP2GFmaCount = 256;
 
+// Two rounded contributions w * val into their planes.  FMA: one packed
+// multiply-add with 1.5 * 2^23 rounds both halves; each is, in scalars,
+//   __float_as_int(fmaf(w, val, 12582912.0f)) - 0x4B400000;
 template <bool FMA>
-__device__ __forceinline__ int p2g_fixed(float w, float val) {
-  if constexpr (FMA)
-    return __float_as_int(fmaf(w, val, 12582912.0f)) - 0x4B400000;
-  else
-    return __float2int_rn(w * val);
-}
-
-template <int KIND, bool FMA = false>
-__device__ __forceinline__ void p2g_scatter(const SceneDev& s, const MatDev* mats, uint32_t* err, const P2GPart& q,
-                                            int ox, int oy, int oz, float Sm, float Sp, int (*sm)[Geo<KIND>::NS]) {
-  Sten<KIND> st;
-  if (!st.set(q.X.x * s.inv_dx, q.X.y * s.inv_dx, q.X.z * s.inv_dx, ox, oy, oz)) {
-    flag_error(err, CK_ERR_INTERNAL);
-    return;
+__device__ __forceinline__ void p2g_add2(int* a, int* b, f2 w, f2 val) {
+  if constexpr (FMA) {
+    const f2 f = fma2(w, val, dup(12582912.0f));
+    atomicAdd(a, __float_as_int(f.x) - 0x4B400000);
+    atomicAdd(b, __float_as_int(f.y) - 0x4B400000);
+  } else {
+    const f2 f = mul2(w, val);
+    atomicAdd(a, __float2int_rn(f.x));
+    atomicAdd(b, __float2int_rn(f.y));
   }
-  const float M[9] = {q.a.w, q.b.x, q.b.y, q.b.z, q.b.w, q.c.x, q.c.y, q.c.z, q.c.w};
-  // A^ = M D^-1 / dx so that A (x_i - x_p) = A^ (offset in cells), pre-scaled
-  float A[9];
-  mul_dinv(st, M, s.inv_dx * Sp, A);
-  const float mass = mats[__float_as_uint(q.X.w)].mass;
-  const float ms = mass * Sm;
-  const float px = mass * q.a.x * Sp, py = mass * q.a.y * Sp, pz = mass * q.a.z * Sp;
-  for_nodes(st, [&](int j, float w, float dx, float dy, float dz) {
-    atomicAdd(&sm[0][j], p2g_fixed<FMA>(w, ms));
-    atomicAdd(&sm[1][j], p2g_fixed<FMA>(w, px + A[0] * dx + A[1] * dy + A[2] * dz));
-    atomicAdd(&sm[2][j], p2g_fixed<FMA>(w, py + A[3] * dx + A[4] * dy + A[5] * dz));
-    atomicAdd(&sm[3][j], p2g_fixed<FMA>(w, pz + A[6] * dx + A[7] * dy + A[8] * dz));
-  });
 }
 
-// The same sums with the four components issued in a lane-rotated order.
-// A shared atomic instruction costs about the largest number of its lanes
-// that fall in one bank, and lanes on one address count like lanes on
+// Scatter of one particle.  The four sums of a node lie in four planes (the
+// three momenta, then the mass); plane c is a linear function of the node's
+// offset, w (R0 + R1 dx + R2 dy + R3 dz), with the rows R = (p_c, row c of A^)
+// of the momenta and (m, 0, 0, 0) of the mass, all pre-scaled.  Instruction
+// slots 0, 1 and 2, 3 are computed packed.
+// ROT: a shared atomic instruction costs about the largest number of its
+// lanes that fall in one bank, and lanes on one address count like lanes on
 // distinct addresses of that bank: about three lanes of an instruction share
-// a cell and so every node of the stencil.  Here the instruction of slot c
-// (c = 0..3) adds component (c + rot) & 3, rot = (3 lane) & 3, so
-// neighbouring lanes of one cell write different planes (plane stride
-// kP2GRotPlane, 24 banks apart).  Every component is written as
-// w (R0 + R1 dx + R2 dy + R3 dz) with the rows R of the mass (m, 0, 0, 0) and
-// of the momenta (p_c, row c of A^); the lane's rows are permuted once per
-// particle by two selects each, so no register array is indexed at run
-// time.  pl[c] is the plane that instruction slot c writes.
+// a cell and so every node of the stencil.  Slot c then adds plane
+// (c + rot) & 3, rot = (3 lane) & 3, so neighbouring lanes of one cell write
+// different planes (plane stride kP2GRotPlane, 24 banks apart); the lane's
+// rows are permuted once per particle by two selects each, so no register
+// array is indexed at run time.  pl[c] is the plane that slot c writes.
+// TR: 0 APIC + MLS: A^ = M D^-1 / dx, so that A (x_i - x_p) = A^ (offset in
+// cells).  1 PIC with the kernel gradient (Sec. 4.3): the state holds
+// M = -dt V0 tau (B = 0) and a node receives w m v + M grad w with
+// grad w = -g / dx: the rows multiply g in place of w d.  2 APIC with the
+// kernel gradient: M = m B, T = -dt V0 tau apart, both terms.
 template <int KIND>
 struct P2GRotPlane {
   static constexpr int value = ((Geo<KIND>::NS + 7) / 32) * 32 + 24;  // >= NS, = 24 mod 32
 };
 
-template <int KIND, bool FMA = false>
-__device__ __forceinline__ void p2g_scatter_rot(const SceneDev& s, const MatDev* mats, uint32_t* err,
-                                                const P2GPart& q, int ox, int oy, int oz, float Sm, float Sp,
-                                                int* const* pl, uint32_t rot) {
+// Rows of the four slots, packed by slots (0, 1) and (2, 3): e = 0 the
+// constant, 1..3 the columns of an M3 (the mass row has none).
+struct P2GRows {
+  f2 a, b;
+};
+template <bool ROT>
+__device__ __forceinline__ P2GRows p2g_rows(const V3& mom, float mass, bool r1, bool r2) {
+  if constexpr (!ROT) {
+    return {mom.p, pk(mom.z, mass)};
+  } else {
+    const float t0 = r1 ? mom.p.y : mom.p.x, t1 = r1 ? mom.z : mom.p.y, t2 = r1 ? mass : mom.z, t3 = r1 ? mom.p.x : mass;
+    return {pk(r2 ? t2 : t0, r2 ? t3 : t1), pk(r2 ? t0 : t2, r2 ? t1 : t3)};
+  }
+}
+
+template <int KIND, int TR, bool ROT, bool FMA>
+__device__ __forceinline__ void p2g_scatter(const SceneDev& s, const MatDev* mats, uint32_t* err, const P2GPart& q,
+                                            const M3& T, int ox, int oy, int oz, float Sm, float Sp, int* const* pl,
+                                            uint32_t rot) {
   Sten<KIND> st;
   if (!st.set(q.X.x * s.inv_dx, q.X.y * s.inv_dx, q.X.z * s.inv_dx, ox, oy, oz)) {
     flag_error(err, CK_ERR_INTERNAL);
     return;
   }
-  const float M[9] = {q.a.w, q.b.x, q.b.y, q.b.z, q.b.w, q.c.x, q.c.y, q.c.z, q.c.w};
-  float A[9];
-  mul_dinv(st, M, s.inv_dx * Sp, A);
+  const M3 M = unpack_m3(q.b, q.c, q.a.w);
   const float mass = mats[__float_as_uint(q.X.w)].mass;
-  const float R[4][4] = {{mass * Sm, 0.f, 0.f, 0.f},
-                         {mass * q.a.x * Sp, A[0], A[1], A[2]},
-                         {mass * q.a.y * Sp, A[3], A[4], A[5]},
-                         {mass * q.a.z * Sp, A[6], A[7], A[8]}};
+  const V3 p = (mass * Sp) * V3{pk(q.a.x, q.a.y), q.a.z};
   const bool r1 = (rot & 1u) != 0u, r2 = (rot & 2u) != 0u;
-  float T[4][4], Q[4][4];
+  // Q: constant and APIC columns; H: kernel-gradient columns
+  P2GRows Q[4], H[4];
+  Q[0] = p2g_rows<ROT>(p, mass * Sm, r1, r2);
+  if constexpr (TR != 1) {
+    const M3 A = mul_dinv(st, M, s.inv_dx * Sp);
 #pragma unroll
-  for (int c = 0; c < 4; ++c)
+    for (int e = 0; e < 3; ++e) Q[e + 1] = p2g_rows<ROT>(A.c[e], 0.f, r1, r2);
+  }
+  if constexpr (TR != 0) {
+    st.set_grad();
+    const float sc = -s.inv_dx * Sp;
 #pragma unroll
-    for (int e = 0; e < 4; ++e) T[c][e] = r1 ? R[(c + 1) & 3][e] : R[c][e];
+    for (int e = 0; e < 3; ++e) H[e + 1] = p2g_rows<ROT>(sc * (TR == 1 ? M.c[e] : T.c[e]), 0.f, r1, r2);
+  }
+  constexpr int N = Geo<KIND>::N;
 #pragma unroll
-  for (int c = 0; c < 4; ++c)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) Q[c][e] = r2 ? T[(c + 2) & 3][e] : T[c][e];
-  if constexpr (KIND == 0) {
-#pragma unroll
-    for (int g = 0; g < 2; ++g) {
-      const int E = g == 0 ? 5 : 6;
-      const int jb = (g == 0 ? 0 : 125) + (st.r[g][2] * E + st.r[g][1]) * E + st.r[g][0];
-      int* const b0 = pl[0] + jb;
-      int* const b1 = pl[1] + jb;
-      int* const b2 = pl[2] + jb;
-      int* const b3 = pl[3] + jb;
-#pragma unroll
-      for (int sz = 0; sz < 2; ++sz)
-#pragma unroll
-        for (int sy = 0; sy < 2; ++sy) {
-          const float wyz = st.w[g][1][sy] * st.w[g][2][sz];
-          const float dy = st.d[g][1][sy], dz = st.d[g][2][sz];
-          float e[4];
-#pragma unroll
-          for (int c = 0; c < 4; ++c) e[c] = fmaf(Q[c][3], dz, fmaf(Q[c][2], dy, Q[c][0]));
-#pragma unroll
-          for (int sx = 0; sx < 2; ++sx) {
-            const int o = (sz * E + sy) * E + sx;
-            const float w = st.w[g][0][sx] * wyz;
-            const float dx = st.d[g][0][sx];
-            atomicAdd(b0 + o, p2g_fixed<FMA>(w, fmaf(Q[0][1], dx, e[0])));
-            atomicAdd(b1 + o, p2g_fixed<FMA>(w, fmaf(Q[1][1], dx, e[1])));
-            atomicAdd(b2 + o, p2g_fixed<FMA>(w, fmaf(Q[2][1], dx, e[2])));
-            atomicAdd(b3 + o, p2g_fixed<FMA>(w, fmaf(Q[3][1], dx, e[3])));
-          }
-        }
-    }
-  } else {
-    const int jb = (st.r[2] * 6 + st.r[1]) * 6 + st.r[0];
+  for (int g = 0; g < Geo<KIND>::NG; ++g) {
+    const int E = pitch<KIND>(g), jb = first_node<KIND>(st, g);
     int* const b0 = pl[0] + jb;
     int* const b1 = pl[1] + jb;
     int* const b2 = pl[2] + jb;
     int* const b3 = pl[3] + jb;
 #pragma unroll
-    for (int sz = 0; sz < 3; ++sz)
+    for (int sz = 0; sz < N; ++sz)
 #pragma unroll
-      for (int sy = 0; sy < 3; ++sy) {
-        const float wyz = st.w[1][sy] * st.w[2][sz];
-        const float dy = st.d[1][sy], dz = st.d[2][sz];
-        float e[4];
+      for (int sy = 0; sy < N; ++sy) {
+        const float wy = st.w(g, sy).p.y, wz = st.w(g, sz).z, wyz = wy * wz;
+        const float dy = st.d(g, sy).p.y, dz = st.d(g, sz).z;
+        f2 ea = Q[0].a, eb = Q[0].b, ha, hb;
+        if constexpr (TR != 1) {
+          ea = fma2(Q[3].a, dup(dz), fma2(Q[2].a, dup(dy), ea));
+          eb = fma2(Q[3].b, dup(dz), fma2(Q[2].b, dup(dy), eb));
+        }
+        if constexpr (TR != 0) {
+          // w e + g H = wx (wyz e + K'y wz H2 + wy K'z H3) + K'x (wyz H1)
+          const float kyz = st.k(g, sy).p.y * wz, ykz = wy * st.k(g, sz).z;
+          ea = fma2(H[3].a, dup(ykz), fma2(H[2].a, dup(kyz), mul2(dup(wyz), ea)));
+          eb = fma2(H[3].b, dup(ykz), fma2(H[2].b, dup(kyz), mul2(dup(wyz), eb)));
+          ha = mul2(dup(wyz), H[1].a);
+          hb = mul2(dup(wyz), H[1].b);
+        }
 #pragma unroll
-        for (int c = 0; c < 4; ++c) e[c] = fmaf(Q[c][3], dz, fmaf(Q[c][2], dy, Q[c][0]));
-#pragma unroll
-        for (int sx = 0; sx < 3; ++sx) {
-          const int o = (sz * 6 + sy) * 6 + sx;
-          const float w = st.w[0][sx] * wyz;
-          const float dx = st.d[0][sx];
-          atomicAdd(b0 + o, p2g_fixed<FMA>(w, fmaf(Q[0][1], dx, e[0])));
-          atomicAdd(b1 + o, p2g_fixed<FMA>(w, fmaf(Q[1][1], dx, e[1])));
-          atomicAdd(b2 + o, p2g_fixed<FMA>(w, fmaf(Q[2][1], dx, e[2])));
-          atomicAdd(b3 + o, p2g_fixed<FMA>(w, fmaf(Q[3][1], dx, e[3])));
+        for (int sx = 0; sx < N; ++sx) {
+          const int o = (sz * E + sy) * E + sx;
+          const float wx = st.w(g, sx).p.x, dx = st.d(g, sx).p.x;
+          if constexpr (TR == 0) {
+            const f2 w = dup(wx * wyz);
+            p2g_add2<FMA>(b0 + o, b1 + o, w, fma2(Q[1].a, dup(dx), ea));
+            p2g_add2<FMA>(b2 + o, b3 + o, w, fma2(Q[1].b, dup(dx), eb));
+          } else {
+            f2 va = ea, vb = eb;
+            if constexpr (TR == 2) {
+              const float wdx = wyz * dx;
+              va = fma2(Q[1].a, dup(wdx), va);
+              vb = fma2(Q[1].b, dup(wdx), vb);
+            }
+            const float kx = st.k(g, sx).p.x;
+            va = fma2(dup(kx), ha, mul2(dup(wx), va));
+            vb = fma2(dup(kx), hb, mul2(dup(wx), vb));
+            p2g_add2<FMA>(b0 + o, b1 + o, dup(1.0f), va);
+            p2g_add2<FMA>(b2 + o, b3 + o, dup(1.0f), vb);
+          }
         }
       }
   }
-}
-
-// PIC transfer (Sec. 4.3 with the kernel gradient): the state holds
-// M = -dt V0 tau (B = 0), and a node receives w m v + M grad w with
-// grad w = -g / dx, i.e. w m v + A g with A = -M / dx, pre-scaled.
-template <int KIND>
-__device__ __forceinline__ void p2g_scatter_pic(const SceneDev& s, const MatDev* mats, uint32_t* err,
-                                                const P2GPart& q, int ox, int oy, int oz, float Sm, float Sp,
-                                                int (*sm)[Geo<KIND>::NS]) {
-  Sten<KIND> st;
-  if (!st.set(q.X.x * s.inv_dx, q.X.y * s.inv_dx, q.X.z * s.inv_dx, ox, oy, oz)) {
-    flag_error(err, CK_ERR_INTERNAL);
-    return;
-  }
-  st.set_grad();
-  const float M[9] = {q.a.w, q.b.x, q.b.y, q.b.z, q.b.w, q.c.x, q.c.y, q.c.z, q.c.w};
-  const float sc = -s.inv_dx * Sp;
-  float A[9];
-#pragma unroll
-  for (int r = 0; r < 9; ++r) A[r] = sc * M[r];
-  const float mass = mats[__float_as_uint(q.X.w)].mass;
-  const float ms = mass * Sm;
-  const float px = mass * q.a.x * Sp, py = mass * q.a.y * Sp, pz = mass * q.a.z * Sp;
-  for_nodes_grad(st, [&](int j, float w, float gx, float gy, float gz, float, float, float) {
-    atomicAdd(&sm[0][j], __float2int_rn(w * ms));
-    atomicAdd(&sm[1][j], __float2int_rn(fmaf(w, px, A[0] * gx + A[1] * gy + A[2] * gz)));
-    atomicAdd(&sm[2][j], __float2int_rn(fmaf(w, py, A[3] * gx + A[4] * gy + A[5] * gz)));
-    atomicAdd(&sm[3][j], __float2int_rn(fmaf(w, pz, A[6] * gx + A[7] * gy + A[8] * gz)));
-  });
-}
-
-// APIC with the kernel gradient: M = m B (state), T = -dt V0 tau (separate
-// arrays); a node receives w (m v + A d) + G g with A = m B D^-1 / dx (the
-// APIC momentum) and G = -T / dx (the force), both pre-scaled.
-template <int KIND>
-__device__ __forceinline__ void p2g_scatter_grad(const SceneDev& s, const MatDev* mats, uint32_t* err,
-                                                 const P2GPart& q, const float* T, int ox, int oy, int oz, float Sm,
-                                                 float Sp, int (*sm)[Geo<KIND>::NS]) {
-  Sten<KIND> st;
-  if (!st.set(q.X.x * s.inv_dx, q.X.y * s.inv_dx, q.X.z * s.inv_dx, ox, oy, oz)) {
-    flag_error(err, CK_ERR_INTERNAL);
-    return;
-  }
-  st.set_grad();
-  const float M[9] = {q.a.w, q.b.x, q.b.y, q.b.z, q.b.w, q.c.x, q.c.y, q.c.z, q.c.w};
-  float A[9], G[9];
-  mul_dinv(st, M, s.inv_dx * Sp, A);
-  const float sc = -s.inv_dx * Sp;
-#pragma unroll
-  for (int r = 0; r < 9; ++r) G[r] = sc * T[r];
-  const float mass = mats[__float_as_uint(q.X.w)].mass;
-  const float ms = mass * Sm;
-  const float px = mass * q.a.x * Sp, py = mass * q.a.y * Sp, pz = mass * q.a.z * Sp;
-  for_nodes_grad(st, [&](int j, float w, float gx, float gy, float gz, float dx, float dy, float dz) {
-    atomicAdd(&sm[0][j], __float2int_rn(w * ms));
-    atomicAdd(&sm[1][j], __float2int_rn(fmaf(w, px + A[0] * dx + A[1] * dy + A[2] * dz,
-                                             G[0] * gx + G[1] * gy + G[2] * gz)));
-    atomicAdd(&sm[2][j], __float2int_rn(fmaf(w, py + A[3] * dx + A[4] * dy + A[5] * dz,
-                                             G[3] * gx + G[4] * gy + G[5] * gz)));
-    atomicAdd(&sm[3][j], __float2int_rn(fmaf(w, pz + A[6] * dx + A[7] * dy + A[8] * dz,
-                                             G[6] * gx + G[7] * gy + G[8] * gz)));
-  });
 }
 
 // Replicated accumulators: with REP = 2 the staged sums exist twice and a
@@ -824,25 +704,24 @@ struct P2GRep {
 };
 
 // TR: transfer, 0 APIC + MLS, 1 PIC, 2 APIC with the kernel gradient.
-// ROT (APIC + MLS, one copy): components issued in the lane-rotated order of
-// p2g_scatter_rot, planes kP2GRotPlane apart.  FMA (APIC + MLS): blocks of
-// at least kP2GFmaCount particles round their contributions by p2g_fixed's
-// fused multiply-add instead of a conversion.
+// ROT (one copy): components issued in the lane-rotated order of p2g_scatter,
+// planes kP2GRotPlane apart.  FMA: blocks of at least kP2GFmaCount particles
+// round their contributions by p2g_add2's multiply-add instead of a
+// conversion.
 template <int KIND, int TR, int REP, int ROT = 0, int FMA = 0>
 __global__ void __launch_bounds__(kP2GWarp) k_p2g(StepView v) {
   constexpr int NS = Geo<KIND>::NS;
-  static_assert(ROT == 0 || (REP == 1 && TR == 0), "the rotated order takes one copy and APIC + MLS");
-  static_assert(FMA == 0 || TR == 0, "fused-multiply-add rounding is built for APIC + MLS");
+  static_assert(ROT == 0 || REP == 1, "the rotated order takes one copy");
   constexpr int PL = ROT ? P2GRotPlane<KIND>::value : NS;  // plane stride of the components
   constexpr int RS = ROT ? 4 * PL : P2GRep<KIND, REP>::stride;
   constexpr uint32_t CAP = kP2GStage, C = kP2GStage / 32;
   static_assert(C % 2 == 1, "lane stride must be odd");
   static_assert(RS % 4 == 0, "copies must keep 16-byte alignment");
   __shared__ __align__(16) int small[REP * RS];
-  int(*sm)[NS] = reinterpret_cast<int(*)[NS]>(small + (REP == 1 ? 0 : (int)(threadIdx.x & 1u) * RS));
-  const uint32_t rot = (threadIdx.x * 3u) & 3u;
-  int* const pl[4] = {small + ((0u + rot) & 3u) * PL, small + ((1u + rot) & 3u) * PL,
-                      small + ((2u + rot) & 3u) * PL, small + ((3u + rot) & 3u) * PL};
+  const uint32_t rot = ROT ? (threadIdx.x * 3u) & 3u : 0u;
+  int* const copy = small + (REP == 1 ? 0 : (int)(threadIdx.x & 1u) * RS);
+  int* const pl[4] = {copy + ((0u + rot) & 3u) * PL, copy + ((1u + rot) & 3u) * PL, copy + ((2u + rot) & 3u) * PL,
+                      copy + ((3u + rot) & 3u) * PL};
   __shared__ float4 sX[CAP], sA[CAP], sB[CAP], sC[CAP];
   constexpr uint32_t TCAP = TR == 2 ? CAP : 1;  // the stress term T (kernel-gradient APIC only)
   __shared__ float4 sT0[TCAP], sT1[TCAP];
@@ -892,24 +771,13 @@ __global__ void __launch_bounds__(kP2GWarp) k_p2g(StepView v) {
       for (uint32_t r = 0; r < C; ++r) {
         const uint32_t i = lane * C + r;
         if (i < m) {
-          const P2GPart q{sX[i], sA[i], sB[i], sC[i]};
-          if constexpr (TR == 1) {
-            p2g_scatter_pic<KIND>(s, v.mats, v.err, q, ox, oy, oz, Sm, Sp, sm);
-          } else if constexpr (TR == 2) {
-            const float4 t0 = sT0[i], t1 = sT1[i];
-            const float T[9] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w, sT2[i]};
-            p2g_scatter_grad<KIND>(s, v.mats, v.err, q, T, ox, oy, oz, Sm, Sp, sm);
-          } else if constexpr (ROT != 0) {
-            if (FMA && cnt >= kP2GFmaCount)
-              p2g_scatter_rot<KIND, true>(s, v.mats, v.err, q, ox, oy, oz, Sm, Sp, pl, rot);
-            else
-              p2g_scatter_rot<KIND, false>(s, v.mats, v.err, q, ox, oy, oz, Sm, Sp, pl, rot);
-          } else {
-            if (FMA && cnt >= kP2GFmaCount)
-              p2g_scatter<KIND, true>(s, v.mats, v.err, q, ox, oy, oz, Sm, Sp, sm);
-            else
-              p2g_scatter<KIND, false>(s, v.mats, v.err, q, ox, oy, oz, Sm, Sp, sm);
-          }
+          const P2GPart part{sX[i], sA[i], sB[i], sC[i]};
+          M3 T{};
+          if constexpr (TR == 2) T = unpack_m3(sT0[i], sT1[i], sT2[i]);
+          if (FMA && cnt >= kP2GFmaCount)
+            p2g_scatter<KIND, TR, ROT != 0, true>(s, v.mats, v.err, part, T, ox, oy, oz, Sm, Sp, pl, rot);
+          else
+            p2g_scatter<KIND, TR, ROT != 0, false>(s, v.mats, v.err, part, T, ox, oy, oz, Sm, Sp, pl, rot);
         }
       }
       __syncwarp();  // the next chunk overwrites the staged copies
@@ -924,13 +792,13 @@ __global__ void __launch_bounds__(kP2GWarp) k_p2g(StepView v) {
         q[c] = small[c * PL + j];
         if (REP == 2) q[c] += small[RS + c * NS + j];
       }
-      if (q[0] != 0) {
+      if (q[3] != 0) {
         int g, lx, ly, lz;
         staged_coords<KIND>(j, g, lx, ly, lz);
         long long gi = pool_index<KIND>(bslot, g, lx, ly, lz);
         if (gi >= 0)
-          atomicAdd(&v.Gacc[gi], make_float4((float)q[0] * iSm, (float)q[1] * iSp, (float)q[2] * iSp,
-                                             (float)q[3] * iSp));
+          atomicAdd(&v.Gacc[gi], make_float4((float)q[3] * iSm, (float)q[0] * iSp, (float)q[1] * iSp,
+                                             (float)q[2] * iSp));
       }
     }
     // (the block's bounds are cleared after G2P, by the float64 pass: other
@@ -1005,6 +873,16 @@ __device__ __forceinline__ float min3(float a, float b, float c) { return fminf(
 constexpr int kG2PWarp = 32;
 __host__ __device__ constexpr int g2p_stage(int minb) { return minb >= 5 ? 64 : 128; }  // particles per chunk
 
+// |A| + |B| elementwise (the bound of the kernel-gradient APIC's two terms)
+__device__ __forceinline__ M3 abs_sum(const M3& A, const M3& B) {
+  M3 r;
+#pragma unroll
+  for (int q = 0; q < 3; ++q)
+    r.c[q] = {pk(fabsf(A.c[q].p.x) + fabsf(B.c[q].p.x), fabsf(A.c[q].p.y) + fabsf(B.c[q].p.y)),
+              fabsf(A.c[q].z) + fabsf(B.c[q].z)};
+  return r;
+}
+
 // Result of one particle's G2P: its next key and P2G contribution bounds,
 // whether its constitutive update was deferred to the float64 pass, and
 // whether its new state is finite.
@@ -1014,179 +892,239 @@ struct G2POut {
   bool use64, fin;
 };
 
+// What a particle's update reads of its scene, in 16-byte groups.
+struct alignas(16) SceneStep {
+  float inv_dx, dt, dx, mdtv;               // mdtv = -dt V0
+  float gs, hi, j_tol, cond_tol;            // gs = dt / dx; hi = res - 1/2
+  float gap_tol;
+  int npb;
+  uint32_t key_base;
+  int res;
+  __device__ __forceinline__ void set(const SceneDev& s) {
+    inv_dx = s.inv_dx;
+    dt = s.dt;
+    dx = s.dx;
+    mdtv = -s.dt * s.V0;
+    gs = s.dt * s.inv_dx;
+    hi = (float)s.res - 0.5f;
+    j_tol = s.j_tol;
+    cond_tol = s.cond_tol;
+    gap_tol = s.gap_tol;
+    npb = s.npb;
+    key_base = s.key_base;
+    res = s.res;
+  }
+};
+
+// One particle's staged state (shared memory).  Read where it is used: the
+// position and the material index a second time after the gather, instead of
+// in registers across it.
+struct G2PIn {
+  const float4 *X, *F0, *F1;
+  const float *F2, *E;
+  const uint32_t* ID;
+};
+
+// A second read of a staged value that the compiler does not merge with the
+// first (which would keep it in registers in between).
+__device__ __forceinline__ float4 again(const float4* p) {
+  float4 r;
+  const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w) : "r"(a));
+  return r;
+}
+
 // G2P of one particle (slot t of the current binned order): gather v and B
 // (or the kernel-gradient sums) from the staged grid velocities sv, F update,
 // constitutive update (or listing for the float64 pass), advection, next key
 // and bounds; stores the new state at slot t of nxt.  Returns false (and
 // flags CK_ERR_INTERNAL) for a particle outside its block.
 template <int KIND, int TR>
-__device__ __forceinline__ bool g2p_particle(const StepView& v, const SceneDev& s, int ox, int oy, int oz,
-                                             const float4* sv, uint32_t t, const float4 X, const float4 f0,
-                                             const float4 f1, const float f2, const uint32_t id, const float Eraw,
-                                             G2POut& out, const MatDev* smat = nullptr) {
+__device__ __forceinline__ bool g2p_particle(const StepView& v, const SceneStep* sc, int ox, int oy, int oz,
+                                             const Nodes& sv, uint32_t t, const G2PIn& in, G2POut& out,
+                                             const MatDev* smat = nullptr) {
   out.use64 = false;
-  const uint32_t mi = __float_as_uint(X.w);
-  // the material table from shared memory when the kernel staged it there
-  const MatDev mt = smat ? smat[mi] : v.mats[mi];
-  float mu = mt.mu, lam = mt.lam;
-  float Ep = 0.f;
-  if (v.cur.E) {
-    Ep = Eraw;
-    mu = Ep / (2.0f * (1.0f + mt.nu));
-    lam = Ep * mt.nu / ((1.0f + mt.nu) * (1.0f - 2.0f * mt.nu));
-  }
   Sten<KIND> st;
-  if (!st.set(X.x * s.inv_dx, X.y * s.inv_dx, X.z * s.inv_dx, ox, oy, oz)) {
-    flag_error(v.err, CK_ERR_INTERNAL);
-    return false;
+  {
+    const float4 X = *in.X;
+    const float inv_dx = sc->inv_dx;
+    if (!st.set(X.x * inv_dx, X.y * inv_dx, X.z * inv_dx, ox, oy, oz)) {
+      flag_error(v.err, CK_ERR_INTERNAL);
+      return false;
+    }
   }
-  float vel[3], Bh[9], G[9];
+  V3 vel;
+  M3 Bh, C;  // C = dt grad v
   if constexpr (TR == 1) {
-    // grad v = -Gr / dx (Gr in Bh); F' = (I + dt grad v) F
+    // grad v = -Gr / dx (Gr in Bh)
     st.set_grad();
-    g2p_gather_grad(st, sv, vel, Bh);
-    const float sc = -s.dt * s.inv_dx;
+    g2p_gather_grad<KIND>(st, sv, vel, Bh);
+    const float gs = -sc->gs;
 #pragma unroll
-    for (int q = 0; q < 9; ++q) G[q] = sc * Bh[q];
+    for (int q = 0; q < 3; ++q) C.c[q] = gs * Bh.c[q];
   } else if constexpr (TR == 2) {
     // B from the APIC moments, grad v = -Gr / dx from the derivative sums
-    g2p_gather(st, sv, vel, Bh);
+    g2p_gather<KIND>(st, sv, vel, Bh);
     st.set_grad();
-    float vg[3];
-    g2p_gather_grad(st, sv, vg, G);
-    const float sc = -s.dt * s.inv_dx;
+    V3 vg;
+    g2p_gather_grad<KIND>(st, sv, vg, C);
+    const float gs = -sc->gs;
 #pragma unroll
-    for (int q = 0; q < 9; ++q) G[q] *= sc;
+    for (int q = 0; q < 3; ++q) C.c[q] = gs * C.c[q];
   } else {
-    // C = B D^-1 = Bh D^-1 / dx ; F' = (I + dt C) F
-    g2p_gather(st, sv, vel, Bh);
-    mul_dinv(st, Bh, s.dt * s.inv_dx, G);
+    // grad v = B D^-1 = Bh D^-1 / dx
+    g2p_gather<KIND>(st, sv, vel, Bh);
+    C = mul_dinv(st, Bh, sc->gs);
   }
-  const float vx = vel[0], vy = vel[1], vz = vel[2];
-  G[0] += 1.0f;
-  G[4] += 1.0f;
-  G[8] += 1.0f;
-  const float Fo[9] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w, f2};
-  float F[9];
-#pragma unroll
-  for (int r = 0; r < 3; ++r)
-#pragma unroll
-    for (int q = 0; q < 3; ++q)
-      F[r * 3 + q] = G[r * 3 + 0] * Fo[0 * 3 + q] + G[r * 3 + 1] * Fo[1 * 3 + q] + G[r * 3 + 2] * Fo[2 * 3 + q];
+  const float vx = vel.p.x, vy = vel.p.y, vz = vel.z;
+  const float4 X = again(in.X);
+  const uint32_t mi = __float_as_uint(X.w);
+  // the material table from shared memory when the kernel staged it there
+  const MatDev* mt = (smat ? smat : v.mats) + mi;
+  const float4 m4 = *reinterpret_cast<const float4*>(mt);  // mass, mu, lam, dpc
+  const int model = mt->model;
+  float mu = m4.y, lam = m4.z;
+  float Ep = 0.f;
+  if (v.cur.E) {
+    Ep = *in.E;
+    const float nu = mt->nu;
+    mu = Ep / (2.0f * (1.0f + nu));
+    lam = Ep * nu / ((1.0f + nu) * (1.0f - 2.0f * nu));
+  }
+  // F' = (I + dt grad v) F
+  const M3 Fo = unpack_m3(*in.F0, *in.F1, *in.F2);
+  M3 F = mul_add(C, Fo, Fo);
   // constitutive update in float32 from the left stretch; degenerate or
   // inverted F is deferred to the float64 pass (precision extension):
-  // this kernel stores F' and M = m B' (no stress) and lists the particle
-  float tau[9];
+  // this kernel stores F' and M = m B' (no stress) and lists the particle.
+  // ft: -dt V0 tau
+  M3 ft;
+  const float4 s4 = *reinterpret_cast<const float4*>(sc);  // inv_dx, dt, dx, mdtv
+  const float inv_dx = s4.x, dt = s4.y, dx = s4.z, mdtv = s4.w;
   // Drucker-Prager at small stretch: matrix log/exp series, no eigen-
   // decomposition (such F is far from every float64 criterion)
-  float Xs[6];
-  const float xr = mt.model == 1 ? left_strain(F, Xs) : 1.f;
-  const bool small_dp = mt.model == 1 && s.gap_tol <= 0.f && s.j_tol < 0.9f && s.cond_tol < 0.9f &&
+  Sym Xs;
+  const float xr = model == 1 ? left_strain(F, Xs) : 1.f;
+  const bool small_dp = model == 1 && sc->gap_tol <= 0.f && sc->j_tol < 0.9f && sc->cond_tol < 0.9f &&
                         xr <= (1.f / 48.f);
   const int sdeg = dp_lane_degree(xr);
-  if (mt.model == 2) {
-    // J-based fluid: volume ratio only, stress from J (no decomposition)
-    fluid_update<float>(F, mt.E, mt.gamma, tau);
-  } else if (small_dp) {
-    dp_small_strain(F, Xs, sdeg, mu, lam, mt.dpc, tau);
+  if (small_dp) {
+    Sym tau;
+    dp_small_strain(F, Xs, sdeg, mu, lam, m4.w, mdtv, tau);
+    ft = sym_m3(tau);
   } else {
-    // b = F F^T = U diag(sigma^2) U^T
-    float bq[9], U[9], e[3], sg[3];
-#pragma unroll
-    for (int r = 0; r < 3; ++r)
-#pragma unroll
-      for (int q = r; q < 3; ++q) {
-        const float d = F[r * 3] * F[q * 3] + F[r * 3 + 1] * F[q * 3 + 1] + F[r * 3 + 2] * F[q * 3 + 2];
-        bq[r * 3 + q] = d;
-        bq[q * 3 + r] = d;
-      }
-    sym_eig3<float>(bq, U, e);
-    sg[0] = sqrtf(fmaxf(e[0], 0.f));
-    sg[1] = sqrtf(fmaxf(e[1], 0.f));
-    sg[2] = sqrtf(fmaxf(e[2], 0.f));
-    const float J = F[0] * (F[4] * F[8] - F[5] * F[7]) - F[1] * (F[3] * F[8] - F[5] * F[6]) +
-                    F[2] * (F[3] * F[7] - F[4] * F[6]);
-    const float smax = fmaxf(sg[0], fmaxf(sg[1], sg[2]));
-    const float smin = min3(sg[0], sg[1], sg[2]);
-    const float gap = min3(fabsf(sg[0] - sg[1]), fabsf(sg[0] - sg[2]), fabsf(sg[1] - sg[2]));
-    const bool use64 = !(J > 0.f) || (fabsf(J) < s.j_tol) || (smin < s.cond_tol * smax) ||
-                       (gap < s.gap_tol * smax);
-    out.use64 = use64;
-    if (use64) {
-      const unsigned long long slot = atomicAdd(v.fp64_count, 1ull);
-      v.fp64_list[slot] = t;
-#pragma unroll
-      for (int q = 0; q < 9; ++q) tau[q] = 0.f;
+    float Fr[9], tau[9];
+    to_rows(F, Fr);
+    if (model == 2) {
+      // J-based fluid: volume ratio only, stress from J (no decomposition)
+      fluid_update<float>(Fr, mt->E, mt->gamma, tau);
     } else {
-      constitutive_left<float>(mt.model, F, mu, lam, mt.alpha, tau, U, e, sg);
+      // b = F F^T = U diag(sigma^2) U^T
+      float bq[9], U[9], e[3], sg[3];
+#pragma unroll
+      for (int r = 0; r < 3; ++r)
+#pragma unroll
+        for (int q = r; q < 3; ++q) {
+          const float d = Fr[r * 3] * Fr[q * 3] + Fr[r * 3 + 1] * Fr[q * 3 + 1] + Fr[r * 3 + 2] * Fr[q * 3 + 2];
+          bq[r * 3 + q] = d;
+          bq[q * 3 + r] = d;
+        }
+      sym_eig3<float>(bq, U, e);
+      sg[0] = sqrtf(fmaxf(e[0], 0.f));
+      sg[1] = sqrtf(fmaxf(e[1], 0.f));
+      sg[2] = sqrtf(fmaxf(e[2], 0.f));
+      const float J = det3<float>(Fr);
+      const float smax = fmaxf(sg[0], fmaxf(sg[1], sg[2]));
+      const float smin = min3(sg[0], sg[1], sg[2]);
+      const float gap = min3(fabsf(sg[0] - sg[1]), fabsf(sg[0] - sg[2]), fabsf(sg[1] - sg[2]));
+      const bool use64 = !(J > 0.f) || (fabsf(J) < sc->j_tol) || (smin < sc->cond_tol * smax) ||
+                         (gap < sc->gap_tol * smax);
+      out.use64 = use64;
+      if (use64) {
+        const unsigned long long slot = atomicAdd(v.fp64_count, 1ull);
+        v.fp64_list[slot] = t;
+#pragma unroll
+        for (int q = 0; q < 9; ++q) tau[q] = 0.f;
+      } else {
+        constitutive_left<float>(model, Fr, mu, lam, mt->alpha, tau, U, e, sg);
+      }
     }
+    F = from_rows(Fr);
+    ft = from_rows(tau);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) ft.c[q] = mdtv * ft.c[q];
   }
   // M' = m B' - dt V0 tau, B' = dx Bh (APIC) or 0 (PIC); the kernel-
   // gradient APIC keeps M' = m B' and T' = -dt V0 tau apart
-  const float mdx = mt.mass * s.dx, dtv = s.dt * s.V0;
-  float Mn[9];
+  const float mdx = m4.x * dx;
+  M3 Mn;
 #pragma unroll
-  for (int q = 0; q < 9; ++q)
-    Mn[q] = TR == 1 ? -dtv * tau[q] : TR == 2 ? mdx * Bh[q] : mdx * Bh[q] - dtv * tau[q];
-  float4 Xn = make_float4(X.x + s.dt * vx, X.y + s.dt * vy, X.z + s.dt * vz, X.w);
+  for (int q = 0; q < 3; ++q) Mn.c[q] = TR == 1 ? ft.c[q] : TR == 2 ? mdx * Bh.c[q] : fma3(mdx, Bh.c[q], ft.c[q]);
+  float4 Xn = make_float4(X.x + dt * vx, X.y + dt * vy, X.z + dt * vz, X.w);
   // next key; particles leaving the interior are clamped and flagged
-  float ux = Xn.x * s.inv_dx, uy = Xn.y * s.inv_dx, uz = Xn.z * s.inv_dx;
+  float ux = Xn.x * inv_dx, uy = Xn.y * inv_dx, uz = Xn.z * inv_dx;
   // x was finite, so x + dt v is finite when v is.  x * 0 is 0 for a finite
   // x and NaN for an infinite or NaN one, so one sum of such products tests
   // every value at one fused multiply-add each
-  float z = fmaf(vx, 0.f, fmaf(vy, 0.f, vz * 0.f));
+  V3 z = 0.f * vel;
 #pragma unroll
-  for (int q = 0; q < 9; ++q) {
-    z = fmaf(F[q], 0.f, fmaf(Mn[q], 0.f, z));
-    if constexpr (TR == 2) z = fmaf(tau[q], 0.f, z);
+  for (int q = 0; q < 3; ++q) {
+    z = fma3(0.f, F.c[q], fma3(0.f, Mn.c[q], z));
+    if constexpr (TR == 2) z = fma3(0.f, ft.c[q], z);
   }
-  const bool fin = z == 0.f;
+  const bool fin = z.p.x + z.p.y + z.z == 0.f;
   if (!fin) flag_error(v.err, CK_ERR_NONFINITE);
   out.fin = fin;
-  if (!(in_domain(ux, s.res) && in_domain(uy, s.res) && in_domain(uz, s.res))) {
+  const float uhi = sc->hi;
+  if (!(ux >= 0.5f && ux < uhi && uy >= 0.5f && uy < uhi && uz >= 0.5f && uz < uhi)) {  // in_domain
     flag_error(v.err, CK_ERR_DOMAIN);
-    const float lo = 0.5f, hi = (float)s.res - 0.5f - 1e-3f;
+    const float lo = 0.5f, hi = (float)sc->res - 0.5f - 1e-3f;
     ux = fminf(fmaxf(isfinite(ux) ? ux : lo, lo), hi);
     uy = fminf(fmaxf(isfinite(uy) ? uy : lo, lo), hi);
     uz = fminf(fmaxf(isfinite(uz) ? uz : lo, lo), hi);
-    Xn.x = ux * s.dx;
-    Xn.y = uy * s.dx;
-    Xn.z = uz * s.dx;
-    ux = Xn.x * s.inv_dx;
-    uy = Xn.y * s.inv_dx;
-    uz = Xn.z * s.inv_dx;
+    Xn.x = ux * dx;
+    Xn.y = uy * dx;
+    Xn.z = uz * dx;
+    ux = Xn.x * inv_dx;
+    uy = Xn.y * inv_dx;
+    uz = Xn.z * inv_dx;
   }
-  const uint32_t nk = particle_key<KIND>(s, ux, uy, uz);
+  const uint32_t nk = particle_key<KIND>(*sc, ux, uy, uz);
   v.nxt.X[t] = Xn;
-  v.nxt.VM0[t] = make_float4(vx, vy, vz, Mn[0]);
-  v.nxt.VM1[t] = make_float4(Mn[1], Mn[2], Mn[3], Mn[4]);
-  v.nxt.VM2[t] = make_float4(Mn[5], Mn[6], Mn[7], Mn[8]);
-  v.nxt.F0[t] = make_float4(F[0], F[1], F[2], F[3]);
-  v.nxt.F1[t] = make_float4(F[4], F[5], F[6], F[7]);
-  v.nxt.F2[t] = F[8];
-  v.nxt.ID[t] = id;
+  float4 a, b;
+  float c;
+  pack_m3(Mn, a, b, c);
+  v.nxt.VM0[t] = make_float4(vx, vy, vz, c);
+  v.nxt.VM1[t] = a;
+  v.nxt.VM2[t] = b;
+  pack_m3(F, a, b, c);
+  v.nxt.F0[t] = a;
+  v.nxt.F1[t] = b;
+  v.nxt.F2[t] = c;
+  v.nxt.ID[t] = *in.ID;
   if (v.nxt.E) v.nxt.E[t] = Ep;
   v.key_nxt[t] = nk;
   out.nk = nk;
-  float& bmass = out.bmass;
-  float& bmom = out.bmom;
   if constexpr (TR == 2) {
-    float Tn[9], Mb[9];
-#pragma unroll
-    for (int q = 0; q < 9; ++q) {
-      Tn[q] = -dtv * tau[q];
-      Mb[q] = fabsf(Mn[q]) + fabsf(Tn[q]);
-    }
-    v.nxt.T0[t] = make_float4(Tn[0], Tn[1], Tn[2], Tn[3]);
-    v.nxt.T1[t] = make_float4(Tn[4], Tn[5], Tn[6], Tn[7]);
-    v.nxt.T2[t] = Tn[8];
-    p2g_bounds<KIND>(s.inv_dx, mt.mass, vx, vy, vz, Mb, bmass, bmom);
+    pack_m3(ft, a, b, c);
+    v.nxt.T0[t] = a;
+    v.nxt.T1[t] = b;
+    v.nxt.T2[t] = c;
+    p2g_bounds<KIND>(inv_dx, m4.x, vel, abs_sum(Mn, ft), out.bmass, out.bmom);
   } else {
-    p2g_bounds<KIND>(s.inv_dx, mt.mass, vx, vy, vz, Mn, bmass, bmom);
+    p2g_bounds<KIND>(inv_dx, m4.x, vel, Mn, out.bmass, out.bmom);
   }
   return true;
 }
 
+// Bound by its issue slots and the packed multiply-adds (68% of the slots
+// issue; DRAM 0.6 of the copy rate).  Measured against the scalar form (16.27 M
+// particles / dam break, 4.18 M): 0.637 -> 0.590 ms / 0.165 -> 0.152, with the
+// warp instructions per particle of the dam break down from 35 to 27; without
+// the staged scene and the second read of the position 16-byte spills put it
+// at 0.61 / 0.163, and a 16-byte node in place of NodeVel's 8 + 4 at 0.596 /
+// 0.158.  (P2G, bound by its shared atomics: 0.507 -> 0.491 / 0.148 -> 0.145.)
+//
 // G2P with the next chunk's particle state in flight.  Chunks of 32
 // particles (one per lane; each lane stages and reads only its own
 // particle's slot) alternate between two staging buffers: while chunk k is
@@ -1206,13 +1144,14 @@ __global__ void __launch_bounds__(kG2PWarp, 4 * MINB) k_g2p(StepView v) {
   constexpr int D = NB - 1;   // chunks in flight ahead of the computed one
   constexpr int PS = 2 * NB;  // slots of binned-order indices (D + 2 live at a time)
   static_assert((NB & (NB - 1)) == 0, "NB must be a power of two");
-  __shared__ float4 sv[NS];
+  __shared__ NodeVel<NS> svel;
   __shared__ float4 sX[NB][CH], sF0[NB][CH], sF1[NB][CH];
   __shared__ float sF2[NB][CH], sE[NB][CH];
   __shared__ uint32_t sID[NB][CH];
   __shared__ uint32_t sP[PS][CH];
   __shared__ uint32_t bslot[8];
   __shared__ MatDev smat[kSmemMats];
+  __shared__ SceneStep sstep;  // the unit's scene, read where it is used (registers)
   const uint32_t lane = threadIdx.x;
   const bool mat_smem = v.n_mats <= (uint32_t)kSmemMats;
   if (mat_smem) {
@@ -1227,7 +1166,8 @@ __global__ void __launch_bounds__(kG2PWarp, 4 * MINB) k_g2p(StepView v) {
     Unit q;
     if (!unit_of(v, u, CH, q)) continue;
     const uint32_t key = q.key, start = q.start, lo = q.lo, hi = q.hi;
-    const SceneDev s = v.scenes[q.scene];
+    const SceneDev& s = v.scenes[q.scene];
+    if (lane == 0) sstep.set(s);
     int ox, oy, oz;
     decode_block(s, key, ox, oy, oz);
     load_block_slots(v, s, ox, oy, oz, bslot);
@@ -1252,9 +1192,9 @@ __global__ void __launch_bounds__(kG2PWarp, 4 * MINB) k_g2p(StepView v) {
       staged_coords<KIND>(j, g, lx, ly, lz);
       const long long gi = pool_index<KIND>(bslot, g, lx, ly, lz);
       if (gi >= 0)
-        cp_async16(&sv[j], &v.Gvel[gi]);
+        stage_node(svel, j, &v.Gvel[gi]);
       else
-        sv[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+        svel.xy[j] = make_float2(0.f, 0.f), svel.z[j] = 0.f;
     }
     auto stage = [&](uint32_t c, uint32_t p) {
       const uint32_t b = c & (NB - 1);
@@ -1288,9 +1228,8 @@ __global__ void __launch_bounds__(kG2PWarp, 4 * MINB) k_g2p(StepView v) {
       const uint32_t i = lo + k * CH + lane;
       if (i < hi) {
         G2POut o;
-        if (g2p_particle<KIND, TR>(v, s, ox, oy, oz, sv, start + i, sX[b][lane], sF0[b][lane], sF1[b][lane],
-                                   sF2[b][lane], sID[b][lane], v.cur.E ? sE[b][lane] : 0.f, o,
-                                   mat_smem ? smat : nullptr))
+        const G2PIn in{&sX[b][lane], &sF0[b][lane], &sF1[b][lane], &sF2[b][lane], &sE[b][lane], &sID[b][lane]};
+        if (g2p_particle<KIND, TR>(v, &sstep, ox, oy, oz, Nodes{svel.xy, svel.z}, start + i, in, o, mat_smem ? smat : nullptr))
           warp_aggregated_bin(v.cnt_nxt, v.bnd_nxt, o.nk, o.bmass, o.bmom);
       }
       __syncwarp();  // chunk k + NB is staged into this buffer next
@@ -1324,7 +1263,7 @@ struct FuseSmem {
   static constexpr int NS = Geo<KIND>::NS;
   static constexpr int CAP = g2p_stage(MINB);
   struct Ph1 {
-    float4 sv[NS];
+    NodeVel<NS> svel;
     float4 sX[CAP], sF0[CAP], sF1[CAP];
     float sF2[CAP], sE[CAP];
     uint32_t sID[CAP];
@@ -1358,6 +1297,7 @@ __global__ void __launch_bounds__(kG2PWarp, 4 * MINB) k_g2p2g(StepView v) {
   __shared__ __align__(16) unsigned char arena[SM::bytes];
   __shared__ uint32_t stay[kFuseMaxCnt / 32];
   __shared__ uint32_t bslot[8];
+  __shared__ SceneStep sstep;
   auto& p1 = *reinterpret_cast<typename SM::Ph1*>(arena);
   auto& p2 = *reinterpret_cast<typename SM::Ph2*>(arena);
   const uint32_t nunits = *v.n_pb * v.splits;
@@ -1371,6 +1311,7 @@ __global__ void __launch_bounds__(kG2PWarp, 4 * MINB) k_g2p2g(StepView v) {
     int ox, oy, oz;
     decode_block(s, key, ox, oy, oz);
     load_block_slots(v, s, ox, oy, oz, bslot);  // this step's grid (gather)
+    if (lane == 0) sstep.set(s);
     __syncwarp();
     // ---- pass 1: G2P of the block
     float bm_max = 0.f, bp_max = 0.f;
@@ -1393,9 +1334,9 @@ __global__ void __launch_bounds__(kG2PWarp, 4 * MINB) k_g2p2g(StepView v) {
           staged_coords<KIND>(j, g, lx, ly, lz);
           long long gi = pool_index<KIND>(bslot, g, lx, ly, lz);
           if (gi >= 0)
-            cp_async16(&p1.sv[j], &v.Gvel[gi]);
+            stage_node(p1.svel, j, &v.Gvel[gi]);
           else
-            p1.sv[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+            p1.svel.xy[j] = make_float2(0.f, 0.f), p1.svel.z[j] = 0.f;
         }
       }
       cp_async_wait_all();
@@ -1403,8 +1344,8 @@ __global__ void __launch_bounds__(kG2PWarp, 4 * MINB) k_g2p2g(StepView v) {
       for (uint32_t i = lane; i < m; i += 32) {
         const uint32_t t = start + c0 + i;
         G2POut o;
-        const bool ok = g2p_particle<KIND, 0>(v, s, ox, oy, oz, p1.sv, t, p1.sX[i], p1.sF0[i], p1.sF1[i],
-                                              p1.sF2[i], p1.sID[i], v.cur.E ? p1.sE[i] : 0.f, o);
+        const G2PIn in{&p1.sX[i], &p1.sF0[i], &p1.sF1[i], &p1.sF2[i], &p1.sE[i], &p1.sID[i]};
+        const bool ok = g2p_particle<KIND, 0>(v, &sstep, ox, oy, oz, Nodes{p1.svel.xy, p1.svel.z}, t, in, o);
         if (ok) warp_aggregated_bin(v.cnt_nxt, v.bnd_nxt, o.nk, o.bmass, o.bmom);
         const bool st = ok && track && o.nk == key && !o.use64 && o.fin;
         if (st) {
@@ -1429,6 +1370,7 @@ __global__ void __launch_bounds__(kG2PWarp, 4 * MINB) k_g2p2g(StepView v) {
         bslot[lane] = v.table_nxt[s.table_base + ((long long)bz * s.nb + by) * s.nb + bx];
       }
       for (int j = lane; j < NS; j += 32) reinterpret_cast<int4*>(&p2.sm[0][0])[j] = make_int4(0, 0, 0, 0);
+      int* const pl[4] = {p2.sm[0], p2.sm[1], p2.sm[2], p2.sm[3]};
       const float fst = (float)nstay;
       const float Sm = bm_max > 0.f ? 1073741824.0f / (fst * bm_max) : 1.0f;
       const float Sp = bp_max > 0.f ? 1073741824.0f / (fst * bp_max) : 1.0f;
@@ -1453,21 +1395,21 @@ __global__ void __launch_bounds__(kG2PWarp, 4 * MINB) k_g2p2g(StepView v) {
           const uint32_t q = c0 - lo + i;
           if (i < m && ((stay[q >> 5] >> (q & 31)) & 1u)) {
             const P2GPart part{p2.sX[i], p2.sA[i], p2.sB[i], p2.sC[i]};
-            p2g_scatter<KIND>(s, v.mats, v.err, part, ox, oy, oz, Sm, Sp, p2.sm);
+            p2g_scatter<KIND, 0, false, false>(s, v.mats, v.err, part, M3{}, ox, oy, oz, Sm, Sp, pl, 0u);
           }
         }
         __syncwarp();
       }
       const float iSm = 1.0f / Sm, iSp = 1.0f / Sp;
       for (int j = lane; j < NS; j += 32) {
-        const int mi = p2.sm[0][j];
+        const int mi = p2.sm[3][j];
         if (mi != 0) {
           int g, lx, ly, lz;
           staged_coords<KIND>(j, g, lx, ly, lz);
           const long long gi = pool_index<KIND>(bslot, g, lx, ly, lz);
           if (gi >= 0)
-            atomicAdd(&v.Gacc[gi], make_float4((float)mi * iSm, (float)p2.sm[1][j] * iSp,
-                                               (float)p2.sm[2][j] * iSp, (float)p2.sm[3][j] * iSp));
+            atomicAdd(&v.Gacc[gi], make_float4((float)mi * iSm, (float)p2.sm[0][j] * iSp,
+                                               (float)p2.sm[1][j] * iSp, (float)p2.sm[2][j] * iSp));
           else
             flag_error(v.err, CK_ERR_POOL);
         }
@@ -1520,14 +1462,12 @@ __global__ void __launch_bounds__(128) k_p2g_leftover(StepView v) {
       flag_error(v.err, CK_ERR_INTERNAL);
       continue;
     }
-    float M[9];
     const float4 a = v.nxt.VM0[t], b = v.nxt.VM1[t], c = v.nxt.VM2[t];
-    M[0] = a.w; M[1] = b.x; M[2] = b.y; M[3] = b.z; M[4] = b.w; M[5] = c.x; M[6] = c.y; M[7] = c.z; M[8] = c.w;
     float A[9];
-    mul_dinv(st, M, s.inv_dx, A);
+    to_rows(mul_dinv(st, unpack_m3(b, c, a.w), s.inv_dx), A);
     const float mass = mt.mass;
     const float px = mass * a.x, py = mass * a.y, pz = mass * a.z;
-    for_nodes(st, [&](int j, float w, float dx, float dy, float dz) {
+    for_nodes<KIND>(st, [&](int j, float w, float dx, float dy, float dz) {
       int g, lx, ly, lz;
       staged_coords<KIND>(j, g, lx, ly, lz);
       const int ix = ox + lx, iy = oy + ly, iz = oz + lz;
@@ -1540,6 +1480,41 @@ __global__ void __launch_bounds__(128) k_p2g_leftover(StepView v) {
                             w * (py + A[3] * dx + A[4] * dy + A[5] * dz), w * (pz + A[6] * dx + A[7] * dy + A[8] * dz)));
     });
   }
+}
+
+// One particle's matrices by rows (stored by pack.cuh's order).
+__device__ __forceinline__ void load_F(const Pool& P, uint32_t t, float* F) {
+  to_rows(unpack_m3(P.F0[t], P.F1[t], P.F2[t]), F);
+}
+__device__ __forceinline__ void store_F(const Pool& P, uint32_t t, const float* F) {
+  float4 a, b;
+  float c;
+  pack_m3(from_rows(F), a, b, c);
+  P.F0[t] = a;
+  P.F1[t] = b;
+  P.F2[t] = c;
+}
+__device__ __forceinline__ void load_M(const Pool& P, uint32_t t, float* M) {
+  to_rows(unpack_m3(P.VM1[t], P.VM2[t], P.VM0[t].w), M);
+}
+__device__ __forceinline__ void store_M(const Pool& P, uint32_t t, const float* M) {
+  float4 a, b;
+  float c;
+  pack_m3(from_rows(M), a, b, c);
+  P.VM0[t].w = c;
+  P.VM1[t] = a;
+  P.VM2[t] = b;
+}
+__device__ __forceinline__ void load_T(const Pool& P, uint32_t t, float* T) {
+  to_rows(unpack_m3(P.T0[t], P.T1[t], P.T2[t]), T);
+}
+__device__ __forceinline__ void store_T(const Pool& P, uint32_t t, const float* T) {
+  float4 a, b;
+  float c;
+  pack_m3(from_rows(T), a, b, c);
+  P.T0[t] = a;
+  P.T1[t] = b;
+  P.T2[t] = c;
 }
 
 // Float64 pass of the precision extension: the particles G2P listed (F
@@ -1575,51 +1550,35 @@ __global__ void __launch_bounds__(128) k_g2p_fp64(StepView v) {
       mu = E / (2.0 * (1.0 + nu));
       lam = E * nu / ((1.0 + nu) * (1.0 - 2.0 * nu));
     }
-    const float4 f0 = v.nxt.F0[t], f1 = v.nxt.F1[t];
-    double F[9] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w, v.nxt.F2[t]};
+    float Ff[9];
+    load_F(v.nxt, t, Ff);
+    double F[9];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) F[q] = Ff[q];
     double tau[9], sg[3];
     constitutive<double>(mt.model, F, mu, lam, (double)mt.alpha, tau, sg);
     const double dtv = (double)s.dt * (double)s.V0;
-    float4 a = v.nxt.VM0[t], b = v.nxt.VM1[t], c = v.nxt.VM2[t];
-    float Tn[9];
+    const float4 a = v.nxt.VM0[t];
+    float Mn[9], Tn[9];
+    load_M(v.nxt, t, Mn);
     const bool sep = v.nxt.T0 != nullptr;  // stress term kept apart from m B
-#pragma unroll
-    for (int q = 0; q < 9; ++q) Tn[q] = (float)(-dtv * tau[q]);
-    if (sep) {
-      v.nxt.T0[t] = make_float4(Tn[0], Tn[1], Tn[2], Tn[3]);
-      v.nxt.T1[t] = make_float4(Tn[4], Tn[5], Tn[6], Tn[7]);
-      v.nxt.T2[t] = Tn[8];
-    } else {
-      a.w = (float)(a.w - dtv * tau[0]);
-      b = make_float4((float)(b.x - dtv * tau[1]), (float)(b.y - dtv * tau[2]), (float)(b.z - dtv * tau[3]),
-                      (float)(b.w - dtv * tau[4]));
-      c = make_float4((float)(c.x - dtv * tau[5]), (float)(c.y - dtv * tau[6]), (float)(c.z - dtv * tau[7]),
-                      (float)(c.w - dtv * tau[8]));
-    }
-    float Ff[9];
-    bool fin = isfinite(a.w) && isfinite(b.x) && isfinite(b.y) && isfinite(b.z) && isfinite(b.w) &&
-               isfinite(c.x) && isfinite(c.y) && isfinite(c.z) && isfinite(c.w);
-#pragma unroll
-    for (int q = 0; q < 9; ++q) fin = fin && isfinite(Tn[q]);
+    bool fin = true;
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
+      Tn[q] = (float)(-dtv * tau[q]);
+      if (!sep) Mn[q] = (float)(Mn[q] - dtv * tau[q]);
       Ff[q] = (float)F[q];
-      fin = fin && isfinite(Ff[q]);
+      fin = fin && isfinite(Mn[q]) && isfinite(Tn[q]) && isfinite(Ff[q]);
     }
     if (!fin) flag_error(v.err, CK_ERR_NONFINITE);
-    v.nxt.VM0[t] = a;
-    v.nxt.VM1[t] = b;
-    v.nxt.VM2[t] = c;
-    v.nxt.F0[t] = make_float4(Ff[0], Ff[1], Ff[2], Ff[3]);
-    v.nxt.F1[t] = make_float4(Ff[4], Ff[5], Ff[6], Ff[7]);
-    v.nxt.F2[t] = Ff[8];
-    float Mn[9] = {a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w};
-    if (sep) {
-#pragma unroll
-      for (int q = 0; q < 9; ++q) Mn[q] = fabsf(Mn[q]) + fabsf(Tn[q]);
-    }
+    if (sep)
+      store_T(v.nxt, t, Tn);
+    else
+      store_M(v.nxt, t, Mn);
+    store_F(v.nxt, t, Ff);
+    const M3 Mb = sep ? abs_sum(from_rows(Mn), from_rows(Tn)) : from_rows(Mn);
     float bmass, bmom;
-    p2g_bounds<KIND>(s.inv_dx, mt.mass, a.x, a.y, a.z, Mn, bmass, bmom);
+    p2g_bounds<KIND>(s.inv_dx, mt.mass, V3{pk(a.x, a.y), a.z}, Mb, bmass, bmom);
     const uint32_t nk = v.key_nxt[t];
     atomicMax(&v.bnd_nxt[2 * nk], __float_as_uint(bmass));
     atomicMax(&v.bnd_nxt[2 * nk + 1], __float_as_uint(bmom));
@@ -1645,27 +1604,6 @@ __device__ __forceinline__ void stress_of(const MatDev& mt, const float* F, floa
     fluid_tau_of_J<float>(det3(F), mt.E, mt.gamma, tau);
   else
     stress_only<float>(mt.model, F, mu, lam, tau);
-}
-
-__device__ __forceinline__ void load_F(const Pool& P, uint32_t t, float* F) {
-  float4 a = P.F0[t], b = P.F1[t];
-  F[0] = a.x; F[1] = a.y; F[2] = a.z; F[3] = a.w;
-  F[4] = b.x; F[5] = b.y; F[6] = b.z; F[7] = b.w;
-  F[8] = P.F2[t];
-}
-
-__device__ __forceinline__ void load_M(const Pool& P, uint32_t t, float* M) {
-  float4 a = P.VM0[t], b = P.VM1[t], c = P.VM2[t];
-  M[0] = a.w; M[1] = b.x; M[2] = b.y; M[3] = b.z;
-  M[4] = b.w; M[5] = c.x; M[6] = c.y; M[7] = c.z; M[8] = c.w;
-}
-
-__device__ __forceinline__ void store_M(Pool& P, uint32_t t, const float* M) {
-  float4 a = P.VM0[t];
-  a.w = M[0];
-  P.VM0[t] = a;
-  P.VM1[t] = make_float4(M[1], M[2], M[3], M[4]);
-  P.VM2[t] = make_float4(M[5], M[6], M[7], M[8]);
 }
 
 __device__ __forceinline__ void lame_of(const MatDev& mt, const Pool& P, uint32_t t, float& mu, float& lam) {
@@ -1757,10 +1695,7 @@ __global__ void __launch_bounds__(256) k_read_particles(Pool P, const SceneDev* 
             Cell<KIND> cx, cy, cz;
             cx.set(ux); cy.set(uy); cz.set(uz);
             st.set(ux, uy, uz, cx.block() * 4, cy.block() * 4, cz.block() * 4);
-            float C[9];
-            mul_dinv(st, r[u], s.inv_dx * s.inv_dx, C);
-#pragma unroll
-            for (int q = 0; q < 9; ++q) r[u][q] = C[q];
+            to_rows(mul_dinv(st, from_rows(r[u]), s.inv_dx * s.inv_dx), r[u]);
           }
         }
       }
@@ -1810,9 +1745,7 @@ __global__ void k_write_particles(Pool P, const SceneDev* scenes, const MatDev* 
       float B[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
       if (!pic) recover_B(P, s, mt, t, B);
       if (field == 4) {
-        P.F0[t] = make_float4(in[9 * id], in[9 * id + 1], in[9 * id + 2], in[9 * id + 3]);
-        P.F1[t] = make_float4(in[9 * id + 4], in[9 * id + 5], in[9 * id + 6], in[9 * id + 7]);
-        P.F2[t] = in[9 * id + 8];
+        store_F(P, t, in + 9 * (size_t)id);
       } else if (P.E) {
         P.E[t] = in[id];
       }
@@ -1821,9 +1754,8 @@ __global__ void k_write_particles(Pool P, const SceneDev* scenes, const MatDev* 
       lame_of(mt, P, t, mu, lam);
       stress_of(mt, F, mu, lam, tau);
       if (P.T0) {  // m B stays; the stress term follows the new F (or E)
-        P.T0[t] = make_float4(-dtv * tau[0], -dtv * tau[1], -dtv * tau[2], -dtv * tau[3]);
-        P.T1[t] = make_float4(-dtv * tau[4], -dtv * tau[5], -dtv * tau[6], -dtv * tau[7]);
-        P.T2[t] = -dtv * tau[8];
+        for (int q = 0; q < 9; ++q) tau[q] *= -dtv;
+        store_T(P, t, tau);
       } else {
         for (int q = 0; q < 9; ++q) M[q] = mt.mass * B[q] - dtv * tau[q];
         store_M(P, t, M);
@@ -1915,8 +1847,8 @@ __global__ void k_admit(Pool P, uint32_t* key, uint32_t* cnt, uint32_t* bnd, con
     P.VM0[t] = make_float4(vx, vy, vz, 0.f);
     P.VM1[t] = make_float4(0.f, 0.f, 0.f, 0.f);
     P.VM2[t] = make_float4(0.f, 0.f, 0.f, 0.f);
-    P.F0[t] = make_float4(1.f, 0.f, 0.f, 0.f);
-    P.F1[t] = make_float4(1.f, 0.f, 0.f, 0.f);
+    P.F0[t] = make_float4(1.f, 0.f, 0.f, 1.f);
+    P.F1[t] = make_float4(0.f, 0.f, 0.f, 0.f);
     P.F2[t] = 1.f;
     P.ID[t] = i;
     if (P.E) P.E[t] = E ? E[i] : 0.f;
@@ -1927,9 +1859,9 @@ __global__ void k_admit(Pool P, uint32_t* key, uint32_t* cnt, uint32_t* bnd, con
     }
     uint32_t k = particle_key<KIND>(s, ux, uy, uz);
     key[t] = k;
-    const float M0[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    const M3 M0 = {{v3(0.f), v3(0.f), v3(0.f)}};
     float bmass, bmom;
-    p2g_bounds<KIND>(s.inv_dx, mats[m].mass, vx, vy, vz, M0, bmass, bmom);
+    p2g_bounds<KIND>(s.inv_dx, mats[m].mass, V3{pk(vx, vy), vz}, M0, bmass, bmom);
     warp_aggregated_bin(cnt, bnd, k, bmass, bmom);
   }
 }
@@ -1962,15 +1894,11 @@ __global__ void k_rekey(Pool P, uint32_t* key, uint32_t* cnt, uint32_t* bnd, con
     }
     uint32_t k = particle_key<KIND>(s, ux, uy, uz);
     key[t] = k;
-    const float4 a = P.VM0[t], b = P.VM1[t], c = P.VM2[t];
-    float M[9] = {a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w};
-    if (P.T0) {
-      const float4 t0 = P.T0[t], t1 = P.T1[t];
-      const float T[9] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w, P.T2[t]};
-      for (int q = 0; q < 9; ++q) M[q] = fabsf(M[q]) + fabsf(T[q]);
-    }
+    const float4 a = P.VM0[t];
+    M3 M = unpack_m3(P.VM1[t], P.VM2[t], a.w);
+    if (P.T0) M = abs_sum(M, unpack_m3(P.T0[t], P.T1[t], P.T2[t]));
     float bmass, bmom;
-    p2g_bounds<KIND>(s.inv_dx, mt.mass, a.x, a.y, a.z, M, bmass, bmom);
+    p2g_bounds<KIND>(s.inv_dx, mt.mass, V3{pk(a.x, a.y), a.z}, M, bmass, bmom);
     warp_aggregated_bin(cnt, bnd, k, bmass, bmom);
   }
 }
@@ -2016,9 +1944,9 @@ static void launch_all(const LaunchCfg& lc, StepView v, int which) {
   switch (which) {
     case LK_P2G:
       if (lc.transfer == 1)
-        k_p2g<KIND, 1, 1><<<lc.sm_count * 32, kP2GWarp, 0, lc.stream>>>(v);
+        k_p2g<KIND, 1, 1, KIND == 0, 1><<<lc.sm_count * 32, kP2GWarp, 0, lc.stream>>>(v);
       else if (lc.transfer == 2)
-        k_p2g<KIND, 2, 1><<<lc.sm_count * 32, kP2GWarp, 0, lc.stream>>>(v);
+        k_p2g<KIND, 2, 1, KIND == 0, 1><<<lc.sm_count * 32, kP2GWarp, 0, lc.stream>>>(v);
       else
         launch_p2g_apic<KIND>(lc, v);
       break;
