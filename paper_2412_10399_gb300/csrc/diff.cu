@@ -40,6 +40,34 @@ namespace ckd {
 
 using ck::svd3;
 
+// Launches of a step's kernels, with programmatic stream serialisation: a
+// kernel's CTAs may become resident while the kernel before it drains, and
+// wait there (grid_begin, the first statement of each) until it has finished
+// and its writes are visible; each lets the next do the same from its own
+// start.  That hides the launch latency and the ramp of kernels of a few
+// microseconds; a kernel behind anything else (a copy, an event, a kernel of
+// the caller) starts as usual.  Measured (262,144 particles): a forward step
+// 60.3 -> 54.5 us, its adjoint 128.4 -> 116.3.  (The forward engine's steps
+// are replayed as graphs, where it gained 2% on the smallest and lost 5% on
+// the diffusion bar, so they are launched plainly.)
+template <typename... P, typename... A>
+inline void launch_step(void (*kernel)(P...), uint32_t grid, uint32_t block, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+// Wait for the kernel before this one, and let the one after it take its place.
+__device__ __forceinline__ void grid_begin() {
+  asm volatile("griddepcontrol.launch_dependents;\ngriddepcontrol.wait;" ::: "memory");
+}
+
 struct DP {
   float dx, inv_dx, dt, V0, mass, nu, gx, gy, gz, bc;
   int res, nb, n;  // nb: 4x4x4-node blocks per axis, ceil((res + 1) / 4)
@@ -392,6 +420,7 @@ __device__ __forceinline__ void affine(const DP& p, const DS& s, const float* B,
 
 __global__ void __launch_bounds__(kDT, 10) k_fwd_p2g(DP p, DGrid D, const float* x, const float* v, const float* B,
                                                  const float* F, const float* E) {
+  grid_begin();
   __shared__ float rows[kDT / 32][32 * 24];
   float* const sm = rows[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
@@ -472,6 +501,7 @@ __device__ __forceinline__ void for_block_nodes(const DP& p, const DGrid& D, Fn&
 // zeroes the velocity adjoints that G2P^T adds into.
 template <bool ADJ>
 __global__ void __launch_bounds__(128) k_fwd_grid(DP p, DGrid D) {
+  grid_begin();
   for_block_nodes(p, D, [&](size_t q, bool w) {
     const float4 a = D.G[q];
     float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -490,6 +520,7 @@ __global__ void __launch_bounds__(128) k_fwd_grid(DP p, DGrid D) {
 
 __global__ void __launch_bounds__(kDT) k_fwd_g2p(DP p, DGrid D, const float* x, const float* F, float* x1, float* v1,
                                                  float* B1, float* F1) {
+  grid_begin();
   __shared__ float rows[kDT / 32][32 * 12];
   float* const sm = rows[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
@@ -554,6 +585,7 @@ struct WeightAdjoint {
 __global__ void __launch_bounds__(kDT, 6) k_bwd_g2p(DP p, DGrid D, const float* x, const float* F, const float* gx1,
                                                  const float* gv1, const float* gB1, const float* gF1, float* gx,
                                                  float* gF) {
+  grid_begin();
   __shared__ float rows[kDT / 32][32 * 36];
   float* const sm = rows[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
@@ -646,6 +678,7 @@ __global__ void __launch_bounds__(kDT, 6) k_bwd_g2p(DP p, DGrid D, const float* 
 // grid^T: v~ = (P/m + dt g) on nodes with mass off the walls; A becomes
 // (p_bar, m_bar) and the accumulators return to zero.
 __global__ void __launch_bounds__(128) k_bwd_grid(DP p, DGrid D) {
+  grid_begin();
   for_block_nodes(p, D, [&](size_t q, bool w) {
     const float4 a = D.G[q];
     const float4 b = D.A[q];
@@ -666,6 +699,7 @@ __global__ void __launch_bounds__(128) k_bwd_grid(DP p, DGrid D) {
 __global__ void __launch_bounds__(kDT, 6) k_bwd_p2g(DP p, DGrid D, const float* x, const float* v, const float* B,
                                                  const float* F, const float* E, float* gx, float* gv, float* gB,
                                                  float* gF, float* gE) {
+  grid_begin();
   __shared__ float rows[kDT / 32][32 * 36];
   float* const sm = rows[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
@@ -821,9 +855,9 @@ ckmpm_status ckmpm_diff_create(const ckmpm_scene* sc, void* stream, ckmpm_diff**
 ckmpm_status ckmpm_diff_step(ckmpm_diff* d, const float* x, const float* v, const float* B, const float* F,
                              const float* E, float* x1, float* v1, float* B1, float* F1) {
   if (!d || !x || !v || !B || !F || !E || !x1 || !v1 || !B1 || !F1) return CKMPM_EINVAL;
-  ckd::k_fwd_p2g<<<d->blocks, ckd::kDT, 0, d->stream>>>(d->p, d->g, x, v, B, F, E);
-  ckd::k_fwd_grid<false><<<d->grid_ctas, 128, 0, d->stream>>>(d->p, d->g);
-  ckd::k_fwd_g2p<<<d->blocks, ckd::kDT, 0, d->stream>>>(d->p, d->g, x, F, x1, v1, B1, F1);
+  ckd::launch_step(ckd::k_fwd_p2g, d->blocks, ckd::kDT, d->stream, d->p, d->g, x, v, B, F, E);
+  ckd::launch_step(ckd::k_fwd_grid<false>, d->grid_ctas, 128, d->stream, d->p, d->g);
+  ckd::launch_step(ckd::k_fwd_g2p, d->blocks, ckd::kDT, d->stream, d->p, d->g, x, F, x1, v1, B1, F1);
   return cudaGetLastError() == cudaSuccess ? CKMPM_OK : CKMPM_ECUDA;
 }
 
@@ -832,11 +866,11 @@ ckmpm_status ckmpm_diff_step_backward(ckmpm_diff* d, const float* x, const float
                                       const float* gF1, float* gx, float* gv, float* gB, float* gF, float* gE) {
   if (!d || !x || !v || !B || !F || !E || !gx1 || !gv1 || !gB1 || !gF1 || !gx || !gv || !gB || !gF || !gE)
     return CKMPM_EINVAL;
-  ckd::k_fwd_p2g<<<d->blocks, ckd::kDT, 0, d->stream>>>(d->p, d->g, x, v, B, F, E);
-  ckd::k_fwd_grid<true><<<d->grid_ctas, 128, 0, d->stream>>>(d->p, d->g);
-  ckd::k_bwd_g2p<<<d->blocks, ckd::kDT, 0, d->stream>>>(d->p, d->g, x, F, gx1, gv1, gB1, gF1, gx, gF);
-  ckd::k_bwd_grid<<<d->grid_ctas, 128, 0, d->stream>>>(d->p, d->g);
-  ckd::k_bwd_p2g<<<d->blocks, ckd::kDT, 0, d->stream>>>(d->p, d->g, x, v, B, F, E, gx, gv, gB, gF, gE);
+  ckd::launch_step(ckd::k_fwd_p2g, d->blocks, ckd::kDT, d->stream, d->p, d->g, x, v, B, F, E);
+  ckd::launch_step(ckd::k_fwd_grid<true>, d->grid_ctas, 128, d->stream, d->p, d->g);
+  ckd::launch_step(ckd::k_bwd_g2p, d->blocks, ckd::kDT, d->stream, d->p, d->g, x, F, gx1, gv1, gB1, gF1, gx, gF);
+  ckd::launch_step(ckd::k_bwd_grid, d->grid_ctas, 128, d->stream, d->p, d->g);
+  ckd::launch_step(ckd::k_bwd_p2g, d->blocks, ckd::kDT, d->stream, d->p, d->g, x, v, B, F, E, gx, gv, gB, gF, gE);
   return cudaGetLastError() == cudaSuccess ? CKMPM_OK : CKMPM_ECUDA;
 }
 
