@@ -14,8 +14,9 @@
 // gathers them back to the particles; weights, offsets and D depend on x and
 // are differentiated in closed form (K1 is C^2, so dK1 is continuous).  The
 // stress adjoint goes through the polar decomposition F = R S with
-// dR = R Omega, Omega S + S Omega = R^T dF - dF^T R, whose (sigma_i + sigma_j)
-// denominators stay well conditioned when singular values coincide.
+// dR = R Omega, Omega S + S Omega = R^T dF - dF^T R: a 3x3 system in the axial
+// vector of Omega whose determinant, the product of the sigma_i + sigma_j,
+// stays well conditioned when singular values coincide.
 //
 // Grid layout and its upkeep.  A node holds one float4 (m, P), (v~, 0) or
 // (p_bar, m_bar), so that a scatter is one 16-byte vector reduction per node
@@ -335,21 +336,96 @@ __device__ __forceinline__ void lame(const DP& p, float E, float& mu, float& lam
   lam = E * p.nu / ((1.0f + p.nu) * (1.0f - 2.0f * p.nu));
 }
 
-// tau = 2 mu (F - R) F^T + lam J (J - 1) I
-__device__ __forceinline__ void fc_stress(const float* F, float mu, float lam, float* tau, float* U, float* sig, float* V) {
+// Rotation of the polar decomposition F = R S.  For det F well above zero by
+// Newton's iteration R <- (R + R^-T) / 2 (Higham, "Computing the polar
+// decomposition -- with applications", 1986), R^-T = cof(R) / det R: it
+// converges quadratically, an update of size d leaving an error of d^2 / 2, so
+// it stops after an update below 2^-12.  Elastic strains of some per cent take
+// three to four rounds of about 35 instructions, where the singular value
+// decomposition takes some 600; P2G and P2G^T need nothing else of it.
+// Degenerate or inverted F goes through the decomposition (det R = +1).
+__device__ __noinline__ void rotation_by_svd(const float* F, float* R) {
+  float U[9], V[9], sig[3];
   svd3<float>(F, U, sig, V);
-  ck::fc_tau<float>(F, U, sig, V, mu, lam, tau);
+  mat3_bt(U, V, R);
+}
+
+__device__ __forceinline__ void cofactor(const float* F, float* C) {
+  C[0] = F[4] * F[8] - F[5] * F[7];
+  C[1] = F[5] * F[6] - F[3] * F[8];
+  C[2] = F[3] * F[7] - F[4] * F[6];
+  C[3] = F[2] * F[7] - F[1] * F[8];
+  C[4] = F[0] * F[8] - F[2] * F[6];
+  C[5] = F[1] * F[6] - F[0] * F[7];
+  C[6] = F[1] * F[5] - F[2] * F[4];
+  C[7] = F[2] * F[3] - F[0] * F[5];
+  C[8] = F[0] * F[4] - F[1] * F[3];
+}
+
+// R of F, and cof(F) and J = det F
+__device__ __forceinline__ void rotation(const float* F, float* R, float* cof, float& J) {
+  cofactor(F, cof);
+  J = F[0] * cof[0] + F[1] * cof[1] + F[2] * cof[2];
+  bool ok = false;
+  if (J > 0.05f) {
+    float C[9], det = J;
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+      R[q] = F[q];
+      C[q] = cof[q];
+    }
+#pragma unroll 1
+    for (int it = 0; it < 10; ++it) {
+      const float h = 0.5f / det;
+      float d2 = 0.f;
+#pragma unroll
+      for (int q = 0; q < 9; ++q) {
+        const float n = fmaf(h, C[q], 0.5f * R[q]), d = n - R[q];
+        R[q] = n;
+        d2 = fmaf(d, d, d2);
+      }
+      if (d2 < 5.9604645e-8f) {  // (2^-12)^2
+        ok = true;
+        break;
+      }
+      cofactor(R, C);
+      det = R[0] * C[0] + R[1] * C[1] + R[2] * C[2];
+    }
+  }
+  if (!ok) {
+    float Ft[9], Rt[9];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) Ft[q] = F[q];
+    rotation_by_svd(Ft, Rt);
+#pragma unroll
+    for (int q = 0; q < 9; ++q) R[q] = Rt[q];
+  }
+}
+
+// tau = 2 mu (F - R) F^T + lam J (J - 1) I
+__device__ __forceinline__ void fc_stress(const float* F, const float* R, float J, float mu, float lam, float* tau) {
+  float D[9];
+#pragma unroll
+  for (int q = 0; q < 9; ++q) D[q] = F[q] - R[q];
+  mat3_bt(D, F, tau);
+  const float vol = lam * J * (J - 1.0f);
+#pragma unroll
+  for (int q = 0; q < 9; ++q) tau[q] = 2.0f * mu * tau[q] + (q % 4 == 0 ? vol : 0.0f);
+}
+
+// m(M) with M - M^T = [m]x
+__device__ __forceinline__ void axial(const float* M, float* m) {
+  m[0] = M[7] - M[5];
+  m[1] = M[2] - M[6];
+  m[2] = M[3] - M[1];
 }
 
 // Adjoint of tau(F; E) for the fixed-corotated model: F_bar += d tau/dF ^T : tb,
-// E_bar += <tb, tau> / E (tau is proportional to E at fixed F).
-// (tau and its decomposition F = U diag(sig) V^T come from fc_stress.)
-__device__ __forceinline__ void fc_stress_vjp(const float* F, float E, float mu, float lam, const float* tau,
-                                              const float* U, const float* sig, const float* V, const float* tb,
-                                              float* Fb, float& Eb) {
-  float R[9];
-  mat3_bt(U, V, R);
-  float J = sig[0] * sig[1] * sig[2];
+// E_bar += <tb, tau> / E (tau is proportional to E at fixed F).  (tau, R,
+// cof F and J come from fc_stress and rotation.)
+__device__ __forceinline__ void fc_stress_vjp(const float* F, const float* R, const float* cof, float J, float E,
+                                              float mu, float lam, const float* tau, const float* tb, float* Fb,
+                                              float& Eb) {
   float G[9];
 #pragma unroll
   for (int q = 0; q < 9; ++q) G[q] = F[q] - R[q];
@@ -360,34 +436,35 @@ __device__ __forceinline__ void fc_stress_vjp(const float* F, float E, float mu,
 #pragma unroll
   for (int q = 0; q < 9; ++q) Fb[q] += 2.0f * mu * (t1[q] + t2[q]);
   // lam (2J - 1) tr(tb) cof(F)
-  float tr = tb[0] + tb[4] + tb[8];
-  float cof[9] = {F[4] * F[8] - F[5] * F[7], F[5] * F[6] - F[3] * F[8], F[3] * F[7] - F[4] * F[6],
-                  F[2] * F[7] - F[1] * F[8], F[0] * F[8] - F[2] * F[6], F[1] * F[6] - F[0] * F[7],
-                  F[1] * F[5] - F[2] * F[4], F[2] * F[3] - F[0] * F[5], F[0] * F[4] - F[1] * F[3]};
-  float kv = lam * (2.0f * J - 1.0f) * tr;
+  const float kv = lam * (2.0f * J - 1.0f) * (tb[0] + tb[4] + tb[8]);
 #pragma unroll
   for (int q = 0; q < 9; ++q) Fb[q] += kv * cof[q];
-  // R_bar = -2 mu tb F ; F_bar += 2 U Z V^T, Z_ij = skew(U^T R_bar V)_ij / (sig_i + sig_j)
-  float Rb[9];
+  // R_bar = -2 mu tb F.  dR = R [w]x with Omega S + S Omega = R^T dF - dF^T R,
+  // Omega = [w]x, i.e. K w = m(R^T dF), K = tr(S) I - S; so <R_bar, dR> =
+  // m(R^T R_bar) . w = z . m(R^T dF) with K z = m(R^T R_bar), and F_bar += R [z]x.
+  // det K = prod (sigma_i + sigma_j).
+  float S[9], N[9], m[3];
+  mat3_at(R, F, S);
+  mat3_at(R, t1, N);
+  axial(N, m);
+  const float tr = S[0] + S[4] + S[8];
+  const float s01 = 0.5f * (S[1] + S[3]), s02 = 0.5f * (S[2] + S[6]), s12 = 0.5f * (S[5] + S[7]);
+  const float K[9] = {tr - S[0], -s01, -s02, -s01, tr - S[4], -s12, -s02, -s12, tr - S[8]};
+  float C[9];
+  cofactor(K, C);
+  // (K's eigenvalues are the sigma_i + sigma_j >= 0: at least 1e-6 each, by
+  // the sum of their products)
+  const float det = fmaxf(K[0] * C[0] + K[1] * C[1] + K[2] * C[2], fmaf(1e-6f, C[0] + C[4] + C[8], 1e-18f));
+  const float h = -2.0f * mu / det;
+  float z[3];
 #pragma unroll
-  for (int q = 0; q < 9; ++q) Rb[q] = -2.0f * mu * t1[q];
-  float T[9], A[9];
-  mat3_at(U, Rb, T);
-  mat3(T, V, A);
-  float Z[9];
+  for (int i = 0; i < 3; ++i) z[i] = h * (C[3 * i] * m[0] + C[3 * i + 1] * m[1] + C[3 * i + 2] * m[2]);
 #pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      float den = sig[i] + sig[j];
-      den = fabsf(den) < 1e-6f ? (den < 0.f ? -1e-6f : 1e-6f) : den;
-      Z[i * 3 + j] = (i == j) ? 0.0f : 0.5f * (A[i * 3 + j] - A[j * 3 + i]) / den;
-    }
-  float UZ[9], UZV[9];
-  mat3(U, Z, UZ);
-  mat3_bt(UZ, V, UZV);
-#pragma unroll
-  for (int q = 0; q < 9; ++q) Fb[q] += 2.0f * UZV[q];
+  for (int i = 0; i < 3; ++i) {
+    Fb[3 * i] += R[3 * i + 1] * z[2] - R[3 * i + 2] * z[1];
+    Fb[3 * i + 1] += R[3 * i + 2] * z[0] - R[3 * i] * z[2];
+    Fb[3 * i + 2] += R[3 * i] * z[1] - R[3 * i + 1] * z[0];
+  }
   float dot = 0.f;
 #pragma unroll
   for (int q = 0; q < 9; ++q) dot += tb[q] * tau[q];
@@ -445,9 +522,10 @@ __global__ void __launch_bounds__(kDT, 10) k_fwd_p2g(DP p, DGrid D, const float*
     if (lane < cnt) atomicOr(D.err, 1u);
     return;
   }
-  float tau[9], U[9], V[9], sig[3], mu, lam, M[9], A[9];
+  float tau[9], R[9], cof[9], J, mu, lam, M[9], A[9];
   lame(p, E[p0 + lane], mu, lam);
-  fc_stress(Fi, mu, lam, tau, U, sig, V);
+  rotation(Fi, R, cof, J);
+  fc_stress(Fi, R, J, mu, lam, tau);
   affine(p, s, Bi, tau, M, A);
   const float mv[3] = {p.mass * vi[0], p.mass * vi[1], p.mass * vi[2]};
 #pragma unroll
@@ -724,10 +802,11 @@ __global__ void __launch_bounds__(kDT, 6) k_bwd_p2g(DP p, DGrid D, const float* 
   DS s;
   s.set(p, xi[0], xi[1], xi[2]);
   if (lane < cnt && nodes_in_range(p, s)) {
-    float tau[9], U[9], V[9], sig[3], mu, lam, M[9], A[9];
+    float tau[9], R[9], cof[9], J, mu, lam, M[9], A[9];
     const float Ei = E[p0 + lane];
     lame(p, Ei, mu, lam);
-    fc_stress(Fi, mu, lam, tau, U, sig, V);
+    rotation(Fi, R, cof, J);
+    fc_stress(Fi, R, J, mu, lam, tau);
     affine(p, s, Bi, tau, M, A);
     const float mv[3] = {p.mass * vi[0], p.mass * vi[1], p.mass * vi[2]};
     // S = sum w p_bar, Ab = sum w p_bar d^T; a node's contribution
@@ -778,7 +857,7 @@ __global__ void __launch_bounds__(kDT, 6) k_bwd_p2g(DP p, DGrid D, const float* 
       tb[q] = -p.dt * p.V0 * Mb[q];
       Mb[q] *= p.mass;
     }
-    fc_stress_vjp(Fi, Ei, mu, lam, tau, U, sig, V, tb, Fb, Eb);
+    fc_stress_vjp(Fi, R, cof, J, Ei, mu, lam, tau, tb, Fb, Eb);
 #pragma unroll
     for (int a = 0; a < 3; ++a) vb[a] = p.mass * S[a];
     gE[p0 + lane] += Eb;
