@@ -170,8 +170,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_final(StepView v, BinScra
   if (blockIdx.x == 0 && threadIdx.x == 0) {  // the step's counters
     *v.n_g = 0u;
     *v.fp64_count = 0ull;
-    v.work[0] = 0u;
-    v.work[1] = 0u;
+    v.work[0] = v.work0[0];
+    v.work[1] = v.work0[1];
     if (v.lo_count) *v.lo_count = 0u;
   }
   if (blockIdx.x == gridDim.x - 1 && threadIdx.x == kScanThreads - 1) {

@@ -81,6 +81,21 @@ struct Pool {
   float* T2;
 };
 
+// Work units of a transfer kernel: `splits` parts of every particle block, of
+// `unit` particles each (a block that holds more than splits * unit is cut into
+// equal parts; the last parts of a thin one are empty).
+struct Units {
+  uint32_t splits, unit;
+};
+enum { kUnitsP2G = 0, kUnitsG2P = 1 };
+// The parts a step of npb blocks uses: no more than give `most` units, so that
+// a body spread over many thin blocks does not pay for parts without
+// particles (a part then takes more than `unit`).
+__device__ __forceinline__ Units limit_units(Units w, uint32_t npb, uint32_t most) {
+  w.splits = min(w.splits, max(1u, (most + npb - 1u) / max(npb, 1u)));
+  return w;
+}
+
 // Everything the per-step kernels read; passed by value.
 struct StepView {
   Pool cur, nxt;
@@ -116,7 +131,9 @@ struct StepView {
   uint32_t n_keys;      // size of the key space
   uint32_t n_cur;       // particles in cur (including dead ones)
   uint32_t keep_gacc;   // probe: the grid update leaves Gacc, P2G keeps bnd_cur
-  uint32_t splits;      // work units per particle block of the transfer kernels (>= 1)
+  Units units[2];       // work units of P2G and of G2P
+  uint32_t work0[2];    // what the scan sets work[] to: the CTAs of a step of split blocks, else 0
+  uint32_t unit_most;   // limit_units' bound (32 per SM)
   uint32_t n_mats;      // entries of the material table
   // fused G2P2G step only (else null): the block table of the next step's
   // grid (the gather reads Gvel through `table`, the scatter adds to Gacc
@@ -132,40 +149,47 @@ struct StepView {
 
 __device__ __forceinline__ void flag_error(uint32_t* err, uint32_t bit) { atomicOr(err, bit); }
 
-// Work unit u of the transfer kernels: particle block u / splits, part
-// u % splits of its particles, in whole chunks of `align` particles (a step
-// with few blocks splits each over several units so that every resident
-// warp gets work).  A block's entries are three independent loads: its key
-// and first slot, the next block's first slot, its scene.
 struct Unit {
   uint32_t key, scene, start, cnt;  // the block
   uint32_t lo, hi;                  // the unit's particles: [lo, hi) of [0, cnt)
 };
 
-// Returns false when the part is empty.
-__device__ __forceinline__ bool unit_of(const StepView& v, uint32_t u, uint32_t align, Unit& q) {
-  const uint32_t S = v.splits;
-  const uint32_t bi = u / S, part = u - bi * S;
+// Unit u: block u / splits, part u % splits, in whole chunks of ALIGN
+// particles; false when the part is empty.  A block's entries are three
+// independent loads: its key and first slot, the next block's first slot, its
+// scene.
+template <uint32_t ALIGN, bool SPLIT = true>
+__device__ __forceinline__ bool unit_of(const StepView& v, const Units& w, uint32_t u, Unit& q) {
+  const uint32_t bi = SPLIT ? u / w.splits : u, part = SPLIT ? u - bi * w.splits : 0u;
   const uint2 b = v.pb[bi];
   const uint32_t end = v.pb[bi + 1].y;
   q.scene = v.pb_scene[bi];
   q.key = b.x;
   q.start = b.y;
   q.cnt = end - b.y;
-  const uint32_t per = ((q.cnt + S - 1) / S + align - 1) / align * align;
+  if (!SPLIT) {
+    q.lo = 0u;
+    q.hi = q.cnt;
+    return true;  // listed blocks hold particles
+  }
+  const uint32_t per = max(w.unit, ((q.cnt + w.splits - 1) / w.splits + ALIGN - 1) / ALIGN * ALIGN);
   q.lo = part * per;
   q.hi = min(q.cnt, q.lo + per);
   return q.lo < q.hi;
 }
 
-// The next unit of a persistent one-warp CTA: one at a time from the step's
-// counter.
+// Unit schedule of a persistent one-warp CTA.  Units come one at a time from
+// the step's counter; a few thousand CTAs asking one address at once are
+// served one after the other (about 3 ns each), so in a step of split blocks
+// the first unit is the CTA's own index.  A step of whole blocks keeps that
+// first queue: it staggers the CTAs, which otherwise gather and compute in
+// step (G2P of 16.27 M particles 0.64 -> 0.67 ms).
+// (The scan starts the counter at the number of CTAs then: work0.)
 __device__ __forceinline__ uint32_t next_unit(uint32_t* work) {
   uint32_t u = 0;
   if (threadIdx.x == 0) u = atomicAdd(work, 1u);
   return __shfl_sync(0xffffffffu, u, 0);
 }
-
 // Cell decomposition shared by every kernel that maps a position to nodes.
 // u0 = x/dx.  CK: t = u0 + 1/4, b+ = floor(t), f+ = t - b+ (exact when dx is a
 // power of two), b- = b+ or b+ - 1 with f- = f+ -+ 1/2 (Sec. 4.2 offsets).

@@ -108,7 +108,7 @@ struct ckmpm_ctx {
   // fused G2P2G steps: a second block-table set for the next step's grid,
   // which one maps the current grid velocities, and whether they are current
   bool fused = false;
-  int splits_override = 0;  // CKMPM_SPLITS: work units per block (else chosen from the particle count)
+  int splits_override = 0;  // CKMPM_SPLITS: work units per block (else step_units' rule)
   // steady-state steps replayed as CUDA graphs, one per parity of the
   // double-buffered state (particle buffer cur, plus table set tsel for
   // fused steps); dropped whenever the launch sequence or its arguments change
@@ -272,16 +272,18 @@ ck::StepView make_view(ckmpm_ctx* ctx) {
     v.tile_ne = ctx->tile_ne;
   }
   v.keep_gacc = 0;
-  // a step with few particles splits each block over several work units, so
-  // that the resident warps of the transfer kernels (about 20 per SM) get two
-  // units of a few hundred particles each; large steps keep whole blocks
-  {
-    int64_t n_live = 0;
-    for (auto& s : ctx->scenes) n_live += s.alive ? s.n : 0;
-    const int64_t target = (int64_t)ctx->sm_count * 20 * 2 * 512;
-    v.splits = (uint32_t)std::max<int64_t>(1, std::min<int64_t>(8, target / std::max<int64_t>(n_live, 1)));
-    if (ctx->splits_override > 0) v.splits = (uint32_t)ctx->splits_override;
+  int64_t n_live = 0;
+  for (auto& s : ctx->scenes) n_live += s.alive ? s.n : 0;
+  const ck::LaunchCfg& lc = ctx->lc;
+  const int warps[2] = {ck::p2g_warps(ctx->kind, lc.transfer, lc.p2g_rep),
+                        ctx->fused ? ck::fused_warps(ctx->kind) : ck::g2p_warps(ctx->kind, lc.transfer, lc.g2p_minb)};
+  for (int k = 0; k < 2; ++k) {
+    v.units[k] = ck::step_units(k, n_live, ctx->sm_count, warps[k]);
+    if (ctx->splits_override > 0) v.units[k] = {(uint32_t)ctx->splits_override, 0u};
+    // split blocks: the first units are the CTAs' own, the counter starts behind them
+    v.work0[k] = v.units[k].splits > 1 ? (uint32_t)(ctx->sm_count * warps[k]) : 0u;
   }
+  v.unit_most = ck::p2g_ctas(ctx->sm_count);
   if (ctx->fused) {  // binning zeroes the leftover count every step
     v.lo_list = ctx->lo_list;
     v.lo_count = ctx->counters + 9;

@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "common.cuh"
@@ -18,6 +19,46 @@ struct LaunchCfg {
   int p2g_rot = 0;      // one copy: components in the lane-rotated order (1) or in order (0)
   int p2g_fma = 0;      // APIC + MLS: fused-multiply-add rounding in blocks of >= 256 particles (1)
 };
+
+// One-warp CTAs per SM of the transfer kernels.  P2G of whole blocks launches
+// more than fit (they take units until none is left); split blocks, where a
+// CTA's first unit is its index, take one resident wave: what shared memory
+// or registers leave room for (rep: copies of the APIC + MLS accumulators).
+constexpr int p2g_warps(int kind, int transfer, int rep) {
+  if (transfer == 2) return kind == 0 ? 14 : 12;
+  if (transfer == 0 && rep == 2) return kind == 0 ? 12 : 16;
+  return kind == 1 && transfer == 1 ? 16 : 18;
+}
+inline uint32_t p2g_ctas(int sm_count) { return (uint32_t)sm_count * 32u; }
+// G2P and the fused kernel: one resident wave at their register budgets
+constexpr int fused_warps(int kind) { return kind == 0 ? 20 : 16; }
+inline int g2p_warps(int kind, int transfer, int minb) {
+  if (transfer == 1) return kind == 0 ? 20 : 16;
+  if (transfer == 2) return kind == 0 ? 16 : 12;
+  return 4 * minb;
+}
+
+// Units of a step of n particles for a kernel of that many warps per SM.  A
+// step with a full block of 512 for every G2P warp (20 per SM) keeps whole
+// blocks, because a unit costs a warp several microseconds of its own (its
+// chain of dependent loads, the staged nodes, a partly filled last chunk).  A
+// smaller one is cut so that full blocks give about one unit per warp, in
+// whole chunks; P2G, where a unit also clears and flushes its nodes, into no
+// less than two chunks of 96 unless the step has not a G2P chunk per warp.
+// Measured, P2G / G2P us on the granular column (346,112 particles, compact
+// kernel): units of 96 24.9 / 29.4, 128 27.3 / 24.0, 192 20.6 / 26.9, 256
+// 21.0 / 26.6; on the diffusion bar (224,000, PIC): 21.1 / 24.6, 20.6 / 29.2,
+// 16.9 / 31.0, 21.1 / 39.7; on a sand box of 592,704 (with the events' 6 us),
+// P2G in parts of 192 39.5, of 256 32.7.
+inline Units step_units(int which, int64_t n, int sm_count, int warps) {
+  const int64_t sm = sm_count, block = 512;
+  if (n >= sm * 20 * block) return Units{1u, (uint32_t)block};
+  const int64_t want = std::max<int64_t>(2, std::min<int64_t>(16, sm * warps * block / std::max<int64_t>(n, 1)));
+  const int64_t chunk = which == kUnitsP2G ? 96 : 32;
+  int64_t unit = ((block + want - 1) / want + chunk - 1) / chunk * chunk;
+  if (which == kUnitsP2G && n >= sm * 20 * 32) unit = std::max<int64_t>(192, unit);
+  return Units{(uint32_t)((block + unit - 1) / unit), (uint32_t)unit};
+}
 
 enum { LK_P2G = 0, LK_UPDATE = 1, LK_G2P = 2, LK_CLEAR = 3, LK_G2P_FP64 = 4, LK_G2P2G = 5, LK_LEFTOVER = 6 };
 

@@ -703,13 +703,24 @@ struct P2GRep {
   static constexpr int stride = REP == 1 ? 4 * NS : ((4 * NS + 15) / 32) * 32 + 16;  // ints per copy
 };
 
+// CTAs per SM that P2G's registers leave room for: what its shared memory
+// allows, or fewer where that would spill (left to itself the compiler took up
+// to 186 registers for the twin's 27 unrolled nodes: 32.8 us instead of 26.9
+// on the granular column).
+constexpr int p2g_min_ctas(int kind, int tr, int rep) {
+  return tr == 2 ? (kind == 0 ? 16 : 12) : rep == 2 || (kind == 1 && tr == 1) ? 16 : 20;
+}
+
 // TR: transfer, 0 APIC + MLS, 1 PIC, 2 APIC with the kernel gradient.
 // ROT (one copy): components issued in the lane-rotated order of p2g_scatter,
 // planes kP2GRotPlane apart.  FMA: blocks of at least kP2GFmaCount particles
 // round their contributions by p2g_add2's multiply-add instead of a
 // conversion.
-template <int KIND, int TR, int REP, int ROT = 0, int FMA = 0>
-__global__ void __launch_bounds__(kP2GWarp) k_p2g(StepView v) {
+// SPLIT: blocks in parts; the form for whole blocks (a large step) is kept
+// apart, because the units' arithmetic showed in it (16.27 M particles: 0.497
+// against 0.491 ms here, 0.585 against 0.576 in G2P).
+template <int KIND, int TR, int REP, int ROT, int FMA, bool SPLIT>
+__global__ void __launch_bounds__(kP2GWarp, p2g_min_ctas(KIND, TR, REP)) k_p2g(StepView v) {
   constexpr int NS = Geo<KIND>::NS;
   static_assert(ROT == 0 || REP == 1, "the rotated order takes one copy");
   constexpr int PL = ROT ? P2GRotPlane<KIND>::value : NS;  // plane stride of the components
@@ -727,12 +738,14 @@ __global__ void __launch_bounds__(kP2GWarp) k_p2g(StepView v) {
   __shared__ float4 sT0[TCAP], sT1[TCAP];
   __shared__ float sT2[TCAP];
   __shared__ uint32_t bslot[8];
-  const uint32_t nunits = *v.n_pb * v.splits;
   const uint32_t lane = threadIdx.x;
   // dynamic scheduling: one work unit (a block or a part of one) at a time
-  for (uint32_t u = next_unit(&v.work[0]); u < nunits; u = next_unit(&v.work[0])) {
+  const uint32_t npb = *v.n_pb;
+  const Units units = SPLIT ? limit_units(v.units[kUnitsP2G], npb, v.unit_most) : Units{1u, 0u};
+  const uint32_t nunits = npb * units.splits;
+  for (uint32_t u = SPLIT ? blockIdx.x : next_unit(&v.work[0]); u < nunits; u = next_unit(&v.work[0])) {
     Unit q;
-    if (!unit_of(v, u, CAP, q)) continue;
+    if (!unit_of<CAP, SPLIT>(v, units, u, q)) continue;
     const uint32_t key = q.key, start = q.start, cnt = q.cnt, lo = q.lo, hi = q.hi;
     const SceneDev s = v.scenes[q.scene];
     // the block's largest contribution bounds, recorded when its particles
@@ -1136,7 +1149,8 @@ __device__ __forceinline__ bool g2p_particle(const StepView& v, const SceneStep*
 // spill store waited for the load).
 
 // TR: transfer, 0 APIC + MLS, 1 PIC, 2 APIC with the kernel gradient.
-template <int KIND, int MINB, int TR>
+// SPLIT as in k_p2g.
+template <int KIND, int MINB, int TR, bool SPLIT>
 __global__ void __launch_bounds__(kG2PWarp, 4 * MINB) k_g2p(StepView v) {
   constexpr int NS = Geo<KIND>::NS;
   constexpr int CH = 32;
@@ -1161,10 +1175,12 @@ __global__ void __launch_bounds__(kG2PWarp, 4 * MINB) k_g2p(StepView v) {
     for (uint32_t w = lane; w < words; w += CH) dst[w] = src[w];
   }
   __syncwarp();
-  const uint32_t nunits = *v.n_pb * v.splits;
-  for (uint32_t u = next_unit(&v.work[1]); u < nunits; u = next_unit(&v.work[1])) {
+  const uint32_t npb = *v.n_pb;
+  const Units units = SPLIT ? limit_units(v.units[kUnitsG2P], npb, v.unit_most) : Units{1u, 0u};
+  const uint32_t nunits = npb * units.splits;
+  for (uint32_t u = SPLIT ? blockIdx.x : next_unit(&v.work[1]); u < nunits; u = next_unit(&v.work[1])) {
     Unit q;
-    if (!unit_of(v, u, CH, q)) continue;
+    if (!unit_of<32, SPLIT>(v, units, u, q)) continue;
     const uint32_t key = q.key, start = q.start, lo = q.lo, hi = q.hi;
     const SceneDev& s = v.scenes[q.scene];
     if (lane == 0) sstep.set(s);
@@ -1300,11 +1316,14 @@ __global__ void __launch_bounds__(kG2PWarp, 4 * MINB) k_g2p2g(StepView v) {
   __shared__ SceneStep sstep;
   auto& p1 = *reinterpret_cast<typename SM::Ph1*>(arena);
   auto& p2 = *reinterpret_cast<typename SM::Ph2*>(arena);
-  const uint32_t nunits = *v.n_pb * v.splits;
   const uint32_t lane = threadIdx.x;
-  for (uint32_t u = next_unit(&v.work[1]); u < nunits; u = next_unit(&v.work[1])) {
+  const uint32_t npb = *v.n_pb;
+  const bool split = v.units[kUnitsG2P].splits > 1u;
+  const Units units = limit_units(v.units[kUnitsG2P], npb, v.unit_most);
+  const uint32_t nunits = npb * units.splits;
+  for (uint32_t u = split ? blockIdx.x : next_unit(&v.work[1]); u < nunits; u = next_unit(&v.work[1])) {
     Unit q;
-    if (!unit_of(v, u, CAP, q)) continue;
+    if (!unit_of<32>(v, units, u, q)) continue;
     const uint32_t key = q.key, start = q.start, lo = q.lo, hi = q.hi;
     const SceneDev s = v.scenes[q.scene];
     const bool track = hi - lo <= (uint32_t)kFuseMaxCnt;
@@ -1905,26 +1924,33 @@ __global__ void k_rekey(Pool P, uint32_t* key, uint32_t* cnt, uint32_t* bnd, con
 
 // ------------------------------------------------------------ host launchers
 
+template <int KIND, int TR, int REP, int ROT, int FMA>
+static void launch_p2g(const LaunchCfg& lc, const StepView& v) {
+  if (v.units[kUnitsP2G].splits > 1u)
+    k_p2g<KIND, TR, REP, ROT, FMA, true><<<v.work0[kUnitsP2G], kP2GWarp, 0, lc.stream>>>(v);
+  else
+    k_p2g<KIND, TR, REP, ROT, FMA, false><<<p2g_ctas(lc.sm_count), kP2GWarp, 0, lc.stream>>>(v);
+}
+
 // P2G of the APIC + MLS transfer: accumulator copies, component order and
 // rounding as the launch configuration asks.
 template <int KIND>
-static void launch_p2g_apic(const LaunchCfg& lc, StepView v) {
-  const int g = lc.sm_count * 32;
+static void launch_p2g_apic(const LaunchCfg& lc, const StepView& v) {
   if (lc.p2g_rep == 2) {
     if (lc.p2g_fma)
-      k_p2g<KIND, 0, 2, 0, 1><<<g, kP2GWarp, 0, lc.stream>>>(v);
+      launch_p2g<KIND, 0, 2, 0, 1>(lc, v);
     else
-      k_p2g<KIND, 0, 2, 0, 0><<<g, kP2GWarp, 0, lc.stream>>>(v);
+      launch_p2g<KIND, 0, 2, 0, 0>(lc, v);
   } else if (lc.p2g_rot) {
     if (lc.p2g_fma)
-      k_p2g<KIND, 0, 1, 1, 1><<<g, kP2GWarp, 0, lc.stream>>>(v);
+      launch_p2g<KIND, 0, 1, 1, 1>(lc, v);
     else
-      k_p2g<KIND, 0, 1, 1, 0><<<g, kP2GWarp, 0, lc.stream>>>(v);
+      launch_p2g<KIND, 0, 1, 1, 0>(lc, v);
   } else {
     if (lc.p2g_fma)
-      k_p2g<KIND, 0, 1, 0, 1><<<g, kP2GWarp, 0, lc.stream>>>(v);
+      launch_p2g<KIND, 0, 1, 0, 1>(lc, v);
     else
-      k_p2g<KIND, 0, 1, 0, 0><<<g, kP2GWarp, 0, lc.stream>>>(v);
+      launch_p2g<KIND, 0, 1, 0, 0>(lc, v);
   }
 }
 
@@ -1939,14 +1965,22 @@ static int update_ctas(const LaunchCfg& lc, const StepView& v) {
   return (int)std::max((uint32_t)lc.sm_count * 4u, std::min((uint32_t)lc.sm_count * 64u, est));
 }
 
+template <int KIND, int MINB, int TR>
+static void launch_g2p(const LaunchCfg& lc, const StepView& v, uint32_t g) {
+  if (v.units[kUnitsG2P].splits > 1u)
+    k_g2p<KIND, MINB, TR, true><<<g, kG2PWarp, 0, lc.stream>>>(v);
+  else
+    k_g2p<KIND, MINB, TR, false><<<g, kG2PWarp, 0, lc.stream>>>(v);
+}
+
 template <int KIND>
 static void launch_all(const LaunchCfg& lc, StepView v, int which) {
   switch (which) {
     case LK_P2G:
       if (lc.transfer == 1)
-        k_p2g<KIND, 1, 1, KIND == 0, 1><<<lc.sm_count * 32, kP2GWarp, 0, lc.stream>>>(v);
+        launch_p2g<KIND, 1, 1, KIND == 0, 1>(lc, v);
       else if (lc.transfer == 2)
-        k_p2g<KIND, 2, 1, KIND == 0, 1><<<lc.sm_count * 32, kP2GWarp, 0, lc.stream>>>(v);
+        launch_p2g<KIND, 2, 1, KIND == 0, 1>(lc, v);
       else
         launch_p2g_apic<KIND>(lc, v);
       break;
@@ -1959,24 +1993,24 @@ static void launch_all(const LaunchCfg& lc, StepView v, int which) {
       // warps/SM for the quadratic twin); the kernel-gradient APIC (two
       // gathers) 16 warps/SM for CK and 12 (168 registers, no spills) for
       // the quadratic twin.
-      if (lc.transfer == 1)
-        k_g2p<KIND, KIND == 0 ? 5 : 4, 1><<<lc.sm_count * (KIND == 0 ? 20 : 16), kG2PWarp, 0, lc.stream>>>(v);
-      else if (lc.transfer == 2)
-        k_g2p<KIND, KIND == 0 ? 4 : 3, 2><<<lc.sm_count * (KIND == 0 ? 16 : 12), kG2PWarp, 0, lc.stream>>>(v);
-      else if (lc.g2p_minb >= 6)
-        k_g2p<KIND, 6, 0><<<lc.sm_count * 24, kG2PWarp, 0, lc.stream>>>(v);
-      else if (lc.g2p_minb == 5)
-        k_g2p<KIND, 5, 0><<<lc.sm_count * 20, kG2PWarp, 0, lc.stream>>>(v);
-      else
-        k_g2p<KIND, 4, 0><<<lc.sm_count * 16, kG2PWarp, 0, lc.stream>>>(v);
+      {
+        const uint32_t g = (uint32_t)(lc.sm_count * g2p_warps(KIND, lc.transfer, lc.g2p_minb));
+        if (lc.transfer == 1)
+          launch_g2p<KIND, KIND == 0 ? 5 : 4, 1>(lc, v, g);
+        else if (lc.transfer == 2)
+          launch_g2p<KIND, KIND == 0 ? 4 : 3, 2>(lc, v, g);
+        else if (lc.g2p_minb >= 6)
+          launch_g2p<KIND, 6, 0>(lc, v, g);
+        else if (lc.g2p_minb == 5)
+          launch_g2p<KIND, 5, 0>(lc, v, g);
+        else
+          launch_g2p<KIND, 4, 0>(lc, v, g);
+      }
       break;
     case LK_G2P_FP64: k_g2p_fp64<KIND><<<lc.sm_count * 4, 128, 0, lc.stream>>>(v); break;
     // fused step (APIC + MLS): one resident wave at the G2P register budget
     case LK_G2P2G:
-      if constexpr (KIND == 0)
-        k_g2p2g<KIND, 5><<<lc.sm_count * 20, kG2PWarp, 0, lc.stream>>>(v);
-      else
-        k_g2p2g<KIND, 4><<<lc.sm_count * 16, kG2PWarp, 0, lc.stream>>>(v);
+      k_g2p2g<KIND, fused_warps(KIND) / 4><<<lc.sm_count * fused_warps(KIND), kG2PWarp, 0, lc.stream>>>(v);
       break;
     case LK_LEFTOVER: k_p2g_leftover<KIND><<<lc.sm_count * 4, 128, 0, lc.stream>>>(v); break;
     case LK_CLEAR: k_clear_gacc<KIND><<<lc.persistent_ctas, 128, 0, lc.stream>>>(v); break;
