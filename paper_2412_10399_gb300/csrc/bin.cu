@@ -6,7 +6,8 @@
 //   scan_final    per non-empty key: first slot and scatter cursor; non-empty
 //                 keys become the particle-block list (in key order, so the
 //                 list is deterministic) and flag the 2x2x2 grid blocks they
-//                 touch.  Each CTA takes one tile and sums the tiles before it.
+//                 touch.  Each CTA takes one tile and sums the tiles before it
+//                 (a few tiles: their keys, without tile sums).
 //   scatter_glist perm[cursor[key]++] = particle (warp-aggregated atomics) in
 //                 one part of its CTAs; in the other the flagged grid blocks
 //                 become the active grid-block list, flags cleared
@@ -107,8 +108,9 @@ __device__ __forceinline__ int scene_of_key(const BinScratch& bs, uint32_t key) 
   return (int)bs.scene_tab[2 * lo + 1];
 }
 
-// FUSED: tile_cnt / tile_ne hold the tiles' own sums (else their exclusive scan).
-template <bool FUSED>
+// MODE: what precedes the CTA's tile comes from the tile sums' exclusive scan
+// (0), from the tiles' own sums (1) or from the histogram itself (2).
+template <int MODE>
 __global__ void __launch_bounds__(kScanThreads) k_scan_final(StepView v, BinScratch bs) {
   const uint64_t base = (uint64_t)blockIdx.x * kScanTile + threadIdx.x * kPerThread;
   uint4 x = make_uint4(0u, 0u, 0u, 0u);
@@ -121,10 +123,20 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_final(StepView v, BinScra
   }
   // particles and blocks of the tiles before this one
   uint32_t tpc = 0, tpn = 0;
-  if (FUSED) {
-    for (uint32_t i = threadIdx.x; i < blockIdx.x; i += kScanThreads) {
-      tpc += bs.tile_cnt[i];
-      tpn += bs.tile_ne[i];
+  if (MODE != 0) {
+    if (MODE == 1) {
+      for (uint32_t i = threadIdx.x; i < blockIdx.x; i += kScanThreads) {
+        tpc += bs.tile_cnt[i];
+        tpn += bs.tile_ne[i];
+      }
+    } else {
+      const uint4* c4 = reinterpret_cast<const uint4*>(v.cnt_cur);
+#pragma unroll 4
+      for (uint32_t i = 0; i < blockIdx.x; ++i) {
+        const uint4 y = c4[i * kScanThreads + threadIdx.x];
+        tpc += y.x + y.y + y.z + y.w;
+        tpn += (y.x != 0u) + (y.y != 0u) + (y.z != 0u) + (y.w != 0u);
+      }
     }
     tpc = __reduce_add_sync(0xffffffffu, tpc);
     tpn = __reduce_add_sync(0xffffffffu, tpn);
@@ -158,7 +170,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_final(StepView v, BinScra
   uint32_t pc = ic - tc, pn = in - tn;
 #pragma unroll
   for (int w = 0; w < NW; ++w) {
-    if (FUSED || w == 0) {
+    if (MODE != 0 || w == 0) {
       pc += pcs[w];
       pn += pns[w];
     }
@@ -349,15 +361,19 @@ void launch_bin(cudaStream_t st, const StepView& v, const BinScratch& bs, int wh
   const uint32_t sctas = std::max(1u, std::min(lim, (v.n_cur + 256u * kScatterUnroll - 1u) / (256u * kScatterUnroll)));
   const uint32_t gctas = std::max(1u, std::min(lim, (n_gblocks + 1023u) / 1024u));
   switch (which) {
-    case LB_SCAN_TILES: k_scan_tiles<<<ntiles, kScanThreads, 0, st>>>(v, bs); break;
+    case LB_SCAN_TILES:
+      if (!scan_direct(v.n_keys)) k_scan_tiles<<<ntiles, kScanThreads, 0, st>>>(v, bs);
+      break;
     case LB_SCAN_TOP:
       if (!fused) k_scan_top<<<1, 1024, 0, st>>>(bs, ntiles);
       break;
     case LB_SCAN_FINAL:
-      if (fused)
-        k_scan_final<true><<<ntiles, kScanThreads, 0, st>>>(v, bs);
+      if (scan_direct(v.n_keys))
+        k_scan_final<2><<<ntiles, kScanThreads, 0, st>>>(v, bs);
+      else if (fused)
+        k_scan_final<1><<<ntiles, kScanThreads, 0, st>>>(v, bs);
       else
-        k_scan_final<false><<<ntiles, kScanThreads, 0, st>>>(v, bs);
+        k_scan_final<0><<<ntiles, kScanThreads, 0, st>>>(v, bs);
       break;
     case LB_SCATTER_GLIST: k_scatter_glist<<<sctas + gctas, 256, 0, st>>>(v, n_gblocks, sctas); break;
     case LB_GLIST: k_scatter_glist<<<gctas, 256, 0, st>>>(v, n_gblocks, 0u); break;

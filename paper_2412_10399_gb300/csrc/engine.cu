@@ -267,7 +267,7 @@ ck::StepView make_view(ckmpm_ctx* ctx) {
   v.n_mats = (uint32_t)ctx->cap_mats;
   v.n_keys = (uint32_t)std::max<int64_t>(ctx->keys_alloc.high, 1);
   v.n_cur = (uint32_t)ctx->n_cur;
-  if (ck::scan_fused(v.n_keys)) {
+  if (ck::scan_fused(v.n_keys) && !ck::scan_direct(v.n_keys)) {
     v.tile_cnt = ctx->tile_cnt;
     v.tile_ne = ctx->tile_ne;
   }
@@ -667,7 +667,7 @@ ckmpm_status run_step(ckmpm_ctx* ctx, bool probe) {
   ckmpm_ctx::EvPair ep{};
   const bool fused_scan = ck::scan_fused(v.n_keys);
   if (ctx->keys_dirty) ctx->tiles_keys = 0;
-  const bool own_tiles = !fused_scan || ctx->tiles_keys != v.n_keys;
+  const bool own_tiles = !fused_scan || (!ck::scan_direct(v.n_keys) && ctx->tiles_keys != v.n_keys);
   const bool steady =
       !probe && !ctx->timing && !ctx->grids_dirty && !ctx->keys_dirty && !(fused_scan && own_tiles);
   if (probe) drop_graphs(ctx);  // the probe refills the block table the graphs were captured with
@@ -798,7 +798,7 @@ ckmpm_status run_step_fused(ckmpm_ctx* ctx) {
   ck::StepView vn = make_view(ctx);
   ctx->tsel = cs;
   const bool fused_scan = ck::scan_fused(vc.n_keys);
-  const bool own_tiles = !fused_scan || ctx->tiles_keys != vc.n_keys;
+  const bool own_tiles = !fused_scan || (!ck::scan_direct(vc.n_keys) && ctx->tiles_keys != vc.n_keys);
   ckmpm_ctx::EvPair ep{};
   if (ctx->timing) cudaEventRecord(ctx->step_a, ctx->stream);
   // the fused kernel gathers through set cs and scatters through set ns

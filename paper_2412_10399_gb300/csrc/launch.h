@@ -76,6 +76,20 @@ void launch_admit(int kind, cudaStream_t st, Pool P, uint32_t* key, uint32_t* cn
 void launch_rekey(int kind, cudaStream_t st, Pool P, uint32_t* key, uint32_t* cnt, uint32_t* bnd,
                   const SceneDev* scenes, const MatDev* mats, uint32_t n, uint32_t* err);
 
+// The allocation-free entry point (noalloc.cu): scene parameters as a kernel
+// argument, which the admission kernel leaves in device memory for the rest.
+constexpr int kStaticMaxMats = 16;
+struct StaticParams {
+  SceneDev scene;
+  MatDev mats[kStaticMaxMats];
+  uint32_t tab[2];
+};
+void launch_static_admit(int kind, cudaStream_t st, const StepView& v, const StaticParams& prm, StaticParams* d_prm,
+                         bool pic, uint32_t nmat, const float* x, const float* vel, const uint8_t* mat, const float* F,
+                         const float* B);
+void launch_static_grids(int kind, cudaStream_t st, const StepView& v, uint32_t n_vblocks, float* grid_m,
+                         float* grid_p);
+
 // bin.cu
 constexpr int kScanTile = 1024;  // keys per scan tile
 // Up to this many tiles every CTA of the scan sums the tiles before its own
@@ -85,6 +99,10 @@ __host__ __device__ inline uint32_t scan_tiles(uint32_t n_keys) {
   const uint32_t t = (uint32_t)(((uint64_t)n_keys + kScanTile - 1) / kScanTile);
   return t ? t : 1u;
 }
+// Up to this many tiles the scan needs no tile sums: every CTA counts the keys
+// before its own tile itself (at most 7 loads of 16 bytes a thread).
+constexpr uint32_t kScanDirectTiles = 8;
+inline bool scan_direct(uint32_t n_keys) { return scan_tiles(n_keys) <= kScanDirectTiles; }
 inline bool scan_fused(uint32_t n_keys) { return scan_tiles(n_keys) <= kScanFusedTiles; }
 struct BinScratch {
   uint32_t* tile_cnt;   // per tile: sum of counts

@@ -45,7 +45,7 @@ namespace {
 
 constexpr int64_t kStaticMaxN = 65536;    // particles per call
 constexpr int kStaticMaxRes = 64;         // cells per axis
-constexpr int kStaticMaxMats = 16;        // materials per scene
+using ck::kStaticMaxMats;                 // materials per scene
 constexpr size_t kStaticBytes = 18u << 20;  // 18 MiB, enough for the limits above
 constexpr int kMaxDevices = 64;
 
@@ -142,24 +142,30 @@ extern "C" CKMPM_API ckmpm_status ckmpm_p2g_grids_static(const ckmpm_scene* sc, 
   P.VM0 = cv.take<float4>(n);
   P.VM1 = cv.take<float4>(n);
   P.VM2 = cv.take<float4>(n);
-  P.F0 = cv.take<float4>(n);
-  P.F1 = cv.take<float4>(n);
-  P.F2 = cv.take<float>(n);
-  P.ID = cv.take<uint32_t>(n);
-  P.E = nullptr;
   ck::StepView v{};
   v.cur = P;
   v.nxt = P;  // not written: no G2P runs here
   v.key_cur = cv.take<uint32_t>(n);
   v.key_nxt = v.key_cur;
-  v.cnt_cur = cv.take<uint32_t>(nkeys);
-  v.cnt_nxt = cv.take<uint32_t>(nkeys);
-  v.bnd_cur = cv.take<uint32_t>(2 * nkeys);
-  v.bnd_nxt = cv.take<uint32_t>(2 * nkeys);
   v.cursor = cv.take<uint32_t>(nkeys);
   v.perm = cv.take<uint32_t>(n);
   v.pb = cv.take<uint2>(nkeys + 1);
   v.pb_scene = cv.take<uint32_t>(nkeys);
+  v.table = cv.take<uint32_t>(nvb);
+  v.g_list = cv.take<uint32_t>(nvb);
+  v.g_scene = cv.take<uint32_t>(nvb);
+  v.pool_cap = (uint32_t)nvb;
+  ck::StaticParams* d_prm = cv.take<ck::StaticParams>(1);
+  ck::BinScratch bs{};
+  bs.tile_cnt = cv.take<uint32_t>(ntiles + 1);
+  bs.tile_ne = cv.take<uint32_t>(ntiles + 1);
+  // what a previous call may have left behind and the kernels expect zero, in
+  // one piece
+  char* const zero = cv.base + cv.used;
+  v.cnt_cur = cv.take<uint32_t>(nkeys);
+  v.cnt_nxt = v.cnt_cur;
+  v.bnd_cur = cv.take<uint32_t>(2 * nkeys);
+  v.bnd_nxt = v.bnd_cur;
   uint32_t* counters = cv.take<uint32_t>(8);
   v.n_pb = counters + 0;
   v.n_g = counters + 1;
@@ -167,31 +173,27 @@ extern "C" CKMPM_API ckmpm_status ckmpm_p2g_grids_static(const ckmpm_scene* sc, 
   v.fp64_count = (unsigned long long*)(counters + 4);
   v.work = counters + 6;
   v.gflag = cv.take<uint32_t>(nvb);
-  v.table = cv.take<uint32_t>(nvb);
-  v.g_list = cv.take<uint32_t>(nvb);
-  v.g_scene = cv.take<uint32_t>(nvb);
-  v.pool_cap = (uint32_t)nvb;
   v.Gacc = cv.take<float4>(nvb * NG * ck::kBlockNodes);
   v.Gvel = v.Gacc;  // the grid update is not run
-  ck::SceneDev* d_scene = cv.take<ck::SceneDev>(1);
-  ck::MatDev* d_mats = cv.take<ck::MatDev>(kStaticMaxMats);
-  uint32_t* scene_tab = cv.take<uint32_t>(2);
-  ck::BinScratch bs{};
-  bs.tile_cnt = cv.take<uint32_t>(ntiles + 1);
-  bs.tile_ne = cv.take<uint32_t>(ntiles + 1);
   if (!cv.ok) return CKMPM_ENOMEM;  // cannot happen within the limits above
-  v.scenes = d_scene;
-  v.mats = d_mats;
+  const size_t zero_bytes = (size_t)(cv.base + cv.used - zero);
+  v.scenes = &d_prm->scene;
+  v.mats = d_prm->mats;
   v.n_mats = kStaticMaxMats;
   v.n_keys = (uint32_t)nkeys;
   v.n_cur = (uint32_t)n;
   v.keep_gacc = 1;
-  v.units[ck::kUnitsP2G] = {1u, 512u};
-  bs.scene_tab = scene_tab;
+  const int rep = kernel == 1 ? 2 : 1;  // a context's choice
+  const int warps = ck::p2g_warps(kernel, pic ? 1 : 0, rep);
+  v.units[ck::kUnitsP2G] = ck::step_units(ck::kUnitsP2G, n, sms, warps);
+  v.unit_most = ck::p2g_ctas(sms);
+  v.work0[0] = v.units[ck::kUnitsP2G].splits > 1 ? (uint32_t)(sms * warps) : 0u;
+  bs.scene_tab = d_prm->tab;
   bs.n_scene_tab = 1;
 
   // scene and material parameters (same definitions as a context's admission)
-  ck::SceneDev h{};
+  ck::StaticParams prm{};
+  ck::SceneDev& h = prm.scene;
   const double V0 = sc->dx * sc->dx * sc->dx / sc->ppc;
   h.dx = (float)sc->dx;
   h.inv_dx = (float)(1.0 / sc->dx);
@@ -210,7 +212,7 @@ extern "C" CKMPM_API ckmpm_status ckmpm_p2g_grids_static(const ckmpm_scene* sc, 
   h.cond_tol = (float)sc->fp64_cond_tol;
   h.gap_tol = (float)sc->fp64_gap_tol;
   h.alive = 1;
-  ck::MatDev hm[kStaticMaxMats] = {};
+  ck::MatDev* const hm = prm.mats;
   double mmax = 0.0;
   for (int i = 0; i < sc->n_materials; ++i) {
     const ckmpm_material& m = sc->materials[i];
@@ -228,36 +230,15 @@ extern "C" CKMPM_API ckmpm_status ckmpm_p2g_grids_static(const ckmpm_scene* sc, 
     mmax = std::max(mmax, m.rho * V0);
   }
   h.mmax = (float)mmax;
-  const uint32_t tab[2] = {0u, 0u};
-  const int64_t nn = (int64_t)(sc->res + 1) * (sc->res + 1) * (sc->res + 1);
 
 #define CK_S(expr)                                   \
   do {                                               \
     if ((expr) != cudaSuccess) return CKMPM_ECUDA;   \
   } while (0)
-  CK_S(cudaMemcpyAsync(d_scene, &h, sizeof(h), cudaMemcpyHostToDevice, st));
-  CK_S(cudaMemcpyAsync(d_mats, hm, sizeof(ck::MatDev) * kStaticMaxMats, cudaMemcpyHostToDevice, st));
-  CK_S(cudaMemcpyAsync(scene_tab, tab, sizeof(tab), cudaMemcpyHostToDevice, st));
-  // everything a previous call may have left behind and the kernels expect zero
-  CK_S(cudaMemsetAsync(v.cnt_cur, 0, sizeof(uint32_t) * nkeys, st));
-  CK_S(cudaMemsetAsync(v.bnd_cur, 0, sizeof(uint32_t) * 2 * nkeys, st));
-  CK_S(cudaMemsetAsync(counters, 0, sizeof(uint32_t) * 8, st));
-  CK_S(cudaMemsetAsync(v.gflag, 0, sizeof(uint32_t) * nvb, st));
-  CK_S(cudaMemsetAsync(v.Gacc, 0, sizeof(float4) * nvb * NG * ck::kBlockNodes, st));
-  CK_S(cudaMemsetAsync(grid_m, 0, sizeof(float) * NG * nn, st));
-  CK_S(cudaMemsetAsync(grid_p, 0, sizeof(float) * 3 * NG * nn, st));
-
-  // particles: x, v, material; B = 0 and F = I, then the caller's F and B
-  ck::launch_admit(kernel, st, P, v.key_cur, v.cnt_cur, v.bnd_cur, d_scene, d_mats, 0, 0u, (uint32_t)sc->n_materials,
-                   0u, (uint32_t)n, sc->x, sc->v, sc->mat, nullptr, v.err);
-  if (F || B) {
-    if (F) ck::launch_write_particles(pic, st, P, d_scene, d_mats, 0, 0u, (uint32_t)n, CKMPM_FIELD_F, F);
-    if (B) ck::launch_write_particles(pic, st, P, d_scene, d_mats, 0, 0u, (uint32_t)n, CKMPM_FIELD_B, B);
-    // M changed: histogram and P2G bounds again
-    CK_S(cudaMemsetAsync(v.cnt_cur, 0, sizeof(uint32_t) * nkeys, st));
-    CK_S(cudaMemsetAsync(v.bnd_cur, 0, sizeof(uint32_t) * 2 * nkeys, st));
-    ck::launch_rekey(kernel, st, P, v.key_cur, v.cnt_cur, v.bnd_cur, d_scene, d_mats, (uint32_t)n, v.err);
-  }
+  CK_S(cudaMemsetAsync(zero, 0, zero_bytes, st));
+  // particles: x, v, material, M of the caller's B and F (B = 0, F = I if
+  // NULL), keys, histogram and P2G bounds; the parameters into device memory
+  ck::launch_static_admit(kernel, st, v, prm, d_prm, pic, (uint32_t)sc->n_materials, sc->x, sc->v, sc->mat, F, B);
   // binning and P2G, as in a context's step
   const int grid_ctas = sms * 4;
   ck::launch_bin(st, v, bs, ck::LB_SCAN_TILES, (uint32_t)nvb, grid_ctas);
@@ -265,10 +246,13 @@ extern "C" CKMPM_API ckmpm_status ckmpm_p2g_grids_static(const ckmpm_scene* sc, 
   ck::launch_bin(st, v, bs, ck::LB_SCAN_FINAL, (uint32_t)nvb, grid_ctas);
   ck::launch_bin(st, v, bs, ck::LB_SCATTER_GLIST, (uint32_t)nvb, grid_ctas);
   ck::LaunchCfg lc{st, sms * 8};
+  lc.sm_count = sms;
   lc.transfer = pic ? 1 : 0;
+  lc.p2g_rep = rep;
+  lc.p2g_rot = kernel == 1 ? 0 : 1;
+  lc.p2g_fma = 1;
   ck::launch_transfer(kernel, lc, v, ck::LK_P2G);
-  ck::launch_read_grid(kernel, st, v, 0, 0, grid_m);
-  ck::launch_read_grid(kernel, st, v, 0, 1, grid_p);
+  ck::launch_static_grids(kernel, st, v, (uint32_t)nvb, grid_m, grid_p);
   CK_S(cudaGetLastError());
   // the error word comes back on the caller's stream: waiting for that
   // stream alone leaves work on the device's other streams running

@@ -1835,6 +1835,89 @@ __global__ void k_read_grid(const float4* Gacc, const float4* Gvel, const uint32
   }
 }
 
+// The allocation-free entry point's admission: the state that k_admit, an
+// upload of F and one of B would leave (M = m B - dt V0 tau(F); pic: no B), its
+// keys, histogram and bounds in one pass.
+template <int KIND>
+__global__ void __launch_bounds__(128) k_static_admit(StepView v, const __grid_constant__ StaticParams prm,
+                                                      StaticParams* d_prm, int pic, uint32_t nmat, const float* x,
+                                                      const float* vel, const uint8_t* mat, const float* Fin,
+                                                      const float* Bin) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *d_prm = prm;
+  const SceneDev& s = prm.scene;
+  const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= v.n_cur) return;
+  float px = x[3 * t], py = x[3 * t + 1], pz = x[3 * t + 2];
+  float ux = px * s.inv_dx, uy = py * s.inv_dx, uz = pz * s.inv_dx;
+  if (!(in_domain(ux, s.res) && in_domain(uy, s.res) && in_domain(uz, s.res))) {
+    flag_error(v.err, CK_ERR_DOMAIN);
+    const float lo = 0.5f, hi = (float)s.res - 0.5f - 1e-3f;
+    ux = fminf(fmaxf(isfinite(ux) ? ux : lo, lo), hi);
+    uy = fminf(fmaxf(isfinite(uy) ? uy : lo, lo), hi);
+    uz = fminf(fmaxf(isfinite(uz) ? uz : lo, lo), hi);
+    px = ux * s.dx; py = uy * s.dx; pz = uz * s.dx;
+    ux = px * s.inv_dx; uy = py * s.inv_dx; uz = pz * s.inv_dx;
+  }
+  uint32_t m = mat ? (uint32_t)mat[t] : 0u;
+  if (m >= nmat) {  // unknown material index: use material 0 and report
+    flag_error(v.err, CK_ERR_INTERNAL);
+    m = 0;
+  }
+  const MatDev& mt = prm.mats[m];
+  const float vx = vel ? vel[3 * t] : 0.f, vy = vel ? vel[3 * t + 1] : 0.f, vz = vel ? vel[3 * t + 2] : 0.f;
+  float M[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  if (Bin && !pic) {
+#pragma unroll
+    for (int q = 0; q < 9; ++q) M[q] = mt.mass * Bin[9 * t + q];
+  }
+  if (Fin) {  // tau(I) = 0 for every model
+    float F[9], tau[9];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) F[q] = Fin[9 * t + q];
+    stress_of(mt, F, mt.mu, mt.lam, tau);
+    const float dtv = s.dt * s.V0;
+#pragma unroll
+    for (int q = 0; q < 9; ++q) M[q] -= dtv * tau[q];
+  }
+  v.cur.X[t] = make_float4(px, py, pz, __uint_as_float(m));
+  v.cur.VM0[t] = make_float4(vx, vy, vz, 0.f);
+  Pool P = v.cur;
+  store_M(P, t, M);
+  const uint32_t k = particle_key<KIND>(s, ux, uy, uz);
+  v.key_cur[t] = k;
+  float bmass, bmom;
+  p2g_bounds<KIND>(s.inv_dx, mt.mass, V3{pk(vx, vy), vz}, from_rows(M), bmass, bmom);
+  warp_aggregated_bin(v.cnt_cur, v.bnd_cur, k, bmass, bmom);
+}
+
+// Its results: mass and momentum of every node of the domain, read from the
+// active blocks (a block is active when its table entry and the slot's list
+// entry agree; entries of other blocks are stale) and zero elsewhere, in one
+// pass that writes each output once.
+template <int KIND>
+__global__ void __launch_bounds__(128) k_static_grids(StepView v, uint32_t n_vblocks, float* gm, float* gp) {
+  constexpr int NG = Geo<KIND>::NG;
+  const int n = v.scenes[0].res + 1, nb = v.scenes[0].nb;
+  const size_t nnode = (size_t)n * n * n;
+  const uint32_t ng = min(*v.n_g, v.pool_cap);
+  for (uint32_t b = blockIdx.x; b < n_vblocks; b += gridDim.x) {
+    const uint32_t sl = v.table[b];
+    const bool on = sl < ng && v.g_list[sl] == b;
+    const int bx = (int)(b % (uint32_t)nb), by = (int)((b / (uint32_t)nb) % (uint32_t)nb), bz = (int)(b / ((uint32_t)nb * nb));
+    for (int t = threadIdx.x; t < NG * kBlockNodes; t += 128) {
+      const int g = t / kBlockNodes, l = t % kBlockNodes;
+      const int ix = bx * 4 + (l & 3), iy = by * 4 + ((l >> 2) & 3), iz = bz * 4 + (l >> 4);
+      if (ix >= n || iy >= n || iz >= n) continue;
+      const float4 a = on ? v.Gacc[((size_t)sl * NG + g) * kBlockNodes + l] : make_float4(0.f, 0.f, 0.f, 0.f);
+      const size_t q = g * nnode + ((size_t)iz * n + iy) * n + ix;
+      gm[q] = a.x;
+      gp[3 * q] = a.y;
+      gp[3 * q + 1] = a.z;
+      gp[3 * q + 2] = a.w;
+    }
+  }
+}
+
 // Append a new scene's particles: X (x, mat_base + mat), v, M = 0 (B = 0 and
 // tau(I) = 0), F = I, ID = index; plus keys and the histogram.
 template <int KIND>
@@ -2064,6 +2147,24 @@ void launch_read_grid(int kind, cudaStream_t st, const StepView& v, int scene, i
   else
     k_read_grid<1><<<1024, 128, 0, st>>>(v.Gacc, v.Gvel, v.g_list, v.g_scene, v.n_g, v.pool_cap, v.scenes, scene,
                                           which, out);
+}
+
+void launch_static_admit(int kind, cudaStream_t st, const StepView& v, const StaticParams& prm, StaticParams* d_prm,
+                         bool pic, uint32_t nmat, const float* x, const float* vel, const uint8_t* mat, const float* F,
+                         const float* B) {
+  const uint32_t blocks = (v.n_cur + 127u) / 128u;
+  if (kind == 0)
+    k_static_admit<0><<<blocks, 128, 0, st>>>(v, prm, d_prm, pic ? 1 : 0, nmat, x, vel, mat, F, B);
+  else
+    k_static_admit<1><<<blocks, 128, 0, st>>>(v, prm, d_prm, pic ? 1 : 0, nmat, x, vel, mat, F, B);
+}
+
+void launch_static_grids(int kind, cudaStream_t st, const StepView& v, uint32_t n_vblocks, float* grid_m,
+                         float* grid_p) {
+  if (kind == 0)
+    k_static_grids<0><<<n_vblocks, 128, 0, st>>>(v, n_vblocks, grid_m, grid_p);
+  else
+    k_static_grids<1><<<n_vblocks, 128, 0, st>>>(v, n_vblocks, grid_m, grid_p);
 }
 
 void launch_admit(int kind, cudaStream_t st, Pool P, uint32_t* key, uint32_t* cnt, uint32_t* bnd,
