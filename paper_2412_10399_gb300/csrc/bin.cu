@@ -339,17 +339,21 @@ void launch_table_reset(cudaStream_t st, uint32_t* table, const uint32_t* g_list
 }
 
 // Retire particles [start, start + n) of the current pool (a released scene):
-// they get the dead key and leave the pool at the next step.
-__global__ void k_mark_dead(uint32_t* key, uint32_t start, uint32_t n) {
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    key[start + i] = CK_DEAD_KEY;
+// they get the dead key and leave the pool at the next step; the histogram and
+// bounds of the scene's key range [k0, k0 + nk) go back to zero.
+__global__ void k_retire(uint32_t* key, uint32_t start, uint32_t n, uint32_t* cnt, uint32_t* bnd, uint32_t k0,
+                         uint32_t nk) {
+  const uint32_t t0 = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+  for (uint64_t i = t0; i < n; i += stride) key[start + i] = CK_DEAD_KEY;
+  for (uint64_t i = t0; i < nk; i += stride) cnt[k0 + i] = 0u;
+  for (uint64_t i = t0; i < 2ull * nk; i += stride) bnd[2ull * k0 + i] = 0u;
 }
 
-void launch_mark_dead(cudaStream_t st, uint32_t* key, uint32_t start, uint32_t n) {
-  int blocks = (int)((n + 255) / 256);
-  if (blocks < 1) blocks = 1;
-  if (blocks > 4096) blocks = 4096;
-  k_mark_dead<<<blocks, 256, 0, st>>>(key, start, n);
+void launch_retire(cudaStream_t st, uint32_t* key, uint32_t start, uint32_t n, uint32_t* cnt, uint32_t* bnd,
+                   uint32_t k0, uint32_t nk) {
+  const uint64_t most = std::max<uint64_t>(n, 2ull * nk);
+  const int blocks = (int)std::max<uint64_t>(1, std::min<uint64_t>(4096, (most + 255) / 256));
+  k_retire<<<blocks, 256, 0, st>>>(key, start, n, cnt, bnd, k0, nk);
 }
 
 void launch_bin(cudaStream_t st, const StepView& v, const BinScratch& bs, int which, uint32_t n_gblocks,

@@ -114,6 +114,7 @@ struct ckmpm_ctx {
   // fused steps); dropped whenever the launch sequence or its arguments change
   bool graphs = false;
   cudaGraphExec_t gexec[4] = {nullptr, nullptr, nullptr, nullptr};
+  bool gvalid[4] = {false, false, false, false};  // gexec[i] holds the current launch sequence
   int64_t graph_steps = 0;  // steps launched as a graph
   int tsel = 0;
   bool grid_valid = false;
@@ -140,6 +141,7 @@ struct ckmpm_ctx {
     int64_t ticket = -1;
   };
   RbSlot rb[2];
+  uint32_t* h_err = nullptr;  // pinned: the device status word as last copied
   cudaStream_t copy_stream = nullptr;
   cudaEvent_t rb_gathered = nullptr;
   int64_t rb_next = 0;
@@ -152,6 +154,7 @@ struct ckmpm_ctx {
   int64_t n_cur = 0;
   std::vector<Seg> layout;
   bool keys_dirty = false, grids_dirty = false;
+  int n_tab = 0;  // entries of scene_tab
   ckmpm_status sticky = CKMPM_OK;
   int64_t steps = 0;
   std::string msg;
@@ -291,12 +294,12 @@ ck::StepView make_view(ckmpm_ctx* ctx) {
   return v;
 }
 
-ck::BinScratch make_bs(ckmpm_ctx* ctx, int n_tab) {
+ck::BinScratch make_bs(ckmpm_ctx* ctx) {
   ck::BinScratch bs{};
   bs.tile_cnt = ctx->tile_cnt;
   bs.tile_ne = ctx->tile_ne;
   bs.scene_tab = ctx->scene_tab;
-  bs.n_scene_tab = n_tab;
+  bs.n_scene_tab = ctx->n_tab;
   return bs;
 }
 
@@ -332,7 +335,10 @@ void harvest_timing(ckmpm_ctx* ctx) {
   cudaGetLastError();
 }
 
-int upload_scene_tab(ckmpm_ctx* ctx) {
+// The table of alive scenes by key range, sent at every admission.  A release
+// leaves its scene's entry there: no particle has a key in that range until a
+// later admission takes it and sends the table again.
+void upload_scene_tab(ckmpm_ctx* ctx) {
   std::vector<uint32_t> tab;
   std::vector<std::pair<int64_t, int>> al;
   for (int s = 0; s < (int)ctx->scenes.size(); ++s)
@@ -347,13 +353,7 @@ int upload_scene_tab(ckmpm_ctx* ctx) {
     tab.push_back(0);
   }
   cudaMemcpyAsync(ctx->scene_tab, tab.data(), tab.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, ctx->stream);
-  return (int)(tab.size() / 2);
-}
-
-int n_scene_tab(ckmpm_ctx* ctx) {
-  int n = 0;
-  for (auto& s : ctx->scenes) n += s.alive ? 1 : 0;
-  return std::max(n, 1);
+  ctx->n_tab = (int)(tab.size() / 2);
 }
 
 void process_pending(ckmpm_ctx* ctx) {
@@ -408,11 +408,13 @@ ckmpm_status apply_device_error(ckmpm_ctx* ctx, uint32_t e) {
   return ctx->sticky;
 }
 
-ckmpm_status read_device_error(ckmpm_ctx* ctx) {
-  uint32_t e = 0;
-  cudaError_t ce = cudaMemcpy(&e, ctx->counters + 2, sizeof(uint32_t), cudaMemcpyDeviceToHost);
-  if (ce != cudaSuccess) return cuda_fail(ctx, ce, "reading the device status word");
-  return apply_device_error(ctx, e);
+// Wait for the context's stream and take the device status word: the word is
+// copied into pinned memory on that stream, so one synchronisation serves both
+// (a blocking copy behind a synchronisation costs a second round trip).
+ckmpm_status sync_and_read_error(ckmpm_ctx* ctx, const char* where) {
+  CK_TRY(cudaMemcpyAsync(ctx->h_err, ctx->counters + 2, sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream), where);
+  CK_TRY(cudaStreamSynchronize(ctx->stream), where);
+  return apply_device_error(ctx, *ctx->h_err);
 }
 
 bool ensure_staging(ckmpm_ctx* ctx, size_t bytes) {
@@ -596,6 +598,7 @@ ckmpm_status init_ctx(ckmpm_ctx* ctx, const ckmpm_config* cfg) {
   ctx->keys_alloc.init(ctx->cap_keys);
   ctx->grid_alloc.init(ctx->cap_vblocks);
   ctx->mat_alloc.init(ctx->cap_mats);
+  CK_TRY(cudaHostAlloc((void**)&ctx->h_err, sizeof(uint32_t), cudaHostAllocDefault), "status word");
   CK_TRY(cudaEventCreate(&ctx->step_a), "event");
   CK_TRY(cudaEventCreate(&ctx->step_b), "event");
   CK_TRY(cudaGetLastError(), "init");
@@ -613,12 +616,19 @@ bool capturing(ckmpm_ctx* ctx) {
   return st != cudaStreamCaptureStatusNone;
 }
 
+// The next step of each parity captures its launch sequence again; the
+// executable graphs stay, to be updated from that capture.
 void drop_graphs(ckmpm_ctx* ctx) {
+  for (auto& g : ctx->gvalid) g = false;
+}
+
+void destroy_graphs(ckmpm_ctx* ctx) {
   for (auto& g : ctx->gexec)
     if (g) {
       cudaGraphExecDestroy(g);
       g = nullptr;
     }
+  drop_graphs(ctx);
 }
 
 // Run a step's launch sequence as the CUDA graph of state parity `key`,
@@ -630,7 +640,7 @@ template <typename Issue>
 bool graph_step(ckmpm_ctx* ctx, int key, Issue&& issue) {
   if (!ctx->graphs) return false;
   cudaGraphExec_t& ex = ctx->gexec[key];
-  if (!ex) {
+  if (!ctx->gvalid[key]) {
     if (cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
       cudaGetLastError();
       ctx->graphs = false;
@@ -639,7 +649,19 @@ bool graph_step(ckmpm_ctx* ctx, int key, Issue&& issue) {
     issue();
     cudaGraph_t g = nullptr;
     const cudaError_t e = cudaStreamEndCapture(ctx->stream, &g);
-    if (e != cudaSuccess || !g || cudaGraphInstantiate(&ex, g, 0) != cudaSuccess) {
+    // after an admission or a release the sequence has the same kernels with
+    // other arguments: updating the executable graph takes microseconds where
+    // instantiating one takes ten times that (a launch in flight keeps what
+    // it was launched with)
+    if (e == cudaSuccess && g && ex) {
+      cudaGraphExecUpdateResultInfo info{};
+      if (cudaGraphExecUpdate(ex, g, &info) != cudaSuccess) {
+        cudaGetLastError();
+        cudaGraphExecDestroy(ex);
+        ex = nullptr;
+      }
+    }
+    if (e != cudaSuccess || !g || (!ex && cudaGraphInstantiate(&ex, g, 0) != cudaSuccess)) {
       if (g) cudaGraphDestroy(g);
       cudaGetLastError();
       ex = nullptr;
@@ -647,10 +669,11 @@ bool graph_step(ckmpm_ctx* ctx, int key, Issue&& issue) {
       return false;
     }
     cudaGraphDestroy(g);
+    ctx->gvalid[key] = true;
   }
   if (cudaGraphLaunch(ex, ctx->stream) != cudaSuccess) {
     cudaGetLastError();
-    drop_graphs(ctx);
+    destroy_graphs(ctx);
     ctx->graphs = false;
     return false;
   }
@@ -697,7 +720,7 @@ ckmpm_status run_step(ckmpm_ctx* ctx, bool probe) {
     CK_TRY(cudaGetLastError(), "step launch");
     return CKMPM_OK;
   }
-  ck::BinScratch bs = make_bs(ctx, n_scene_tab(ctx));
+  ck::BinScratch bs = make_bs(ctx);
   const uint32_t ngb = (uint32_t)std::max<int64_t>(ctx->grid_alloc.high, 1);
   const int grid_ctas = ctx->sm_count * 4;
   // fused contexts keep each table set's assigned entries listed, so that a
@@ -788,7 +811,7 @@ ckmpm_status run_step_fused(ckmpm_ctx* ctx) {
     CK_TRY(cudaGetLastError(), "step launch");
     return CKMPM_OK;
   }
-  ck::BinScratch bs = make_bs(ctx, n_scene_tab(ctx));
+  ck::BinScratch bs = make_bs(ctx);
   const uint32_t ngb = (uint32_t)std::max<int64_t>(ctx->grid_alloc.high, 1);
   const int grid_ctas = ctx->sm_count * 4;
   const int cs = ctx->tsel, ns = cs ^ 1;
@@ -1116,29 +1139,26 @@ ckmpm_status ckmpm_release(ckmpm_ctx* ctx, int scene_id) {
     return fail(ctx, CKMPM_ENOTFOUND, "unknown scene id");
   if (capturing(ctx)) return fail(ctx, CKMPM_EBUSY, "release is not allowed during stream capture");
   SceneHost& h = ctx->scenes[scene_id];
-  // retire its particles now (dead keys, cleared histogram range) so that its
-  // slot, key range, block table and materials can be reused at once; the
-  // particles themselves leave the pool at the next step
+  // retire its particles now (dead keys, cleared histogram and bounds) so that
+  // its slot, key range, block table and materials can be reused at once; the
+  // particles themselves leave the pool at the next step.  (Nothing reads the
+  // scene's parameters again: a dead key says enough.)
+  int64_t start = 0, n = 0;
   for (size_t i = 0; i < ctx->layout.size(); ++i) {
     if (ctx->layout[i].slot == scene_id) {
-      ck::launch_mark_dead(ctx->stream, ctx->key[ctx->cur], (uint32_t)ctx->layout[i].start,
-                           (uint32_t)ctx->layout[i].n);
+      start = ctx->layout[i].start;
+      n = ctx->layout[i].n;
       ctx->layout.erase(ctx->layout.begin() + i);
       break;
     }
   }
-  CK_TRY(cudaMemsetAsync(ctx->cnt[ctx->cur] + h.key_base, 0, sizeof(uint32_t) * h.nkeys, ctx->stream), "memset");
-  CK_TRY(cudaMemsetAsync(ctx->bnd[ctx->cur] + 2 * h.key_base, 0, sizeof(uint32_t) * 2 * h.nkeys, ctx->stream),
-         "memset");
+  ck::launch_retire(ctx->stream, ctx->key[ctx->cur], (uint32_t)start, (uint32_t)n, ctx->cnt[ctx->cur],
+                    ctx->bnd[ctx->cur], (uint32_t)h.key_base, (uint32_t)h.nkeys);
   h.alive = false;
   ctx->grid_valid = false;
   ctx->tiles_keys = 0;
   drop_graphs(ctx);
   ctx->h_scenes[scene_id].alive = 0;
-  CK_TRY(cudaMemcpyAsync(ctx->d_scenes + scene_id, &ctx->h_scenes[scene_id], sizeof(SceneDev), cudaMemcpyHostToDevice,
-                         ctx->stream),
-         "upload scene");
-  upload_scene_tab(ctx);
   ctx->pending_free.push_back(scene_id);
   process_pending(ctx);
   CK_TRY(cudaGetLastError(), "release");
@@ -1164,8 +1184,7 @@ ckmpm_status ckmpm_probe_grids(ckmpm_ctx* ctx) {
 
 ckmpm_status ckmpm_sync(ckmpm_ctx* ctx) {
   if (!ctx) return CKMPM_EINVAL;
-  CK_TRY(cudaStreamSynchronize(ctx->stream), "cudaStreamSynchronize");
-  return read_device_error(ctx);
+  return sync_and_read_error(ctx, "cudaStreamSynchronize");
 }
 
 int64_t ckmpm_scene_particles(const ckmpm_ctx* ctx, int scene_id) {
@@ -1309,8 +1328,7 @@ ckmpm_status ckmpm_readback(ckmpm_ctx* ctx, int scene_id, int field, void* dst, 
   ckmpm_status s = readback_check(ctx, scene_id, field, dst, bytes, &want, &which);
   if (s != CKMPM_OK) return s;
   if ((s = readback_gather(ctx, scene_id, field, which, want, (float*)dst)) != CKMPM_OK) return s;
-  CK_TRY(cudaStreamSynchronize(ctx->stream), "readback");
-  return read_device_error(ctx);
+  return sync_and_read_error(ctx, "readback");
 }
 
 ckmpm_status ckmpm_upload(ckmpm_ctx* ctx, int scene_id, int field, const void* src, size_t bytes, int src_is_device) {
@@ -1340,6 +1358,8 @@ ckmpm_status ckmpm_upload(ckmpm_ctx* ctx, int scene_id, int field, const void* s
   ck::launch_write_particles(ctx->transfer == CKMPM_TRANSFER_PIC, ctx->stream, ctx->pool[ctx->cur], ctx->d_scenes, ctx->d_mats, scene_id, (uint32_t)sg->start,
                              (uint32_t)sg->n, field, in);
   cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(ctx->h_err, ctx->counters + 2, sizeof(uint32_t), cudaMemcpyDeviceToHost, ctx->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
   if (tmp) dev_free(ctx, tmp);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "upload");
@@ -1347,7 +1367,7 @@ ckmpm_status ckmpm_upload(ckmpm_ctx* ctx, int scene_id, int field, const void* s
   // the next step re-bins the pool first
   ctx->keys_dirty = true;
   drop_graphs(ctx);
-  return read_device_error(ctx);
+  return apply_device_error(ctx, *ctx->h_err);
 }
 
 ckmpm_status ckmpm_get_stats(ckmpm_ctx* ctx, ckmpm_stats* out) {
@@ -1403,7 +1423,8 @@ ckmpm_status ckmpm_reset_timing(ckmpm_ctx* ctx) {
 ckmpm_status ckmpm_destroy(ckmpm_ctx* ctx) {
   if (!ctx) return CKMPM_OK;
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
-  drop_graphs(ctx);
+  destroy_graphs(ctx);
+  if (ctx->h_err) cudaFreeHost(ctx->h_err);
   harvest_timing(ctx);
   for (auto& e : ctx->ev_free) {
     cudaEventDestroy(e.a);

@@ -114,7 +114,8 @@ void launch_bin(cudaStream_t st, const StepView& v, const BinScratch& bs, int wh
                 int grid_ctas);
 // LB_SCAN_TOP launches nothing when the scan is fused (scan_fused)
 enum { LB_SCAN_TILES = 0, LB_SCAN_TOP = 1, LB_SCAN_FINAL = 2, LB_SCATTER_GLIST = 3, LB_GLIST = 4 };
-void launch_mark_dead(cudaStream_t st, uint32_t* key, uint32_t start, uint32_t n);
+void launch_retire(cudaStream_t st, uint32_t* key, uint32_t start, uint32_t n, uint32_t* cnt, uint32_t* bnd,
+                   uint32_t k0, uint32_t nk);
 void launch_table_reset(cudaStream_t st, uint32_t* table, const uint32_t* g_list, const uint32_t* n_g,
                         uint32_t pool_cap, int grid_ctas);
 

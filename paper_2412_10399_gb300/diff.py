@@ -87,49 +87,93 @@ def initial_state(x0: torch.Tensor):
     return B0, F0
 
 
+def _empty_state(n: int, device) -> torch.Tensor:
+    """A state (x, v, B, F) of a rollout in one allocation."""
+    return torch.empty(24 * n, dtype=torch.float32, device=device)
+
+
+def _addr(s):
+    """The four device addresses of a state: of its tensors, or of the parts
+    of its one allocation."""
+    if isinstance(s, tuple):
+        return tuple(t.data_ptr() for t in s)
+    a, n = s.data_ptr(), s.shape[0] // 24
+    return a, a + 12 * n, a + 24 * n, a + 60 * n
+
+
 class Rollout(torch.autograd.Function):
     """(x0, v0, E) -> (x_T, v_T) after `steps` steps from B = 0, F = I.
 
     Forward keeps the state every `k` steps; backward replays each segment
     from its checkpoint (keeping the k states of that segment) and runs the
-    per-step adjoints in reverse, accumulating dL/dE over all steps."""
+    per-step adjoints in reverse, accumulating dL/dE over all steps.
+
+    The inputs are checked once; the states in between are the rollout's own,
+    so a step is one allocation and one library call on their addresses (a
+    small body's step takes the device about 15 us, and per-tensor checks and
+    allocations took the host 25)."""
 
     @staticmethod
     def forward(ctx, x0, v0, E, sim: DiffSim, steps: int, k: int):
+        n, dev = sim.n, x0.device
         B0, F0 = initial_state(x0)
-        s = (x0.contiguous(), v0.contiguous(), B0, F0)
+        first = (x0.contiguous(), v0.contiguous(), B0, F0)
+        if steps > 0:
+            sim._check(E=E, **dict(zip("xvBF", first)))
+        lib, h, e = ck.load().ckmpm_diff_step, sim.h, E.data_ptr()
+        s, p = first, _addr(first)
         ckpts = []
+        xT, vT = first[0], first[1]
         for t in range(steps):
             if t % k == 0:
                 ckpts.append(s)
-            s = sim.step(*s, E)
+            nxt = _empty_state(n, dev)
+            q = _addr(nxt)
+            if t == steps - 1:  # the results are tensors of their own
+                xT, vT = torch.empty_like(first[0]), torch.empty_like(first[1])
+                q = (xT.data_ptr(), vT.data_ptr()) + q[2:]
+            sim._chk(lib(h, *p, e, *q))
+            s, p = nxt, q
         ctx.sim, ctx.steps, ctx.k = sim, steps, k
         ctx.ckpts = ckpts
         ctx.save_for_backward(E)
-        return s[0], s[1]
+        return xT, vT
 
     @staticmethod
     def backward(ctx, gx, gv):
         (E,) = ctx.saved_tensors
         sim, steps, k = ctx.sim, ctx.steps, ctx.k
         x0 = ctx.ckpts[0][0]
-        n = x0.shape[0]
+        n, dev = x0.shape[0], x0.device
         gx = torch.zeros_like(x0) if gx is None else gx.contiguous()
         gv = torch.zeros_like(x0) if gv is None else gv.contiguous()
-        gB = torch.zeros(n, 3, 3, dtype=torch.float32, device=x0.device)
+        gB = torch.zeros(n, 3, 3, dtype=torch.float32, device=dev)
         gF = torch.zeros_like(gB)
         gE = torch.zeros_like(E)
-        adj = (gx, gv, gB, gF)
+        sim._check(E=E, gx1=gx, gv1=gv, gE=gE)
+        lib = ck.load()
+        fwd, bwd, h, e, ge = lib.ckmpm_diff_step, lib.ckmpm_diff_step_backward, sim.h, E.data_ptr(), gE.data_ptr()
+        adj = tuple(t.data_ptr() for t in (gx, gv, gB, gF))
+        spare = [_empty_state(n, dev), _empty_state(n, dev)]  # adjoints alternate between two
+        gx0, gv0 = torch.empty_like(x0), torch.empty_like(x0)
+        left = steps
         for seg in reversed(range(len(ctx.ckpts))):
             t0 = seg * k
             t1 = min(steps, t0 + k)
             states = [ctx.ckpts[seg]]
             for _ in range(t0, t1 - 1):
-                states.append(sim.step(*states[-1], E))
+                nxt = _empty_state(n, dev)
+                sim._chk(fwd(h, *_addr(states[-1]), e, *_addr(nxt)))
+                states.append(nxt)
             for j in reversed(range(t1 - t0)):
-                adj = sim.step_backward(*states[j], E, *adj, gE)
+                left -= 1
+                out = _addr(spare[left & 1])
+                if left == 0:
+                    out = (gx0.data_ptr(), gv0.data_ptr()) + out[2:]
+                sim._chk(bwd(h, *_addr(states[j]), e, *adj, *out, ge))
+                adj = out
         ctx.ckpts = None
-        return adj[0], adj[1], gE, None, None, None
+        return gx0, gv0, gE, None, None, None
 
 
 def com_loss(x: torch.Tensor, target: torch.Tensor) -> torch.Tensor:
