@@ -68,7 +68,7 @@ def _peaks():
     return 6800.0, "fallback"
 
 
-KERNEL_SOURCES = ("common.cuh", "launch.h", "svd3.cuh", "transfer.cu")
+KERNEL_SOURCES = ("common.cuh", "launch.h", "pack.cuh", "svd3.cuh", "transfer.cu")
 
 
 def _source_hash():

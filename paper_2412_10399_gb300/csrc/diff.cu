@@ -481,7 +481,8 @@ __device__ __forceinline__ void fc_stress_vjp(const float* F, const float* R, co
 // stride with scalar atomics on dense grids that were cleared and swept whole:
 // P2G 75 -> 30 us, grid 28 (with its clears) -> 5, G2P 25 -> 12, G2P^T 78 ->
 // 35, P2G^T 71 -> 34 (its decomposition taken once, no local memory); a
-// forward step 140 -> 62 us, its adjoint 302 -> 129 us.
+// forward step 140 -> 62 us, its adjoint 302 -> 129 us (51 and 105 with the
+// overlapped launches and the polar iteration).
 
 constexpr int kDT = 64;
 
