@@ -653,7 +653,8 @@ bool graph_step(ckmpm_ctx* ctx, int key, Issue&& issue) {
     // other arguments: updating the executable graph takes microseconds where
     // instantiating one takes ten times that (a launch in flight keeps what
     // it was launched with)
-    if (e == cudaSuccess && g && ex) {
+    bool ok = e == cudaSuccess && g;
+    if (ok && ex) {
       cudaGraphExecUpdateResultInfo info{};
       if (cudaGraphExecUpdate(ex, g, &info) != cudaSuccess) {
         cudaGetLastError();
@@ -661,10 +662,14 @@ bool graph_step(ckmpm_ctx* ctx, int key, Issue&& issue) {
         ex = nullptr;
       }
     }
-    if (e != cudaSuccess || !g || (!ex && cudaGraphInstantiate(&ex, g, 0) != cudaSuccess)) {
-      if (g) cudaGraphDestroy(g);
-      cudaGetLastError();
+    if (ok && !ex && cudaGraphInstantiate(&ex, g, 0) != cudaSuccess) {
       ex = nullptr;
+      ok = false;
+    }
+    if (!ok) {
+      if (g) cudaGraphDestroy(g);
+      destroy_graphs(ctx);
+      cudaGetLastError();
       ctx->graphs = false;
       return false;
     }
