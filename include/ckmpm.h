@@ -268,7 +268,8 @@ CKMPM_API ckmpm_status ckmpm_sync(ckmpm_ctx* ctx);
  * the current state without advancing it, so that GRID_M / GRID_P / GRID_V
  * can be read back.  Enqueued on the context's stream like a step (the
  * readback of a grid field synchronises); the next step first clears the
- * probed accumulators. */
+ * probed accumulators (a step that a stream capture recorded before the probe
+ * does not: enqueue one directly before its replay). */
 CKMPM_API ckmpm_status ckmpm_probe_grids(ckmpm_ctx* ctx);
 
 /* Copy a field of one scene into dst (host or device), in the scene's

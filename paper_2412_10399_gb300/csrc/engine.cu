@@ -122,8 +122,10 @@ struct ckmpm_ctx {
   uint32_t* fp64_list = nullptr;  // particles of the float64 pass (capacity cap_n)
   uint32_t *gflag = nullptr, *table = nullptr, *g_list = nullptr, *g_scene = nullptr;
   uint32_t *tile_cnt = nullptr, *tile_ne = nullptr, *scene_tab = nullptr;
-  // key-space size whose tile sums of cnt[cur] are in tile_cnt / tile_ne (left
-  // there by the last step's float64 pass); 0: the next step takes them itself
+  // key-space size whose tile sums of cnt[cur] are in tile_cnt / tile_ne once
+  // the stream's work is done (left there by the last step's float64 pass); 0:
+  // the next step takes them itself.  A step that a caller's capture records
+  // has not run, so it leaves 0
   uint32_t tiles_keys = 0;
   float4 *Gacc = nullptr, *Gvel = nullptr;
   SceneDev* d_scenes = nullptr;
@@ -588,6 +590,9 @@ ckmpm_status init_ctx(ckmpm_ctx* ctx, const ckmpm_config* cfg) {
   CK_TRY(cudaMemsetAsync(ctx->bnd[0], 0, sizeof(uint32_t) * 2 * ctx->cap_keys, ctx->stream), "memset");
   CK_TRY(cudaMemsetAsync(ctx->bnd[1], 0, sizeof(uint32_t) * 2 * ctx->cap_keys, ctx->stream), "memset");
   CK_TRY(cudaMemsetAsync(ctx->counters, 0, sizeof(uint32_t) * 12, ctx->stream), "memset");
+  const size_t tiles = sizeof(uint32_t) * (ceil_div(ctx->cap_keys, ck::kScanTile) + 1);
+  CK_TRY(cudaMemsetAsync(ctx->tile_cnt, 0, tiles, ctx->stream), "memset");
+  CK_TRY(cudaMemsetAsync(ctx->tile_ne, 0, tiles, ctx->stream), "memset");
   CK_TRY(cudaMemsetAsync(ctx->gflag, 0, sizeof(uint32_t) * ctx->cap_vblocks, ctx->stream), "memset");
   CK_TRY(cudaMemsetAsync(ctx->table, 0xff, sizeof(uint32_t) * ctx->cap_vblocks, ctx->stream), "memset");
   CK_TRY(cudaMemsetAsync(ctx->Gacc, 0, sizeof(float4) * ctx->cap_pool * NG * ck::kBlockNodes, ctx->stream), "memset");
@@ -686,6 +691,16 @@ bool graph_step(ckmpm_ctx* ctx, int key, Issue&& issue) {
   return true;
 }
 
+// Whether a step on a key space of n_keys takes the histogram's tile sums
+// itself.  One that is only recorded does: the step or probe whose sums the
+// host counts on may not have run, and need not be the one before a replay.
+bool takes_own_tiles(ckmpm_ctx* ctx, uint32_t n_keys, bool recorded) {
+  if (!ck::scan_fused(n_keys)) return true;
+  return !ck::scan_direct(n_keys) && (recorded || ctx->tiles_keys != n_keys);
+}
+// the key-space size whose tile sums a step or probe leaves behind
+uint32_t tiles_after(uint32_t n_keys, bool recorded) { return ck::scan_fused(n_keys) && !recorded ? n_keys : 0u; }
+
 ckmpm_status run_step_fused(ckmpm_ctx* ctx);
 
 ckmpm_status run_step(ckmpm_ctx* ctx, bool probe) {
@@ -695,9 +710,10 @@ ckmpm_status run_step(ckmpm_ctx* ctx, bool probe) {
   ckmpm_ctx::EvPair ep{};
   const bool fused_scan = ck::scan_fused(v.n_keys);
   if (ctx->keys_dirty) ctx->tiles_keys = 0;
-  const bool own_tiles = !fused_scan || (!ck::scan_direct(v.n_keys) && ctx->tiles_keys != v.n_keys);
+  const bool recorded = capturing(ctx);
+  const bool own_tiles = takes_own_tiles(ctx, v.n_keys, recorded);
   const bool steady =
-      !probe && !ctx->timing && !ctx->grids_dirty && !ctx->keys_dirty && !(fused_scan && own_tiles);
+      !probe && !recorded && !ctx->timing && !ctx->grids_dirty && !ctx->keys_dirty && !(fused_scan && own_tiles);
   if (probe) drop_graphs(ctx);  // the probe refills the block table the graphs were captured with
   if (ctx->grids_dirty) {
     ck::launch_transfer(ctx->kind, ctx->lc, v, ck::LK_CLEAR);
@@ -758,7 +774,7 @@ ckmpm_status run_step(ckmpm_ctx* ctx, bool probe) {
   };
   if (!(steady && !ctx->fused && graph_step(ctx, ctx->cur, issue))) issue();
   // a probe leaves the tile sums of the current state, a step those of the next
-  ctx->tiles_keys = fused_scan ? v.n_keys : 0;
+  ctx->tiles_keys = tiles_after(v.n_keys, recorded);
   if (probe) {
     ctx->grids_dirty = true;
     CK_TRY(cudaGetLastError(), "probe launch");
@@ -826,7 +842,8 @@ ckmpm_status run_step_fused(ckmpm_ctx* ctx) {
   ck::StepView vn = make_view(ctx);
   ctx->tsel = cs;
   const bool fused_scan = ck::scan_fused(vc.n_keys);
-  const bool own_tiles = !fused_scan || (!ck::scan_direct(vc.n_keys) && ctx->tiles_keys != vc.n_keys);
+  const bool recorded = capturing(ctx);
+  const bool own_tiles = takes_own_tiles(ctx, vc.n_keys, recorded);
   ckmpm_ctx::EvPair ep{};
   if (ctx->timing) cudaEventRecord(ctx->step_a, ctx->stream);
   // the fused kernel gathers through set cs and scatters through set ns
@@ -865,7 +882,7 @@ ckmpm_status run_step_fused(ckmpm_ctx* ctx) {
     issue_fused();
   };
   if (ctx->grid_valid) {
-    if (!(was_clean && !(fused_scan && own_tiles) && graph_step(ctx, ctx->cur + 2 * ctx->tsel, issue_steady)))
+    if (!(was_clean && !recorded && !(fused_scan && own_tiles) && graph_step(ctx, ctx->cur + 2 * ctx->tsel, issue_steady)))
       issue_steady();
   } else {
     // every table set is cleared of the entries its last fill assigned (its
@@ -886,7 +903,7 @@ ckmpm_status run_step_fused(ckmpm_ctx* ctx) {
     issue_fused();
     ctx->grid_valid = true;
   }
-  ctx->tiles_keys = fused_scan ? vc.n_keys : 0;
+  ctx->tiles_keys = tiles_after(vc.n_keys, recorded);
   if (ctx->timing) cudaEventRecord(ctx->step_b, ctx->stream);
   CK_TRY(cudaGetLastError(), "step launch");
   ctx->cur ^= 1;
