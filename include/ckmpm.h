@@ -226,7 +226,8 @@ CKMPM_API ckmpm_status ckmpm_create_server(const ckmpm_config* cfg, ckmpm_ctx** 
  *                         conversion (0) or, in blocks of 256 or more
  *                         particles, by a fused multiply-add (1, default)
  *   CKMPM_SPLITS=1..8     work units per particle block (default: chosen per
- *                         step from the particle count)
+ *                         step from the numbers of particles and of blocks
+ *                         and from the fullest block)
  *   CKMPM_CTAS_PER_SM=k   CTAs per SM of the kernel that clears the grid
  *                         accumulators after ckmpm_probe_grids (default 8) */
 

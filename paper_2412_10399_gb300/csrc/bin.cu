@@ -147,6 +147,10 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_final(StepView v, BinScra
   const uint32_t c[kPerThread] = {x.x, x.y, x.z, x.w};
   const uint32_t tc = x.x + x.y + x.z + x.w;
   const uint32_t tn = (x.x != 0u) + (x.y != 0u) + (x.z != 0u) + (x.w != 0u);
+  if (v.fullest) {  // at most one atomic a warp, and none but in dense blocks
+    const uint32_t m = __reduce_max_sync(0xffffffffu, max(max(x.x, x.y), max(x.z, x.w)));
+    if (m > kDenseBlock && (threadIdx.x & 31u) == 0u) atomicMax(v.fullest, m);
+  }
   // block-wide exclusive scan of (tc, tn)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t ic = tc, in = tn;
@@ -317,6 +321,13 @@ __device__ __forceinline__ void list_grid_blocks(const StepView& v, uint32_t n_v
 // The two passes read the scan's results and do not depend on each other: the
 // first `sctas` CTAs scatter, the others list.
 __global__ void __launch_bounds__(256) k_scatter_glist(StepView v, uint32_t n_vblocks, uint32_t sctas) {
+  // (a thread whose warp has the fewest flags to list)
+  if (v.fullest && blockIdx.x == gridDim.x - 1 && threadIdx.x == blockDim.x - 1) {
+    const uint32_t npb = *v.n_pb, fullest = *v.fullest;
+    *v.fullest = 0u;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) v.parts[k] = limit_units(v.units[k], npb, v.unit_most, fullest).splits;
+  }
   if (blockIdx.x < sctas)
     scatter_particles(v, blockIdx.x, sctas);
   else

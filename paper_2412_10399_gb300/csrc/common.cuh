@@ -83,17 +83,38 @@ struct Pool {
 
 // Work units of a transfer kernel: `splits` parts of every particle block, of
 // `unit` particles each (a block that holds more than splits * unit is cut into
-// equal parts; the last parts of a thin one are empty).
+// equal parts; the last parts of a thin one are empty; unit 0: a fixed count of
+// parts).
 struct Units {
   uint32_t splits, unit;
 };
 enum { kUnitsP2G = 0, kUnitsG2P = 1 };
-// The parts a step of npb blocks uses: no more than give `most` units, so that
-// a body spread over many thin blocks does not pay for parts without
-// particles (a part then takes more than `unit`).
-__device__ __forceinline__ Units limit_units(Units w, uint32_t npb, uint32_t most) {
-  w.splits = min(w.splits, max(1u, (most + npb - 1u) / max(npb, 1u)));
+// The host's count of parts is made for blocks of 8 particles per cell, 512,
+// and holds up to this many particles a block; the scan records the fullest
+// block beyond it.
+constexpr uint32_t kDenseBlock = 640;
+// The parts a step of npb blocks uses (one thread of the listing kernel takes
+// them for both transfers, which then read them beside npb: worked out by each
+// CTA they cost the elastic cube's step of 41 us 0.2 us).  Where the fullest block holds more than
+// kDenseBlock particles, as many as cut that block into units (a part of it is
+// the longest chain of the kernel: at 27 particles per cell the kernel-gradient
+// G2P of 343,331 particles took 66 us in three parts a block, 41 in
+// nine).  No more than give `most` units, so that a body spread over many thin
+// blocks does not pay for parts without particles (a part then takes more than
+// `unit`).
+__host__ __device__ inline Units limit_units(Units w, uint32_t npb, uint32_t most, uint32_t fullest) {
+  if (fullest > kDenseBlock && w.unit != 0u) {
+    const uint32_t cut = (fullest + w.unit - 1u) / w.unit;
+    w.splits = w.splits > cut ? w.splits : cut;
+  }
+  const uint32_t lim = npb ? (most + npb - 1u) / npb : 1u;
+  w.splits = w.splits < lim ? w.splits : lim;
   return w;
+}
+// Particles of each part of a block of cnt, in whole chunks of `align`.
+__host__ __device__ inline uint32_t part_size(const Units& w, uint32_t cnt, uint32_t align) {
+  const uint32_t per = ((cnt + w.splits - 1u) / w.splits + align - 1u) / align * align;
+  return w.unit > per ? w.unit : per;
 }
 
 // Everything the per-step kernels read; passed by value.
@@ -134,6 +155,9 @@ struct StepView {
   Units units[2];       // work units of P2G and of G2P
   uint32_t work0[2];    // what the scan sets work[] to: the CTAs of a step of split blocks, else 0
   uint32_t unit_most;   // limit_units' bound (32 per SM)
+  uint32_t* fullest;    // split blocks only (else null): particles of the step's fullest block if above
+                        // kDenseBlock, else 0 (from the scan; the listing kernel returns it to 0)
+  uint32_t* parts;      // the listing kernel's limit_units: parts of a block for P2G and for G2P
   uint32_t n_mats;      // entries of the material table
   // fused G2P2G step only (else null): the block table of the next step's
   // grid (the gather reads Gvel through `table`, the scatter adds to Gacc
@@ -172,7 +196,7 @@ __device__ __forceinline__ bool unit_of(const StepView& v, const Units& w, uint3
     q.hi = q.cnt;
     return true;  // listed blocks hold particles
   }
-  const uint32_t per = max(w.unit, ((q.cnt + w.splits - 1) / w.splits + ALIGN - 1) / ALIGN * ALIGN);
+  const uint32_t per = part_size(w, q.cnt, ALIGN);
   q.lo = part * per;
   q.hi = min(q.cnt, q.lo + per);
   return q.lo < q.hi;

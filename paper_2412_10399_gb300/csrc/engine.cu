@@ -103,8 +103,8 @@ struct ckmpm_ctx {
   uint32_t* bnd[2]{};  // per key: P2G contribution bounds (2 floats as bits)
   uint32_t *cursor = nullptr, *perm = nullptr, *pb_scene = nullptr;
   uint2* pb = nullptr;
-  uint32_t *counters = nullptr;  // [0] n_pb, [1] n_g, [2] err, [4..5] fp64 (64-bit), [6..7] work,
-                                 // [8] n_g of the second table set, [9] leftover count
+  uint32_t *counters = nullptr;  // [0] n_pb, [1] n_g, [2] err, [3] fullest block, [4..5] fp64 (64-bit), [6..7] work,
+                                 // [8] n_g of the second table set, [9] leftover count, [10..11] parts
   // fused G2P2G steps: a second block-table set for the next step's grid,
   // which one maps the current grid velocities, and whether they are current
   bool fused = false;
@@ -289,6 +289,10 @@ ck::StepView make_view(ckmpm_ctx* ctx) {
     v.work0[k] = v.units[k].splits > 1 ? (uint32_t)(ctx->sm_count * warps[k]) : 0u;
   }
   v.unit_most = ck::p2g_ctas(ctx->sm_count);
+  if (v.units[0].splits > 1 || v.units[1].splits > 1) {
+    v.fullest = ctx->counters + 3;
+    v.parts = ctx->counters + 10;
+  }
   if (ctx->fused) {  // binning zeroes the leftover count every step
     v.lo_list = ctx->lo_list;
     v.lo_count = ctx->counters + 9;

@@ -50,6 +50,10 @@ inline int g2p_warps(int kind, int transfer, int minb) {
 // 21.0 / 26.6; on the diffusion bar (224,000, PIC): 21.1 / 24.6, 20.6 / 29.2,
 // 16.9 / 31.0, 21.1 / 39.7; on a sand box of 592,704 (with the events' 6 us),
 // P2G in parts of 192 39.5, of 256 32.7.
+// The count of parts is for blocks of 512; limit_units raises it on the device
+// where blocks are fuller.  Step of 343,331 particles at 27 per cell / 346,111
+// at 64, us, with the count for 512 and with limit_units': compact kernel 89 / 143
+// and 69 / 67, quadratic 93 / 150 and 69 / 69; kernel-gradient APIC at 27: 114 and 76.
 inline Units step_units(int which, int64_t n, int sm_count, int warps) {
   const int64_t sm = sm_count, block = 512;
   if (n >= sm * 20 * block) return Units{1u, (uint32_t)block};

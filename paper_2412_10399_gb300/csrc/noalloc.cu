@@ -166,7 +166,7 @@ extern "C" CKMPM_API ckmpm_status ckmpm_p2g_grids_static(const ckmpm_scene* sc, 
   v.cnt_nxt = v.cnt_cur;
   v.bnd_cur = cv.take<uint32_t>(2 * nkeys);
   v.bnd_nxt = v.bnd_cur;
-  uint32_t* counters = cv.take<uint32_t>(8);
+  uint32_t* counters = cv.take<uint32_t>(12);
   v.n_pb = counters + 0;
   v.n_g = counters + 1;
   v.err = counters + 2;
@@ -187,6 +187,8 @@ extern "C" CKMPM_API ckmpm_status ckmpm_p2g_grids_static(const ckmpm_scene* sc, 
   const int warps = ck::p2g_warps(kernel, pic ? 1 : 0, rep);
   v.units[ck::kUnitsP2G] = ck::step_units(ck::kUnitsP2G, n, sms, warps);
   v.unit_most = ck::p2g_ctas(sms);
+  v.fullest = counters + 3;
+  v.parts = counters + 10;
   v.work0[0] = v.units[ck::kUnitsP2G].splits > 1 ? (uint32_t)(sms * warps) : 0u;
   bs.scene_tab = d_prm->tab;
   bs.n_scene_tab = 1;

@@ -741,7 +741,7 @@ __global__ void __launch_bounds__(kP2GWarp, p2g_min_ctas(KIND, TR, REP)) k_p2g(S
   const uint32_t lane = threadIdx.x;
   // dynamic scheduling: one work unit (a block or a part of one) at a time
   const uint32_t npb = *v.n_pb;
-  const Units units = SPLIT ? limit_units(v.units[kUnitsP2G], npb, v.unit_most) : Units{1u, 0u};
+  const Units units = SPLIT ? Units{v.parts[kUnitsP2G], v.units[kUnitsP2G].unit} : Units{1u, 0u};
   const uint32_t nunits = npb * units.splits;
   for (uint32_t u = SPLIT ? blockIdx.x : next_unit(&v.work[0]); u < nunits; u = next_unit(&v.work[0])) {
     Unit q;
@@ -1176,7 +1176,7 @@ __global__ void __launch_bounds__(kG2PWarp, 4 * MINB) k_g2p(StepView v) {
   }
   __syncwarp();
   const uint32_t npb = *v.n_pb;
-  const Units units = SPLIT ? limit_units(v.units[kUnitsG2P], npb, v.unit_most) : Units{1u, 0u};
+  const Units units = SPLIT ? Units{v.parts[kUnitsG2P], v.units[kUnitsG2P].unit} : Units{1u, 0u};
   const uint32_t nunits = npb * units.splits;
   for (uint32_t u = SPLIT ? blockIdx.x : next_unit(&v.work[1]); u < nunits; u = next_unit(&v.work[1])) {
     Unit q;
@@ -1319,7 +1319,7 @@ __global__ void __launch_bounds__(kG2PWarp, 4 * MINB) k_g2p2g(StepView v) {
   const uint32_t lane = threadIdx.x;
   const uint32_t npb = *v.n_pb;
   const bool split = v.units[kUnitsG2P].splits > 1u;
-  const Units units = limit_units(v.units[kUnitsG2P], npb, v.unit_most);
+  const Units units = split ? Units{v.parts[kUnitsG2P], v.units[kUnitsG2P].unit} : Units{1u, 0u};
   const uint32_t nunits = npb * units.splits;
   for (uint32_t u = split ? blockIdx.x : next_unit(&v.work[1]); u < nunits; u = next_unit(&v.work[1])) {
     Unit q;
