@@ -2037,17 +2037,6 @@ static void launch_p2g_apic(const LaunchCfg& lc, const StepView& v) {
   }
 }
 
-// Grid of the grid update.  A wide one for a large step: each CTA's block loop
-// is short, so the dependent loads of one block (list entry, scene) overlap
-// across CTAs.  A small step has few blocks (about n / 340 at 8 per cell; n /
-// 64 leaves room), and launching 9728 empty CTAs took 5 us of it.  The loop
-// covers any number of blocks.  Measured: 5.7 -> 3.3 us on the elastic cube,
-// 5.9 -> 3.7 on the granular column, 45 on 16.27 M particles either way.
-static int update_ctas(const LaunchCfg& lc, const StepView& v) {
-  const uint32_t est = (std::min(v.pool_cap, v.n_cur / 64u + 256u) + 1u) / 2u;
-  return (int)std::max((uint32_t)lc.sm_count * 4u, std::min((uint32_t)lc.sm_count * 64u, est));
-}
-
 template <int KIND, int MINB, int TR>
 static void launch_g2p(const LaunchCfg& lc, const StepView& v, uint32_t g) {
   if (v.units[kUnitsG2P].splits > 1u)
@@ -2067,7 +2056,9 @@ static void launch_all(const LaunchCfg& lc, StepView v, int which) {
       else
         launch_p2g_apic<KIND>(lc, v);
       break;
-    case LK_UPDATE: k_grid_update<KIND><<<update_ctas(lc, v), 128, 0, lc.stream>>>(v); break;
+    case LK_UPDATE:
+      k_grid_update<KIND><<<update_ctas(KIND, lc.sm_count, v.pool_cap, v.n_cur), 128, 0, lc.stream>>>(v);
+      break;
     case LK_G2P:
       // register budget of G2P: 20 warps/SM (96 registers) by default, the
       // faster for both kernels on the large-impact scene; 16 (119-124

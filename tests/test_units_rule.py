@@ -1,10 +1,12 @@
-"""The rule that cuts particle blocks into work units, evaluated on the host from the headers that the kernels use.
+"""The rules of the launches, evaluated on the host from the headers that the kernels use.
 
 A kernel ends with its longest unit.  Bodies of more than 8 particles per cell have fewer and fuller blocks, so a count
 of parts made for 512 particles a block leaves long units and idle warps.  For blocks of 641 to 8000 particles (up to
 125 per cell) the longest unit must be no longer than the one that the body is cut into, or than that of a count of
 parts by the particle number alone (two units of 512 for each of 20 warps per SM, at most eight parts, in whole chunks).
-Blocks of up to 640 keep the parts measured for them; no body is cut into more units than the limit."""
+Blocks of up to 640 keep the parts measured for them; no body is cut into more units than the limit.
+
+The grid update loops over its blocks in whole waves of the CTAs that are resident together."""
 import shutil
 import subprocess
 
@@ -16,8 +18,10 @@ SMS = 152
 SRC = r"""
 #include <cstdio>
 #include "launch.h"
-int main() {
+int main(int argc, char**) {
   long long which, n, kind, transfer, npb, cnt;
+  while (argc > 1 && std::scanf("%lld %lld %lld", &kind, &n, &cnt) == 3)
+    std::printf("%d\n", ck::update_ctas((int)kind, 152, (unsigned)cnt, (unsigned)n));
   while (std::scanf("%lld %lld %lld %lld %lld %lld", &which, &n, &kind, &transfer, &npb, &cnt) == 6) {
     const int warps = which == 0 ? ck::p2g_warps(kind, transfer, kind == 1 && transfer == 0 ? 2 : 1)
                                  : ck::g2p_warps(kind, transfer, 5);
@@ -40,9 +44,9 @@ def rule(tmp_path_factory):
     subprocess.run([nvcc, *build.ARCH, "-std=c++17", f"-I{build.CSRC}", f"-I{build.INCLUDE}", str(d / "rule.cu"),
                     "-o", exe], check=True, capture_output=True)
 
-    def ask(rows):
+    def ask(rows, *args):
         text = "\n".join(" ".join(map(str, r)) for r in rows)
-        out = subprocess.run([exe], input=text, check=True, capture_output=True, text=True).stdout
+        out = subprocess.run([exe, *args], input=text, check=True, capture_output=True, text=True).stdout
         return [tuple(map(int, line.split())) for line in out.splitlines()]
     return ask
 
@@ -70,3 +74,12 @@ def test_ordinary_blocks_keep_their_parts(rule):
     rows = list(_rows((64, 512, 640)))
     for r, (host, unit, splits, longest) in zip(rows, rule(rows)):
         assert splits == min(host, -(-SMS * 32 // r[4])) and longest >= unit
+
+
+def test_grid_update_launches_whole_waves(rule):
+    rows = [(kind, n, pool) for kind in (0, 1) for n in (1, 4096, 32768, 150000, 346112, 1000000, 16273664)
+            for pool in (64, 4608, 100000, 2000000)]
+    for (kind, n, pool), (ctas,) in zip(rows, rule(rows, "update")):
+        wave = (8 if kind else 10) * SMS
+        assert ctas % wave == 0 and wave <= ctas <= 64 * SMS
+        assert ctas + wave > 64 * SMS or 2 * ctas >= min(pool, n // 64 + 256)
