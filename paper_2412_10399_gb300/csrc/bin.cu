@@ -13,7 +13,8 @@
 //                 become the active grid-block list, flags cleared
 // (A state that changed outside a step first takes its tile sums with
 // scan_tiles; a key space of more than kScanFusedTiles tiles runs scan_tiles
-// and scan_top, one CTA's exclusive scan over the tile sums, every step.)
+// and scan_top, one CTA's exclusive scan over the sums of tiles of
+// kScanTileWide keys, every step.)
 // (G2P clears each histogram entry it has used, so the buffer it fills next
 // step starts at zero without a pass over the whole key space.)
 // Against a scan of three kernels over 4096-key tiles and two further ones
@@ -32,11 +33,10 @@
 namespace ck {
 
 constexpr int kScanThreads = 256;
-constexpr int kPerThread = kScanTile / kScanThreads;  // 4: one 16-byte load; a thread's keys are a serial chain
-static_assert(kPerThread == 4, "the scan loads its keys as one uint4");
 
+template <int TILE>
 __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(StepView v, BinScratch bs) {
-  write_tile_sums<kScanThreads>(v.cnt_cur, v.n_keys, bs.tile_cnt, bs.tile_ne);
+  write_tile_sums<kScanThreads, TILE>(v.cnt_cur, v.n_keys, bs.tile_cnt, bs.tile_ne);
 }
 
 // Exclusive scan of (tile_cnt, tile_ne) in place by one CTA of 1024 threads.
@@ -109,17 +109,26 @@ __device__ __forceinline__ int scene_of_key(const BinScratch& bs, uint32_t key) 
 }
 
 // MODE: what precedes the CTA's tile comes from the tile sums' exclusive scan
-// (0), from the tiles' own sums (1) or from the histogram itself (2).
+// (0: a wide tile, 16 keys a thread), from the tiles' own sums (1) or from the
+// histogram itself (2) (4 keys a thread: they are a serial chain).
 template <int MODE>
 __global__ void __launch_bounds__(kScanThreads) k_scan_final(StepView v, BinScratch bs) {
-  const uint64_t base = (uint64_t)blockIdx.x * kScanTile + threadIdx.x * kPerThread;
-  uint4 x = make_uint4(0u, 0u, 0u, 0u);
-  if (base + kPerThread <= v.n_keys) {
-    x = *reinterpret_cast<const uint4*>(v.cnt_cur + base);
-  } else if (base < v.n_keys) {
-    x.x = v.cnt_cur[base];
-    if (base + 1 < v.n_keys) x.y = v.cnt_cur[base + 1];
-    if (base + 2 < v.n_keys) x.z = v.cnt_cur[base + 2];
+  constexpr int TILE = MODE == 0 ? kScanTileWide : kScanTile, PER = TILE / kScanThreads;
+  static_assert(PER % 4 == 0 && (MODE == 0 || PER == 4), "keys in 16-byte loads, one of them where MODE 2 counts tiles");
+  const uint64_t base = (uint64_t)blockIdx.x * TILE + threadIdx.x * PER;
+  uint32_t c[PER];
+  if (base + PER <= v.n_keys) {
+#pragma unroll
+    for (int q = 0; q < PER; q += 4) {
+      const uint4 x = *reinterpret_cast<const uint4*>(v.cnt_cur + base + q);
+      c[q] = x.x;
+      c[q + 1] = x.y;
+      c[q + 2] = x.z;
+      c[q + 3] = x.w;
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < PER; ++q) c[q] = base + q < v.n_keys ? v.cnt_cur[base + q] : 0u;
   }
   // particles and blocks of the tiles before this one
   uint32_t tpc = 0, tpn = 0;
@@ -144,12 +153,16 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_final(StepView v, BinScra
     tpc = bs.tile_cnt[blockIdx.x];
     tpn = bs.tile_ne[blockIdx.x];
   }
-  const uint32_t c[kPerThread] = {x.x, x.y, x.z, x.w};
-  const uint32_t tc = x.x + x.y + x.z + x.w;
-  const uint32_t tn = (x.x != 0u) + (x.y != 0u) + (x.z != 0u) + (x.w != 0u);
+  uint32_t tc = 0, tn = 0, most = 0;
+#pragma unroll
+  for (int q = 0; q < PER; ++q) {
+    tc += c[q];
+    tn += c[q] != 0u;
+    most = max(most, c[q]);
+  }
   if (v.fullest) {  // at most one atomic a warp, and none but in dense blocks
-    const uint32_t m = __reduce_max_sync(0xffffffffu, max(max(x.x, x.y), max(x.z, x.w)));
-    if (m > kDenseBlock && (threadIdx.x & 31u) == 0u) atomicMax(v.fullest, m);
+    most = __reduce_max_sync(0xffffffffu, most);
+    if (most > kDenseBlock && (threadIdx.x & 31u) == 0u) atomicMax(v.fullest, most);
   }
   // block-wide exclusive scan of (tc, tn)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -202,7 +215,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_final(StepView v, BinScra
   uint64_t khi = 0u;
   long long tbase = 0;
 #pragma unroll
-  for (int q = 0; q < kPerThread; ++q) {
+  for (int q = 0; q < PER; ++q) {
     if (c[q]) {
       const uint32_t k = (uint32_t)base + q;
       v.cursor[k] = pc;
@@ -377,7 +390,11 @@ void launch_bin(cudaStream_t st, const StepView& v, const BinScratch& bs, int wh
   const uint32_t gctas = std::max(1u, std::min(lim, (n_gblocks + 1023u) / 1024u));
   switch (which) {
     case LB_SCAN_TILES:
-      if (!scan_direct(v.n_keys)) k_scan_tiles<<<ntiles, kScanThreads, 0, st>>>(v, bs);
+      if (scan_direct(v.n_keys)) break;
+      if (fused)
+        k_scan_tiles<kScanTile><<<ntiles, kScanThreads, 0, st>>>(v, bs);
+      else
+        k_scan_tiles<kScanTileWide><<<ntiles, kScanThreads, 0, st>>>(v, bs);
       break;
     case LB_SCAN_TOP:
       if (!fused) k_scan_top<<<1, 1024, 0, st>>>(bs, ntiles);

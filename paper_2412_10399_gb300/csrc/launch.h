@@ -115,17 +115,22 @@ void launch_static_grids(int kind, cudaStream_t st, const StepView& v, uint32_t 
 // bin.cu
 constexpr int kScanTile = 1024;  // keys per scan tile
 // Up to this many tiles every CTA of the scan sums the tiles before its own
-// (at most 16 loads a thread); beyond, one CTA scans the tile sums first.
+// (two arrays: at most 32 loads a thread).  Beyond, one CTA scans the tile sums
+// first, 1024 an iteration, and tiles are wide: with 1024 keys its chain was
+// four times as long and the other kernels had four times the CTAs, us a step's
+// binning for res 1024 / 2048 (16.8 M and 134 M keys, 32,767 particles): 67 / 470
+// against 43 / 250.
 constexpr uint32_t kScanFusedTiles = 4096;
+constexpr int kScanTileWide = 4096;
+__host__ __device__ inline bool scan_fused(uint32_t n_keys) { return n_keys <= kScanFusedTiles * kScanTile; }
 __host__ __device__ inline uint32_t scan_tiles(uint32_t n_keys) {
-  const uint32_t t = (uint32_t)(((uint64_t)n_keys + kScanTile - 1) / kScanTile);
-  return t ? t : 1u;
+  const uint32_t tile = scan_fused(n_keys) ? kScanTile : kScanTileWide;
+  return n_keys ? (n_keys - 1u) / tile + 1u : 1u;
 }
 // Up to this many tiles the scan needs no tile sums: every CTA counts the keys
 // before its own tile itself (at most 7 loads of 16 bytes a thread).
 constexpr uint32_t kScanDirectTiles = 8;
 inline bool scan_direct(uint32_t n_keys) { return scan_tiles(n_keys) <= kScanDirectTiles; }
-inline bool scan_fused(uint32_t n_keys) { return scan_tiles(n_keys) <= kScanFusedTiles; }
 struct BinScratch {
   uint32_t* tile_cnt;   // per tile: sum of counts
   uint32_t* tile_ne;    // per tile: non-empty keys

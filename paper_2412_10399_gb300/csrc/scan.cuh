@@ -9,19 +9,19 @@
 
 namespace ck {
 
-// Particles and non-empty keys of every tile of kScanTile keys; T threads per
-// CTA, a loop over tiles.  cnt is 16-byte aligned.
-template <int T>
+// Particles and non-empty keys of every tile of TILE keys; T threads per CTA, a
+// loop over tiles.  cnt is 16-byte aligned.
+template <int T, int TILE>
 __device__ __forceinline__ void write_tile_sums(const uint32_t* cnt, uint32_t n_keys, uint32_t* tile_cnt,
                                                 uint32_t* tile_ne) {
-  static_assert(kScanTile % (4 * T) == 0, "a thread takes whole 16-byte groups");
+  static_assert(TILE % (4 * T) == 0, "a thread takes whole 16-byte groups");
   __shared__ uint32_t sc[T / 32], sn[T / 32];
   const uint32_t ntiles = scan_tiles(n_keys);
   for (uint32_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     uint32_t c = 0, ne = 0;
 #pragma unroll
-    for (int q = 0; q < kScanTile / (4 * T); ++q) {
-      const uint64_t k = (uint64_t)tile * kScanTile + 4u * (q * T + threadIdx.x);
+    for (int q = 0; q < TILE / (4 * T); ++q) {
+      const uint64_t k = (uint64_t)tile * TILE + 4u * (q * T + threadIdx.x);
       if (k + 4 <= n_keys) {
         const uint4 x = *reinterpret_cast<const uint4*>(cnt + k);
         c += x.x + x.y + x.z + x.w;

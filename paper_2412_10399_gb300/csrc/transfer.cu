@@ -1556,7 +1556,7 @@ __global__ void __launch_bounds__(128) k_g2p_fp64(StepView v) {
     v.bnd_cur[2 * key + 1] = 0u;
   }
   // the histogram G2P filled is complete: its tile sums for the next scan
-  if (v.tile_cnt) write_tile_sums<128>(v.cnt_nxt, v.n_keys, v.tile_cnt, v.tile_ne);
+  if (v.tile_cnt) write_tile_sums<128, kScanTile>(v.cnt_nxt, v.n_keys, v.tile_cnt, v.tile_ne);
   const uint32_t n = (uint32_t)min(*v.fp64_count, (unsigned long long)v.n_cur);
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const uint32_t t = v.fp64_list[i];

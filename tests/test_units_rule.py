@@ -6,7 +6,8 @@ of parts made for 512 particles a block leaves long units and idle warps.  For b
 parts by the particle number alone (two units of 512 for each of 20 warps per SM, at most eight parts, in whole chunks).
 Blocks of up to 640 keep the parts measured for them; no body is cut into more units than the limit.
 
-The grid update loops over its blocks in whole waves of the CTAs that are resident together."""
+The grid update loops over its blocks in whole waves of the CTAs that are resident together.  One CTA scans the tile
+sums of a large key space, 1024 an iteration: in iterations of no less than 4 million keys."""
 import shutil
 import subprocess
 
@@ -20,7 +21,9 @@ SRC = r"""
 #include "launch.h"
 int main(int argc, char**) {
   long long which, n, kind, transfer, npb, cnt;
-  while (argc > 1 && std::scanf("%lld %lld %lld", &kind, &n, &cnt) == 3)
+  while (argc == 3 && std::scanf("%lld", &n) == 1)
+    std::printf("%d %u\n", (int)ck::scan_fused((unsigned)n), ck::scan_tiles((unsigned)n));
+  while (argc == 2 && std::scanf("%lld %lld %lld", &kind, &n, &cnt) == 3)
     std::printf("%d\n", ck::update_ctas((int)kind, 152, (unsigned)cnt, (unsigned)n));
   while (std::scanf("%lld %lld %lld %lld %lld %lld", &which, &n, &kind, &transfer, &npb, &cnt) == 6) {
     const int warps = which == 0 ? ck::p2g_warps(kind, transfer, kind == 1 && transfer == 0 ? 2 : 1)
@@ -83,3 +86,9 @@ def test_grid_update_launches_whole_waves(rule):
         wave = (8 if kind else 10) * SMS
         assert ctas % wave == 0 and wave <= ctas <= 64 * SMS
         assert ctas + wave > 64 * SMS or 2 * ctas >= min(pool, n // 64 + 256)
+
+
+def test_one_cta_scans_wide_tiles(rule):
+    rows = [(n,) for n in (1, 1024, 8192, 8193, 1 << 22, (1 << 22) + 1, 175 ** 3, 256 ** 3, 512 ** 3, 2 ** 31 - 1)]
+    for (n,), (fused, tiles) in zip(rows, rule(rows, "scan", "tiles")):
+        assert tiles == -(-n // (1024 if fused else 4096)) and fused == (n <= 1 << 22)
