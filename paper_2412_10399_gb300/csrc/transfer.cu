@@ -65,7 +65,7 @@ __device__ __forceinline__ float fold_2pi(float t) {
 
 // sin(2 pi f) per axis, f in [0, 1): the Taylor series of sin x at x = 2 pi t,
 // |x| <= pi/2, through x^11: coefficients (-1)^k (2 pi)^(2k+1) / (2k+1)!,
-// truncation error below (pi/2)^13 / 13! = 1.5e-8, about 1.6e-7 after float
+// truncation error below (pi/2)^13 / 13! = 5.7e-8, about 1.6e-7 after float
 // rounding.
 __device__ __forceinline__ V3 sin_2pi(const V3& f) {
   V3 t = f - V3{pk(rintf(f.p.x), rintf(f.p.y)), rintf(f.z)};
