@@ -15,8 +15,9 @@
 // scan_tiles; a key space of more than kScanFusedTiles tiles runs scan_tiles
 // and scan_top, one CTA's exclusive scan over the sums of tiles of
 // kScanTileWide keys, every step.)
-// (G2P clears each histogram entry it has used, so the buffer it fills next
-// step starts at zero without a pass over the whole key space.)
+// (The float64 pass clears the histogram entries of the step's blocks, so the
+// buffer that G2P fills next step starts at zero without a pass over the whole
+// key space.)
 // Against a scan of three kernels over 4096-key tiles and two further ones
 // (five launches), with the float64 pass that takes the tile sums: 14.2 -> 8.2
 // us a step on the elastic cube (32,768 particles, 64^3), 17.2 -> 9.7 on the

@@ -46,8 +46,6 @@ struct SceneDev {
   uint32_t key_base;  // first particle-block key of this scene
   long long table_base;  // first entry of this scene's block table
   float j_tol, cond_tol, gap_tol;  // float64 SVD criteria
-  float mmax;         // largest particle mass of the scene's materials
-  int alive;
 };
 
 // Two 16-byte groups of what the update reads together, then the indices.
@@ -123,9 +121,10 @@ struct StepView {
   uint32_t* key_cur;    // keys of cur (input of the sort)
   uint32_t* key_nxt;    // keys written by G2P for nxt
   uint32_t* cnt_cur;    // histogram of key_cur over the key space
-  uint32_t* cnt_nxt;    // histogram written by G2P (all zero before it: G2P clears cnt_cur after use)
+  uint32_t* cnt_nxt;    // histogram written by G2P (all zero before it: the float64 pass, behind the step's
+                        // transfers, clears cnt_cur's entries of the step's blocks)
   uint32_t* bnd_cur;    // per key: P2G contribution bounds (mass, momentum) of cur, float
-                        // bits; P2G clears an active block's pair after use
+                        // bits; cleared with cnt_cur
   uint32_t* bnd_nxt;    // the same for nxt, written by G2P (all zero before it)
   uint32_t* cursor;     // scatter cursors
   uint32_t* perm;       // sorted slot -> index into cur
@@ -151,7 +150,7 @@ struct StepView {
   uint32_t* work;       // [0] next P2G block, [1] next G2P block (dynamic scheduling)
   uint32_t n_keys;      // size of the key space
   uint32_t n_cur;       // particles in cur (including dead ones)
-  uint32_t keep_gacc;   // probe: the grid update leaves Gacc, P2G keeps bnd_cur
+  uint32_t keep_gacc;   // probe: the grid update leaves Gacc
   Units units[2];       // work units of P2G and of G2P
   uint32_t work0[2];    // what the scan sets work[] to: the CTAs of a step of split blocks, else 0
   uint32_t unit_most;   // limit_units' bound (32 per SM)
@@ -270,18 +269,6 @@ __device__ __forceinline__ uint32_t particle_key(const SceneT& s, float ux, floa
   return s.key_base + (uint32_t)((bz * s.npb + by) * s.npb + bx);
 }
 
-__device__ __forceinline__ uint32_t warp_aggregated_inc(uint32_t* counters, uint32_t key) {
-  // lanes with equal keys add once
-  unsigned mask = __activemask();
-  unsigned peers = __match_any_sync(mask, key);
-  int leader = __ffs(peers) - 1;
-  int lane = threadIdx.x & 31;
-  uint32_t base = 0;
-  if (lane == leader) base = atomicAdd(&counters[key], (uint32_t)__popc(peers));
-  base = __shfl_sync(peers, base, leader);
-  return base + __popc(peers & ((1u << lane) - 1u));
-}
-
 // Histogram increment and P2G contribution bounds of particles binned under
 // `key` (lanes with equal keys add once).  The bounds are non-negative floats
 // kept as bit patterns (whose unsigned order is the float order); each warp
@@ -298,10 +285,6 @@ __device__ __forceinline__ void warp_aggregated_bin(uint32_t* cnt, uint32_t* bnd
     atomicMax(&bnd[2 * key], bm);
     atomicMax(&bnd[2 * key + 1], bp);
   }
-}
-
-__device__ __forceinline__ bool finite4(float4 a) {
-  return isfinite(a.x) && isfinite(a.y) && isfinite(a.z) && isfinite(a.w);
 }
 
 }  // namespace ck

@@ -642,9 +642,9 @@ void destroy_graphs(ckmpm_ctx* ctx) {
 
 // Run a step's launch sequence as the CUDA graph of state parity `key`,
 // capturing it on first use; false when the step must be issued directly
-// instead (capture is not possible on this stream -- the legacy stream, or
-// one the caller is capturing itself -- or it failed; graphs are then off
-// for the context and nothing of the sequence has run).
+// instead (capture is not possible on this stream, the legacy stream, or it
+// failed; graphs are then off for the context and nothing of the sequence has
+// run).  Not called while the caller is capturing the stream.
 template <typename Issue>
 bool graph_step(ckmpm_ctx* ctx, int key, Issue&& issue) {
   if (!ctx->graphs) return false;
@@ -1025,11 +1025,7 @@ ckmpm_status admit_impl(ckmpm_ctx* ctx, const ckmpm_scene* sc, int* scene_id) {
   d.j_tol = (float)sc->fp64_j_tol;
   d.cond_tol = (float)sc->fp64_cond_tol;
   d.gap_tol = (float)sc->fp64_gap_tol;
-  d.alive = 1;
   const double V0 = sc->dx * sc->dx * sc->dx / sc->ppc;
-  double mmax = 0.0;
-  for (int i = 0; i < sc->n_materials; ++i) mmax = std::max(mmax, sc->materials[i].rho * V0);
-  d.mmax = (float)mmax;
   for (int i = 0; i < sc->n_materials; ++i) {
     const ckmpm_material& m = sc->materials[i];
     MatDev& md = ctx->h_mats[mb + i];
@@ -1184,7 +1180,6 @@ ckmpm_status ckmpm_release(ckmpm_ctx* ctx, int scene_id) {
   ctx->grid_valid = false;
   ctx->tiles_keys = 0;
   drop_graphs(ctx);
-  ctx->h_scenes[scene_id].alive = 0;
   ctx->pending_free.push_back(scene_id);
   process_pending(ctx);
   CK_TRY(cudaGetLastError(), "release");

@@ -11,7 +11,7 @@ namespace ck {
 
 struct LaunchCfg {
   cudaStream_t stream;
-  int persistent_ctas;  // CTAs of the persistent P2G / update / G2P launches
+  int persistent_ctas;  // CTAs of the kernel that clears a probe's accumulators
   int sm_count = 1;     // SMs of the device (grid of the float64 pass)
   int g2p_minb = 4;     // resident G2P warps per SM / 4 the register budget targets
   int transfer = 0;     // 0 APIC + MLS, 1 PIC, 2 APIC with the kernel gradient
@@ -134,7 +134,7 @@ inline bool scan_direct(uint32_t n_keys) { return scan_tiles(n_keys) <= kScanDir
 struct BinScratch {
   uint32_t* tile_cnt;   // per tile: sum of counts
   uint32_t* tile_ne;    // per tile: non-empty keys
-  const uint32_t* scene_tab;  // sorted (key_base, slot) pairs of alive scenes
+  const uint32_t* scene_tab;  // sorted (key_base, slot) pairs of the scenes at the last admission
   int n_scene_tab;
 };
 void launch_bin(cudaStream_t st, const StepView& v, const BinScratch& bs, int which, uint32_t n_gblocks,

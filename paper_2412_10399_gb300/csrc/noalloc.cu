@@ -48,6 +48,9 @@ constexpr int kStaticMaxRes = 64;         // cells per axis
 using ck::kStaticMaxMats;                 // materials per scene
 constexpr size_t kStaticBytes = 18u << 20;  // 18 MiB, enough for the limits above
 constexpr int kMaxDevices = 64;
+static_assert((kStaticMaxRes / 4) * (kStaticMaxRes / 4) * (kStaticMaxRes / 4) <=
+                  (int)ck::kScanDirectTiles * ck::kScanTile,
+              "the scan counts the keys itself: no tile sums are taken");
 
 }  // namespace
 
@@ -134,7 +137,6 @@ extern "C" CKMPM_API ckmpm_status ckmpm_p2g_grids_static(const ckmpm_scene* sc, 
   const int64_t n = sc->n;
   const int64_t npb = (sc->res + 3) / 4, nb = npb + 1;
   const int64_t nkeys = npb * npb * npb, nvb = nb * nb * nb;
-  const int64_t ntiles = ck::scan_tiles((uint32_t)nkeys);
 
   Carve cv{(char*)base};
   ck::Pool P{};
@@ -157,8 +159,6 @@ extern "C" CKMPM_API ckmpm_status ckmpm_p2g_grids_static(const ckmpm_scene* sc, 
   v.pool_cap = (uint32_t)nvb;
   ck::StaticParams* d_prm = cv.take<ck::StaticParams>(1);
   ck::BinScratch bs{};
-  bs.tile_cnt = cv.take<uint32_t>(ntiles + 1);
-  bs.tile_ne = cv.take<uint32_t>(ntiles + 1);
   // what a previous call may have left behind and the kernels expect zero, in
   // one piece
   char* const zero = cv.base + cv.used;
@@ -213,9 +213,7 @@ extern "C" CKMPM_API ckmpm_status ckmpm_p2g_grids_static(const ckmpm_scene* sc, 
   h.j_tol = (float)sc->fp64_j_tol;
   h.cond_tol = (float)sc->fp64_cond_tol;
   h.gap_tol = (float)sc->fp64_gap_tol;
-  h.alive = 1;
   ck::MatDev* const hm = prm.mats;
-  double mmax = 0.0;
   for (int i = 0; i < sc->n_materials; ++i) {
     const ckmpm_material& m = sc->materials[i];
     hm[i].model = m.model;
@@ -229,9 +227,7 @@ extern "C" CKMPM_API ckmpm_status ckmpm_p2g_grids_static(const ckmpm_scene* sc, 
     hm[i].gamma = (float)m.gamma;
     hm[i].E = (float)m.E;
     hm[i].nu = (float)m.nu;
-    mmax = std::max(mmax, m.rho * V0);
   }
-  h.mmax = (float)mmax;
 
 #define CK_S(expr)                                   \
   do {                                               \
@@ -243,8 +239,6 @@ extern "C" CKMPM_API ckmpm_status ckmpm_p2g_grids_static(const ckmpm_scene* sc, 
   ck::launch_static_admit(kernel, st, v, prm, d_prm, pic, (uint32_t)sc->n_materials, sc->x, sc->v, sc->mat, F, B);
   // binning and P2G, as in a context's step
   const int grid_ctas = sms * 4;
-  ck::launch_bin(st, v, bs, ck::LB_SCAN_TILES, (uint32_t)nvb, grid_ctas);
-  ck::launch_bin(st, v, bs, ck::LB_SCAN_TOP, (uint32_t)nvb, grid_ctas);
   ck::launch_bin(st, v, bs, ck::LB_SCAN_FINAL, (uint32_t)nvb, grid_ctas);
   ck::launch_bin(st, v, bs, ck::LB_SCATTER_GLIST, (uint32_t)nvb, grid_ctas);
   ck::LaunchCfg lc{st, sms * 8};

@@ -137,19 +137,17 @@ template <>
 struct Geo<0> {
   static constexpr int NG = 2;
   static constexpr int N = 2;  // nodes per axis of a stencil
-  static constexpr int E0 = 5, E1 = 6;
+  static constexpr int E0 = 5;
   static constexpr int N0 = 125;
   static constexpr int NS = 341;
-  static constexpr float half = 0.5f;
 };
 template <>
 struct Geo<1> {
   static constexpr int NG = 1;
   static constexpr int N = 3;
-  static constexpr int E0 = 6, E1 = 6;
+  static constexpr int E0 = 6;
   static constexpr int N0 = 216;
   static constexpr int NS = 216;
-  static constexpr float half = 1.0f;
 };
 
 // staged index -> (slot, local node coordinates)
@@ -1524,9 +1522,6 @@ __device__ __forceinline__ void store_M(const Pool& P, uint32_t t, const float* 
   P.VM1[t] = a;
   P.VM2[t] = b;
 }
-__device__ __forceinline__ void load_T(const Pool& P, uint32_t t, float* T) {
-  to_rows(unpack_m3(P.T0[t], P.T1[t], P.T2[t]), T);
-}
 __device__ __forceinline__ void store_T(const Pool& P, uint32_t t, const float* T) {
   float4 a, b;
   float c;
@@ -1979,10 +1974,6 @@ __global__ void k_rekey(Pool P, uint32_t* key, uint32_t* cnt, uint32_t* bnd, con
     float4 X = P.X[t];
     const MatDev mt = mats[__float_as_uint(X.w)];
     const SceneDev s = scenes[mt.scene];
-    if (!s.alive) {
-      key[t] = CK_DEAD_KEY;
-      continue;
-    }
     float ux = X.x * s.inv_dx, uy = X.y * s.inv_dx, uz = X.z * s.inv_dx;
     if (!(in_domain(ux, s.res) && in_domain(uy, s.res) && in_domain(uz, s.res))) {
       flag_error(err, CK_ERR_DOMAIN);
