@@ -71,15 +71,17 @@ inline Units step_units(int which, int64_t n, int sm_count, int warps) {
 // 2.5 us of it.  Whole waves of what an SM holds (registers: ten of the compact
 // kernel's, eight of the quadratic's), up to 64 per SM, since a body spread over
 // more blocks than the estimate keeps them all looping and a part of a wave
-// takes as long as a whole one.  Measured, us with 4, 8, 12, 16 and 64 per SM:
-// 30,000 particles in as many blocks (compact kernel) 233, 158, 186, 159, 149;
-// 150,000 in 111,000 (quadratic) 344, 199, 248, 199, 162; the elastic cube and
-// the granular column 7.9 and 8.1 (with the events' 6) up to 16, 10.4 with 64.
+// takes as long as a whole one; rounded down, because empty CTAs cost a compact
+// body 0.3 ns each (592,704 particles: 0.7% of a step in rounding up).
+// Measured, us with 4, 8, 10, 12, 16 and 64 per SM: 30,000 particles in as many
+// blocks (compact kernel) 233, 158, 148, 186, 159, 149; 150,000 in 111,000
+// (quadratic, without 10) 344, 199, 248, 199, 162; the elastic cube and the
+// granular column 7.9 and 8.1 (with the events' 6) up to 16, 10.4 with 64.
 constexpr int update_wave(int kind) { return kind == 0 ? 10 : 8; }
 inline int update_ctas(int kind, int sm_count, uint32_t pool_cap, uint32_t n_cur) {
   const uint32_t wave = (uint32_t)(sm_count * update_wave(kind)), most = 64u / (uint32_t)update_wave(kind);
   const uint32_t est = (std::min(pool_cap, n_cur / 64u + 256u) + 1u) / 2u;  // two blocks a CTA and turn
-  return (int)(wave * std::max(1u, std::min(most, (est + wave - 1u) / wave)));
+  return (int)(wave * std::max(1u, std::min(most, est / wave)));
 }
 
 enum { LK_P2G = 0, LK_UPDATE = 1, LK_G2P = 2, LK_CLEAR = 3, LK_G2P_FP64 = 4, LK_G2P2G = 5, LK_LEFTOVER = 6 };

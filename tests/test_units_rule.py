@@ -85,7 +85,8 @@ def test_grid_update_launches_whole_waves(rule):
     for (kind, n, pool), (ctas,) in zip(rows, rule(rows, "update")):
         wave = (8 if kind else 10) * SMS
         assert ctas % wave == 0 and wave <= ctas <= 64 * SMS
-        assert ctas + wave > 64 * SMS or 2 * ctas >= min(pool, n // 64 + 256)
+        est = (min(pool, n // 64 + 256) + 1) // 2
+        assert ctas + wave > min(est, 64 * SMS) and (ctas == wave or ctas <= est)
 
 
 def test_one_cta_scans_wide_tiles(rule):
