@@ -478,11 +478,11 @@ __device__ __forceinline__ void decode_block(const SceneDev& s, uint32_t key, in
 
 // Shared-memory accumulation is in 32-bit fixed point: integer shared
 // atomics run about 4x faster than float ones on this part (measured), and
-// integer sums do not depend on the order of the atomics.  A first pass over
-// the block's particles bounds every contribution each can make (p2g_bound,
-// from the largest weight, weight times offset and row sum of D^-1 of the
-// stencil), so with cnt particles no node sum can exceed cnt times the
-// block's largest bound, and the scale maps that to 2^30 (no overflow).
+// integer sums do not depend on the order of the atomics.  Every contribution
+// that a block's particles can make is bounded when they are binned
+// (p2g_bounds, from the largest weight, weight times offset and row sum of
+// D^-1 of the stencil), so with cnt particles no node sum can exceed cnt times
+// the block's largest bound, and the scale maps that to 2^30 (no overflow).
 // Rounding costs at most half a unit per contribution, cnt * bound * 2^-31.
 
 // P2G runs one warp per CTA and streams a block's particles through shared
@@ -526,7 +526,7 @@ struct P2GBound<1> {
 // |w (A^ d)_r| <= sum_k |A^_rk| |w d_k| and the rows of A^ = M D^-1 / dx sum
 // to at most sum_j |M_rj| * dinv / dx.
 // The PIC transfer's contribution w m v + M grad w (M = -dt V0 tau) has the
-// same bound with wd * dinv replaced by the largest |g_a| of for_nodes_grad:
+// same bound with wd * dinv replaced by the largest |g_a| of a stencil:
 // CK 2 (|K1'| <= 2, at |x| = 1/2, times weights <= 1), quadratic 0.5625
 // (|N'| <= 1 times 0.75^2); both are below wd * dinv (4.04 and 0.5644), so
 // one bound serves every transfer.  APIC with the kernel gradient keeps m B
