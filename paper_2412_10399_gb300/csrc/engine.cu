@@ -705,16 +705,16 @@ bool takes_own_tiles(ckmpm_ctx* ctx, uint32_t n_keys, bool recorded) {
 // the key-space size whose tile sums a step or probe leaves behind
 uint32_t tiles_after(uint32_t n_keys, bool recorded) { return ck::scan_fused(n_keys) && !recorded ? n_keys : 0u; }
 
-ckmpm_status run_step_fused(ckmpm_ctx* ctx);
+ckmpm_status run_step_fused(ckmpm_ctx* ctx, bool recorded);
 
-ckmpm_status run_step(ckmpm_ctx* ctx, bool probe) {
-  if (ctx->fused && !probe) return run_step_fused(ctx);
+// recorded: the caller is capturing the stream (asked once a call, not a step)
+ckmpm_status run_step(ckmpm_ctx* ctx, bool probe, bool recorded) {
+  if (ctx->fused && !probe) return run_step_fused(ctx, recorded);
   if (ctx->fused) ctx->grid_valid = false;  // a probe reuses the grid arrays
   ck::StepView v = make_view(ctx);
   ckmpm_ctx::EvPair ep{};
   const bool fused_scan = ck::scan_fused(v.n_keys);
   if (ctx->keys_dirty) ctx->tiles_keys = 0;
-  const bool recorded = capturing(ctx);
   const bool own_tiles = takes_own_tiles(ctx, v.n_keys, recorded);
   const bool steady =
       !probe && !recorded && !ctx->timing && !ctx->grids_dirty && !ctx->keys_dirty && !(fused_scan && own_tiles);
@@ -806,7 +806,7 @@ ckmpm_status run_step(ckmpm_ctx* ctx, bool probe) {
 // and scatters the particles that stayed in their block into that grid; the
 // float64 pass; the leftover P2G (claiming any further grid blocks); the grid
 // update of the new grid; and the sets swap.
-ckmpm_status run_step_fused(ckmpm_ctx* ctx) {
+ckmpm_status run_step_fused(ckmpm_ctx* ctx, bool recorded) {
   const bool was_clean = !ctx->grids_dirty && !ctx->keys_dirty && ctx->grid_valid && !ctx->timing;
   if (ctx->grids_dirty) {
     ck::launch_transfer(ctx->kind, ctx->lc, make_view(ctx), ck::LK_CLEAR);
@@ -846,7 +846,6 @@ ckmpm_status run_step_fused(ckmpm_ctx* ctx) {
   ck::StepView vn = make_view(ctx);
   ctx->tsel = cs;
   const bool fused_scan = ck::scan_fused(vc.n_keys);
-  const bool recorded = capturing(ctx);
   const bool own_tiles = takes_own_tiles(ctx, vc.n_keys, recorded);
   ckmpm_ctx::EvPair ep{};
   if (ctx->timing) cudaEventRecord(ctx->step_a, ctx->stream);
@@ -1190,8 +1189,9 @@ ckmpm_status ckmpm_step(ckmpm_ctx* ctx, int n) {
   if (!ctx) return CKMPM_EINVAL;
   if (n < 0) return fail(ctx, CKMPM_EINVAL, "n must be >= 0");
   if (ctx->sticky != CKMPM_OK) return ctx->sticky;
+  const bool recorded = capturing(ctx);
   for (int i = 0; i < n; ++i) {
-    ckmpm_status st = run_step(ctx, false);
+    ckmpm_status st = run_step(ctx, false, recorded);
     if (st != CKMPM_OK) return st;
   }
   return CKMPM_OK;
@@ -1200,7 +1200,7 @@ ckmpm_status ckmpm_step(ckmpm_ctx* ctx, int n) {
 ckmpm_status ckmpm_probe_grids(ckmpm_ctx* ctx) {
   if (!ctx) return CKMPM_EINVAL;
   if (ctx->sticky != CKMPM_OK) return ctx->sticky;
-  return run_step(ctx, true);
+  return run_step(ctx, true, capturing(ctx));
 }
 
 ckmpm_status ckmpm_sync(ckmpm_ctx* ctx) {
