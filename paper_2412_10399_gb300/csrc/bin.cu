@@ -333,19 +333,20 @@ __device__ __forceinline__ void list_grid_blocks(const StepView& v, uint32_t n_v
 }
 
 // The two passes read the scan's results and do not depend on each other: the
-// first `sctas` CTAs scatter, the others list.
-__global__ void __launch_bounds__(256) k_scatter_glist(StepView v, uint32_t n_vblocks, uint32_t sctas) {
-  // (a thread whose warp has the fewest flags to list)
-  if (v.fullest && blockIdx.x == gridDim.x - 1 && threadIdx.x == blockDim.x - 1) {
+// first `sctas` CTAs scatter, the next `gctas` list.  In a step of split blocks
+// one more sets the parts of a block for the transfers (in a warp that also
+// lists it set the kernel's length on the diffusion bar: 0.2% of its step).
+__global__ void __launch_bounds__(256) k_scatter_glist(StepView v, uint32_t n_vblocks, uint32_t sctas, uint32_t gctas) {
+  if (blockIdx.x < sctas) {
+    scatter_particles(v, blockIdx.x, sctas);
+  } else if (blockIdx.x < sctas + gctas) {
+    list_grid_blocks(v, n_vblocks, blockIdx.x - sctas, gctas);
+  } else if (threadIdx.x == 0) {
     const uint32_t npb = *v.n_pb, fullest = *v.fullest;
     *v.fullest = 0u;
 #pragma unroll
     for (int k = 0; k < 2; ++k) v.parts[k] = limit_units(v.units[k], npb, v.unit_most, fullest).splits;
   }
-  if (blockIdx.x < sctas)
-    scatter_particles(v, blockIdx.x, sctas);
-  else
-    list_grid_blocks(v, n_vblocks, blockIdx.x - sctas, gridDim.x - sctas);
 }
 
 // Fused step: before a block table is filled again, the entries its last
@@ -389,6 +390,7 @@ void launch_bin(cudaStream_t st, const StepView& v, const BinScratch& bs, int wh
   const uint32_t lim = (uint32_t)grid_ctas;
   const uint32_t sctas = std::max(1u, std::min(lim, (v.n_cur + 256u * kScatterUnroll - 1u) / (256u * kScatterUnroll)));
   const uint32_t gctas = std::max(1u, std::min(lim, (n_gblocks + 1023u) / 1024u));
+  const uint32_t pctas = v.fullest ? 1u : 0u;
   switch (which) {
     case LB_SCAN_TILES:
       if (scan_direct(v.n_keys)) break;
@@ -408,8 +410,8 @@ void launch_bin(cudaStream_t st, const StepView& v, const BinScratch& bs, int wh
       else
         k_scan_final<0><<<ntiles, kScanThreads, 0, st>>>(v, bs);
       break;
-    case LB_SCATTER_GLIST: k_scatter_glist<<<sctas + gctas, 256, 0, st>>>(v, n_gblocks, sctas); break;
-    case LB_GLIST: k_scatter_glist<<<gctas, 256, 0, st>>>(v, n_gblocks, 0u); break;
+    case LB_SCATTER_GLIST: k_scatter_glist<<<sctas + gctas + pctas, 256, 0, st>>>(v, n_gblocks, sctas, gctas); break;
+    case LB_GLIST: k_scatter_glist<<<gctas + pctas, 256, 0, st>>>(v, n_gblocks, 0u, gctas); break;
   }
 }
 

@@ -91,9 +91,9 @@ enum { kUnitsP2G = 0, kUnitsG2P = 1 };
 // and holds up to this many particles a block; the scan records the fullest
 // block beyond it.
 constexpr uint32_t kDenseBlock = 640;
-// The parts a step of npb blocks uses (one thread of the listing kernel takes
-// them for both transfers, which then read them beside npb: worked out by each
-// CTA they cost the elastic cube's step of 41 us 0.2 us).  Where the fullest block holds more than
+// The parts a step of npb blocks uses (a CTA of the listing kernel's launch
+// takes them for both transfers, which then read them beside npb: worked out by
+// each CTA they cost the elastic cube's step of 41 us 0.2 us).  Where the fullest block holds more than
 // kDenseBlock particles, as many as cut that block into units (a part of it is
 // the longest chain of the kernel: at 27 particles per cell the kernel-gradient
 // G2P of 343,331 particles took 66 us in three parts a block, 41 in
@@ -155,8 +155,8 @@ struct StepView {
   uint32_t work0[2];    // what the scan sets work[] to: the CTAs of a step of split blocks, else 0
   uint32_t unit_most;   // limit_units' bound (32 per SM)
   uint32_t* fullest;    // split blocks only (else null): particles of the step's fullest block if above
-                        // kDenseBlock, else 0 (from the scan; the listing kernel returns it to 0)
-  uint32_t* parts;      // the listing kernel's limit_units: parts of a block for P2G and for G2P
+                        // kDenseBlock, else 0 (from the scan; the CTA that sets parts returns it to 0)
+  uint32_t* parts;      // limit_units of the step: parts of a block for P2G and for G2P
   uint32_t n_mats;      // entries of the material table
   // fused G2P2G step only (else null): the block table of the next step's
   // grid (the gather reads Gvel through `table`, the scatter adds to Gacc
